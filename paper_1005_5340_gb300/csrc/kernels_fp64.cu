@@ -10,36 +10,62 @@
 // Complex vectors are kept as two real planes; X, V and K are real, so only
 // the D(omega) scaling mixes the planes.
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 
 namespace tddft {
 
 // ---------------------------------------------------------------------------
-// C[M x N] = A[M x K] . B[K x N], all row-major float64 (DFMA).
-// BM x BN tile per CTA (64 x 64, or 32 x 128 when M is small so that few rows
-// of the tile are wasted), 16-deep K slices staged in shared memory through
-// registers (double buffered), (BM/16) x (BN/16) outputs per thread on a
-// 16 x 16 thread grid.  Every edge is bounds-checked (ragged M, N, K).
+// The float64 kernels are bound by the FP64 pipe (about 2 FMA per clock and
+// SM, so one warp-wide DFMA every 15 clocks per SM): loads, address
+// arithmetic and L2 traffic are nearly free next to it.  What counts is that
+// no DFMA is spent on padding and that every SM gets the same share, so the
+// tiles are small, one output per lane where that fills the lanes, and all
+// of them keep one summation order per output whatever the tile or the
+// number of right-hand sides (host-driven, graph and batch launches of the
+// same right-hand side give the same bits).  chi0 z of 3 vectors on 4 atoms:
+// 406 -> 52 us; A z of 48 vectors on 24 atoms: 7.31 -> 3.95 ms (1.03 TFLOP/s
+// of the measured 1.10); of 96 vectors on 64 atoms 89.5 -> 87.6 ms.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr int GB_K = 16;
 
-template <int BM, int BN>
-__global__ void __launch_bounds__(256, (BM == 32 ? 2 : 3)) gemm_f64_nn(int M, int N, int K, const double *__restrict__ A,
-                                                   int64_t lda, const double *__restrict__ B,
-                                                   int64_t ldb, double *__restrict__ C,
-                                                   int64_t ldc, const int *__restrict__ dcnt,
-                                                   int mul_m, int mul_n, int kchunk,
-                                                   int64_t zstride) {
-  constexpr int TM = BM / 16, TN = BN / 16;     // outputs per thread
-  constexpr int LA = BM * GB_K / 256, LB = BN * GB_K / 256;   // loads per thread
-  __shared__ double As[2][GB_K][BM + 2];
-  __shared__ double Bs[2][GB_K][BN];
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const int64_t m0 = (int64_t)blockIdx.y * BM;
-  const int64_t n0 = (int64_t)blockIdx.x * BN;
+int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0
+               ? v : 1;
+  }();
+  return n;
+}
+
+// ---------------------------------------------------------------------------
+// C[M x N] = A[M x K] . B[K x N], all row-major float64 (DFMA).
+// A BM x BN tile per CTA; the four warps take one K quarter each
+// (ceil(K/4) entries, staged per warp through registers into a double
+// buffer in shared memory, no block barrier in the loop), and the quarters
+// are added in order at the end: p0 + p1 + p2 + p3.  The K quarters depend on
+// K alone, so every tile shape sums an output in the same order.
+// A lane holds TM x TN outputs.  Every edge is bounds-checked.
+// ---------------------------------------------------------------------------
+constexpr int GF_WARPS = 4;
+
+template <int BM, int BN, int TM, int TN, int KD>
+__global__ void __launch_bounds__(32 * GF_WARPS)
+    gemm_f64_kernel(int M, int N, int K, const double *__restrict__ A, int64_t lda,
+                    const double *__restrict__ B, int64_t ldb, double *__restrict__ C, int64_t ldc,
+                    const int *__restrict__ dcnt, int mul_m, int mul_n, int m_tiles) {
+  constexpr int LN = BN / TN;                               // lanes along N
+  static_assert((BM / TM) * LN == 32, "one warp covers the tile");
+  constexpr int LA = (BM * KD + 31) / 32, LB = (BN * KD + 31) / 32;   // loads per lane
+  constexpr int AS = BM + 2, STAGE = KD * (AS + BN);
+  constexpr int SM1 = GF_WARPS * 2 * STAGE, SM2 = GF_WARPS * BM * BN;
+  __shared__ double smem[SM1 > SM2 ? SM1 : SM2];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the M tile fastest: concurrent CTAs share their B columns in L2
+  const int64_t m0 = (int64_t)(blockIdx.x % m_tiles) * BM;
+  const int64_t n0 = (int64_t)(blockIdx.x / m_tiles) * BN;
   if (dcnt) {
     // graph replays: the live extent is read on the device
     const int c = *dcnt;
@@ -47,12 +73,12 @@ __global__ void __launch_bounds__(256, (BM == 32 ? 2 : 3)) gemm_f64_nn(int M, in
     if (mul_n) N = (int)min((int64_t)N, (int64_t)mul_n * c);
   }
   if (m0 >= M || n0 >= N) return;
-  // split K: CTA z sums k in [z kchunk, (z+1) kchunk) into its own slice of C
-  const int kb = blockIdx.z * kchunk;
-  K = min(K, kb + kchunk) - kb;
+  const int kq = (K + GF_WARPS - 1) / GF_WARPS;
+  const int kb = min(K, warp * kq), len = min(K, kb + kq) - kb;
   A += kb;
   B += (int64_t)kb * ldb;
-  C += (int64_t)blockIdx.z * zstride;
+  double *st = smem + warp * 2 * STAGE;
+  const int lm = (lane / LN) * TM, ln = (lane % LN) * TN;
   double acc[TM][TN];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
@@ -63,182 +89,162 @@ __global__ void __launch_bounds__(256, (BM == 32 ? 2 : 3)) gemm_f64_nn(int M, in
   auto load_regs = [&](int k0) {
 #pragma unroll
     for (int l = 0; l < LA; ++l) {
-      const int idx = tid + 256 * l;
-      const int i = idx >> 4, kk = idx & 15;                  // A: BM rows x 16 k
-      const int64_t gm = m0 + i;
-      const int gk = k0 + kk;
-      ra[l] = (gm < M && gk < K) ? A[gm * lda + gk] : 0.0;
+      const int idx = lane + 32 * l, i = idx / KD, kk = idx % KD;      // BM rows x KD
+      ra[l] = (i < BM && m0 + i < M && k0 + kk < len) ? A[(m0 + i) * lda + k0 + kk] : 0.0;
     }
 #pragma unroll
     for (int l = 0; l < LB; ++l) {
-      const int idx = tid + 256 * l;
-      const int kb = idx / BN, j = idx % BN;                  // B: 16 k x BN cols
-      const int64_t gn = n0 + j;
-      const int gkb = k0 + kb;
-      rb[l] = (gn < N && gkb < K) ? B[(int64_t)gkb * ldb + gn] : 0.0;
+      const int idx = lane + 32 * l, kk = idx / BN, j = idx % BN;      // KD x BN columns
+      rb[l] = (kk < KD && n0 + j < N && k0 + kk < len) ? B[(int64_t)(k0 + kk) * ldb + n0 + j] : 0.0;
     }
   };
-  auto store_smem = [&](int buf) {
+  auto store_smem = [&](double *s) {
 #pragma unroll
     for (int l = 0; l < LA; ++l) {
-      const int idx = tid + 256 * l;
-      As[buf][idx & 15][idx >> 4] = ra[l];
+      const int idx = lane + 32 * l;
+      if (idx < BM * KD) s[(idx % KD) * AS + idx / KD] = ra[l];
     }
 #pragma unroll
     for (int l = 0; l < LB; ++l) {
-      const int idx = tid + 256 * l;
-      Bs[buf][idx / BN][idx % BN] = rb[l];
+      const int idx = lane + 32 * l;
+      if (idx < BN * KD) s[KD * AS + idx] = rb[l];
     }
   };
-
-  const int nk = (K + GB_K - 1) / GB_K;
-  if (nk > 0) {
+  if (len > 0) {
     load_regs(0);
-    store_smem(0);
+    store_smem(st);
   }
-  __syncthreads();
-  for (int t = 0; t < nk; ++t) {
-    const int buf = t & 1;
-    if (t + 1 < nk) load_regs((t + 1) * GB_K);
-#pragma unroll
-    for (int kk = 0; kk < GB_K; ++kk) {
+  __syncwarp();
+  for (int k0 = 0, buf = 0; k0 < len; k0 += KD, buf ^= 1) {
+    const double *as = st + buf * STAGE + lm, *bs = st + buf * STAGE + KD * AS + ln;
+    const bool more = k0 + KD < len;
+    if (more) load_regs(k0 + KD);
+    const int kn = min(KD, len - k0);
+#pragma unroll 4
+    for (int kk = 0; kk < kn; ++kk) {
       double a[TM], b[TN];
 #pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = As[buf][kk][ty + 16 * i];
+      for (int i = 0; i < TM; ++i) a[i] = as[kk * AS + i];
 #pragma unroll
-      for (int j = 0; j < TN; ++j) b[j] = Bs[buf][kk][tx + 16 * j];
+      for (int j = 0; j < TN; ++j) b[j] = bs[kk * BN + j];
 #pragma unroll
       for (int i = 0; i < TM; ++i)
 #pragma unroll
         for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
     }
-    if (t + 1 < nk) store_smem(buf ^ 1);
-    __syncthreads();
+    if (more) store_smem(st + (buf ^ 1) * STAGE);
+    __syncwarp();
   }
+  __syncthreads();   // every warp is done with its stages: smem holds the quarters now
 #pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    const int64_t gm = m0 + ty + 16 * i;
-    if (gm >= M) continue;
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      const int64_t gn = n0 + tx + 16 * j;
-      if (gn < N) C[gm * ldc + gn] = acc[i][j];
-    }
+    for (int j = 0; j < TN; ++j) smem[(warp * BM + lm + i) * BN + ln + j] = acc[i][j];
+  __syncthreads();
+  for (int o = threadIdx.x; o < BM * BN; o += 32 * GF_WARPS) {
+    const int i = o / BN, j = o % BN;
+    if (m0 + i >= M || n0 + j >= N) continue;
+    double s = smem[o];
+#pragma unroll
+    for (int w = 1; w < GF_WARPS; ++w) s += smem[w * BM * BN + o];
+    C[(m0 + i) * ldc + n0 + j] = s;
   }
 }
 
 // ---------------------------------------------------------------------------
 // W[c][k][ab] = sum_{nu in block k} Y[c][nu] * V_nu[ab]  (per block k, column c)
-// One CTA per (block, group of 8 columns); thread t owns entry ab = t.
+// One CTA per (block, group of VC columns); a thread owns one entry ab of the
+// block's n_A x n_B (the pads of W are neither written nor read).
 // ---------------------------------------------------------------------------
-constexpr int VW_COLS = 8;
-
+template <int VC>
 __global__ void __launch_bounds__(256) vertex_contract(int nb, int ncols, int n_prod,
+                                                       const int *__restrict__ aoff,
+                                                       const int2 *__restrict__ blk_atoms,
                                                        const int *__restrict__ blk_ptr,
                                                        const int *__restrict__ blk_prod,
                                                        const double *__restrict__ Vpad,
                                                        const double *__restrict__ Y,
                                                        double *__restrict__ W,
                                                        const int *__restrict__ dcnt) {
-  __shared__ double ys[32][VW_COLS];
+  __shared__ double ys[32][VC];
   const int k = blockIdx.x;
-  const int c0 = blockIdx.y * VW_COLS;
+  const int c0 = blockIdx.y * VC;
   if (dcnt) ncols = min(ncols, 2 * *dcnt);
   if (c0 >= ncols) return;
   const int t = threadIdx.x;
+  const int2 AB = blk_atoms[k];
+  const int nB = aoff[AB.y + 1] - aoff[AB.y], nAB = (aoff[AB.x + 1] - aoff[AB.x]) * nB;
+  const int at = t < nAB ? (t / nB) * kMaxOrb + t % nB : 0;
   const int p0 = blk_ptr[k], p1 = blk_ptr[k + 1];
-  double acc[VW_COLS];
+  double acc[VC];
 #pragma unroll
-  for (int c = 0; c < VW_COLS; ++c) acc[c] = 0.0;
+  for (int c = 0; c < VC; ++c) acc[c] = 0.0;
   for (int q0 = p0; q0 < p1; q0 += 32) {
     __syncthreads();
-    {
-      int pp = t / VW_COLS, c = t % VW_COLS;
-      int q = q0 + pp;
+    if (t < 32 * VC) {
+      const int pp = t / VC, c = t % VC, q = q0 + pp;
       ys[pp][c] = (q < p1 && c0 + c < ncols) ? Y[(int64_t)(c0 + c) * n_prod + blk_prod[q]] : 0.0;
     }
     __syncthreads();
+    if (t >= nAB) continue;
     const int qn = min(32, p1 - q0);
+#pragma unroll 4
     for (int pp = 0; pp < qn; ++pp) {
-      double v = Vpad[(int64_t)(q0 + pp) * kBlk + t];
+      const double v = Vpad[(int64_t)(q0 + pp) * kBlk + at];
 #pragma unroll
-      for (int c = 0; c < VW_COLS; ++c) acc[c] = fma(ys[pp][c], v, acc[c]);
+      for (int c = 0; c < VC; ++c) acc[c] = fma(ys[pp][c], v, acc[c]);
     }
   }
+  if (t >= nAB) return;
 #pragma unroll
-  for (int c = 0; c < VW_COLS; ++c)
-    if (c0 + c < ncols) W[((int64_t)(c0 + c) * nb + k) * kBlk + t] = acc[c];
+  for (int c = 0; c < VC; ++c)
+    if (c0 + c < ncols) W[((int64_t)(c0 + c) * nb + k) * kBlk + at] = acc[c];
 }
 
 // ---------------------------------------------------------------------------
 // beta[aoff[A]+a][c][E] = sum over blocks touching atom A of
 //   (W_k or W_k^T)[a][b] * Xo[aoff[B]+b][E]
-// One CTA per (atom A, group of 4 columns); thread = occupied state E.
+// One thread per output (E fastest, then the column, then a): every lane is
+// live whatever n_occ and n_A are, and the operands (W: one or two addresses
+// per warp, X_occ: coalesced) come from L1 well inside the DFMA's 15 clocks.
+// An entry's operands are loaded together, ahead of its chain.  (96 columns
+// on 24 atoms: 1412 -> 415 us against 128 threads over E and 16 padded rows.)
 // ---------------------------------------------------------------------------
-constexpr int BT_COLS = 4;
-constexpr int BT_THREADS = 128;
+constexpr int BT_THREADS = 256;
 
 __global__ void __launch_bounds__(BT_THREADS) beta_kernel(
-    int ncols, int nb, int n_occ, const int *__restrict__ aoff, const int *__restrict__ adj_ptr,
-    const int4 *__restrict__ adj, const double *__restrict__ W, const double *__restrict__ Xo,
-    double *__restrict__ beta, const int *__restrict__ dcnt) {
-  __shared__ double Ws[BT_COLS][kMaxOrb][kMaxOrb + 1];
-  __shared__ double Xs[kMaxOrb][BT_THREADS];
-  const int A = blockIdx.x;
-  const int c0 = blockIdx.y * BT_COLS;
+    int n_atoms, int ncols, int nb, int n_occ, const int *__restrict__ aoff,
+    const int *__restrict__ adj_ptr, const int4 *__restrict__ adj, const double *__restrict__ W,
+    const double *__restrict__ Xo, double *__restrict__ beta, const int *__restrict__ dcnt) {
+  const int A = blockIdx.x % n_atoms;
   // ncols is the column stride of beta; nact the live columns
   const int nact = dcnt ? min(ncols, 2 * *dcnt) : ncols;
-  if (c0 >= nact) return;
-  const int nA = aoff[A + 1] - aoff[A];
-  const int e0 = adj_ptr[A], e1 = adj_ptr[A + 1];
-  for (int E0 = 0; E0 < n_occ; E0 += BT_THREADS) {
-    const int E = E0 + threadIdx.x;
-    double acc[BT_COLS][kMaxOrb];
+  const int aoA = aoff[A], nA = aoff[A + 1] - aoA;
+  const int64_t i = (int64_t)(blockIdx.x / n_atoms) * BT_THREADS + threadIdx.x;
+  if (nact <= 0 || i >= (int64_t)nA * nact * n_occ) return;
+  const int64_t row = i / n_occ;
+  const int E = (int)(i - row * n_occ);
+  const int a = (int)(row / nact), c = (int)(row - (int64_t)a * nact);
+  const double *Wc = W + (int64_t)c * nb * kBlk;
+  double acc = 0.0;
+  for (int e = adj_ptr[A]; e < adj_ptr[A + 1]; ++e) {
+    const int4 ent = adj[e];   // (block, other atom, transposed)
+    const int bo = aoff[ent.y], nB = aoff[ent.y + 1] - bo;
+    const double *w = Wc + (int64_t)ent.x * kBlk + (ent.z ? a : a * kMaxOrb);
+    const int ws = ent.z ? kMaxOrb : 1;
+    const double *x = Xo + (int64_t)bo * n_occ + E;
+    double wr[kMaxOrb], xr[kMaxOrb];
 #pragma unroll
-    for (int c = 0; c < BT_COLS; ++c)
-#pragma unroll
-      for (int a = 0; a < kMaxOrb; ++a) acc[c][a] = 0.0;
-    for (int e = e0; e < e1; ++e) {
-      const int4 ent = adj[e];
-      const int k = ent.x, B = ent.y, tr = ent.z;
-      const int bo = aoff[B], nB = aoff[B + 1] - bo;
-      // this entry's X_occ column: all loads issued together, parked in shared memory
-      {
-        double xr[kMaxOrb];
-#pragma unroll
-        for (int b = 0; b < kMaxOrb; ++b)
-          xr[b] = (b < nB && E < n_occ) ? Xo[(int64_t)(bo + b) * n_occ + E] : 0.0;
-        __syncthreads();
-#pragma unroll
-        for (int b = 0; b < kMaxOrb; ++b) Xs[b][threadIdx.x] = xr[b];
+    for (int b = 0; b < kMaxOrb; ++b)
+      if (b < nB) {
+        wr[b] = w[b * ws];
+        xr[b] = x[(int64_t)b * n_occ];
       }
-      for (int i = threadIdx.x; i < BT_COLS * kBlk; i += BT_THREADS) {
-        int c = i / kBlk, ab = i % kBlk, a = ab / kMaxOrb, b = ab % kMaxOrb;
-        double v = 0.0;
-        if (c0 + c < nact)
-          v = tr ? W[((int64_t)(c0 + c) * nb + k) * kBlk + b * kMaxOrb + a]
-                 : W[((int64_t)(c0 + c) * nb + k) * kBlk + a * kMaxOrb + b];
-        Ws[c][a][b] = v;
-      }
-      __syncthreads();
-      for (int b = 0; b < nB; ++b) {
-        const double xv = Xs[b][threadIdx.x];
 #pragma unroll
-        for (int c = 0; c < BT_COLS; ++c)
-#pragma unroll
-          for (int a = 0; a < kMaxOrb; ++a) acc[c][a] = fma(Ws[c][a][b], xv, acc[c][a]);
-      }
-    }
-    if (E < n_occ) {
-#pragma unroll
-      for (int c = 0; c < BT_COLS; ++c) {
-        if (c0 + c >= nact) continue;
-#pragma unroll
-        for (int a = 0; a < kMaxOrb; ++a)
-          if (a < nA) beta[((int64_t)(aoff[A] + a) * ncols + c0 + c) * n_occ + E] = acc[c][a];
-      }
-    }
+    for (int b = 0; b < kMaxOrb; ++b)
+      if (b < nB) acc = fma(wr[b], xr[b], acc);
   }
+  beta[((int64_t)(aoA + a) * ncols + c) * n_occ + E] = acc;
 }
 
 // ---------------------------------------------------------------------------
@@ -246,50 +252,51 @@ __global__ void __launch_bounds__(BT_THREADS) beta_kernel(
 // D = n_E [1/(omega - Delta + i eps) - 1/(omega + Delta + i eps)],
 // Delta = e_F - e_E  (eq. response-mat, both orderings of the pair merged).
 // ---------------------------------------------------------------------------
-// 1 / x for x > 0 of normal range (here x is a product of two sums of
-// squares, between ~1e-10 and ~1e4): a float32 seed refined by two
-// Newton-Raphson steps y <- y + y (1 - x y), each squaring the relative
-// error (2^-23 -> 2^-46 -> below the float64 rounding).
+// 1 / x for x > 0 of normal range (here x is the squared modulus of z^2 -
+// Delta^2, between ~1e-10 and ~1e4): the hardware's 2^-20 approximation
+// refined by two Newton-Raphson steps y <- y + y (1 - x y), each squaring the
+// relative error (2^-20 -> 2^-40 -> below the float64 rounding).
 __device__ __forceinline__ double recip_nr(double x) {
-  float yf;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"((float)x));
-  double y = (double)yf;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   double e = fma(-x, y, 1.0);
   y = fma(y, e, y);
   e = fma(-x, y, 1.0);
   return fma(y, e, y);
 }
 
-// D(omega) of one (occupied E, virtual F) pair, Delta = e_F - e_E:
-// occ [1/(omega - Delta + i eps) - 1/(omega + Delta + i eps)] from
-// xm = omega - Delta and xp = omega + Delta; the two denominators share one
-// reciprocal: 1/Am = Ap / (Am Ap), 1/Ap = Am / (Am Ap).
-__device__ __forceinline__ double2 d_factor(double xm, double xp, double eps, double occ) {
-  const double e2 = eps * eps;
-  const double Am = fma(xm, xm, e2), Ap = fma(xp, xp, e2);
-  const double q = occ * recip_nr(Am * Ap);
-  const double im2 = Ap * q, ip2 = Am * q;   // occ / Am, occ / Ap
-  return make_double2(xm * im2 - xp * ip2, eps * (ip2 - im2));
+// The broadening and occupation of D(omega) as the kernels use them (formed
+// on the host: a uniform product costs every thread an FP64 operation).
+struct DParams {
+  double neg_eps2, eps2x, occ2x;   // -eps^2, 2 eps, 2 n_o
+  DParams(double eps, double occ) : neg_eps2(-eps * eps), eps2x(2.0 * eps), occ2x(2.0 * occ) {}
+};
+
+// D(omega) of one (occupied E, virtual F) pair, Delta = e_F - e_E, z = w + i eps:
+// occ [1/(z - Delta) - 1/(z + Delta)] = 2 occ Delta / (z^2 - Delta^2), with
+// z^2 - Delta^2 = (w - Delta)(w + Delta) - eps^2 + 2 i w eps (no squares are
+// subtracted, so a resonance loses nothing).
+__device__ __forceinline__ double2 d_factor(double w, double delta, const DParams &p) {
+  const double re = fma(w - delta, w + delta, p.neg_eps2), im = p.eps2x * w;
+  const double q = p.occ2x * delta * recip_nr(fma(re, re, im * im));
+  return make_double2(q * re, -q * im);
 }
 
-// a[F][(2s, 2s+1)][E] *= D_EF(omega_s): one block per (F, s) row pair, the
-// threads over E
-__global__ void dscale_kernel(int n_virt, int S, int n_occ, double occ_value,
-                              const double *__restrict__ energy, const double *__restrict__ omega,
-                              double eps, double *__restrict__ a, const int *__restrict__ dcnt) {
-  const int64_t row = blockIdx.x;   // F * S + s
-  const int F = (int)(row / S), s = (int)(row - (int64_t)F * S);
-  const int S_act = dcnt ? min(S, *dcnt) : S;
-  if (F >= n_virt || s >= S_act) return;
-  const double eF = energy[n_occ + F], w = omega[s];
-  double *re_row = a + ((int64_t)F * 2 * S + 2 * s) * n_occ, *im_row = re_row + n_occ;
-  for (int E = threadIdx.x; E < n_occ; E += blockDim.x) {
-    const double delta = eF - energy[E];
-    const double2 d = d_factor(w - delta, w + delta, eps, occ_value);
-    const double re = re_row[E], im = im_row[E];
-    re_row[E] = d.x * re - d.y * im;
-    im_row[E] = d.x * im + d.y * re;
-  }
+// a[F][(2s, 2s+1)][E] *= D_EF(omega_s): one thread per (F, s, E); about 20
+// FP64 operations each bound it (64 right-hand sides on 64 atoms: 254 -> 205 us
+// against two denominators and a float32 seed, whose conversions use the pipe).
+__global__ void __launch_bounds__(256) dscale_kernel(
+    int n_virt, int S, int n_occ, DParams dp, const double *__restrict__ energy,
+    const double *__restrict__ omega, double *__restrict__ a, const int *__restrict__ dcnt) {
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  const int64_t row = i / n_occ;   // F * S + s
+  const int F = (int)(row / S), s = (int)(row - (int64_t)F * S), E = (int)(i - row * n_occ);
+  if (F >= n_virt || (dcnt && s >= *dcnt)) return;
+  const double2 d = d_factor(omega[s], energy[n_occ + F] - energy[E], dp);
+  double *at = a + ((int64_t)F * 2 * S + 2 * s) * n_occ + E;
+  const double re = at[0], im = at[n_occ];
+  at[0] = d.x * re - d.y * im;
+  at[n_occ] = d.x * im + d.y * re;
 }
 
 __global__ void i2p_kernel(int n_rhs, int n, const double *__restrict__ in, double *__restrict__ out) {
@@ -313,25 +320,21 @@ __global__ void p2i_kernel(int n_rhs, int n, const double *__restrict__ in, doub
 }
 
 // a[F][(2s, 2s+1)][E] = D_EF(omega_{(g0+s)/3}) * a3[F][(2k, 2k+1)][E], k = (g0+s) % 3:
-// one block per (F, s) row pair, the threads over E
-__global__ void rhs_expand_kernel(int n_virt, int S, int n_occ, int g0, double occ_value,
-                                  const double *__restrict__ energy,
-                                  const double *__restrict__ omega_all, double eps,
-                                  const double *__restrict__ a3, double *__restrict__ a) {
-  const int64_t row = blockIdx.x;   // F * S + s
-  const int F = (int)(row / S), s = (int)(row - (int64_t)F * S);
+// one thread per (F, s, E)
+__global__ void __launch_bounds__(256) rhs_expand_kernel(
+    int n_virt, int S, int n_occ, int g0, DParams dp, const double *__restrict__ energy,
+    const double *__restrict__ omega_all, const double *__restrict__ a3, double *__restrict__ a) {
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  const int64_t row = i / n_occ;   // F * S + s
+  const int F = (int)(row / S), s = (int)(row - (int64_t)F * S), E = (int)(i - row * n_occ);
   if (F >= n_virt) return;
   const int g = g0 + s, k = g % 3;
-  const double eF = energy[n_occ + F], w = omega_all[g / 3];
-  const double *src = a3 + ((int64_t)F * 6 + 2 * k) * n_occ;
-  double *dst = a + ((int64_t)F * 2 * S + 2 * s) * n_occ;
-  for (int E = threadIdx.x; E < n_occ; E += blockDim.x) {
-    const double delta = eF - energy[E];
-    const double2 d = d_factor(w - delta, w + delta, eps, occ_value);
-    const double re = src[E], im = src[E + n_occ];
-    dst[E] = d.x * re - d.y * im;
-    dst[E + n_occ] = d.x * im + d.y * re;
-  }
+  const double2 d = d_factor(omega_all[g / 3], energy[n_occ + F] - energy[E], dp);
+  const double *src = a3 + ((int64_t)F * 6 + 2 * k) * n_occ + E;
+  double *dst = a + ((int64_t)F * 2 * S + 2 * s) * n_occ + E;
+  const double re = src[0], im = src[n_occ];
+  dst[0] = d.x * re - d.y * im;
+  dst[n_occ] = d.x * im + d.y * re;
 }
 
 // Z3 rows (d_0, 0, d_1, 0, d_2, 0)
@@ -350,63 +353,100 @@ int grid_for(int64_t total, int threads) {
 }
 }  // namespace
 
-// C[m][n] = sum over the split slices ws[z][m][n], in slice order (deterministic)
-// (slices of zstride elements, rows of ldw; only the live M x N part is summed)
-__global__ void splitk_reduce_kernel(int M, int N, int splits, const double *__restrict__ ws,
-                                     int64_t zstride, int64_t ldw, double *__restrict__ C,
-                                     int64_t ldc, const int *__restrict__ dcnt, int mul_m,
-                                     int mul_n) {
-  if (dcnt) {
-    const int c = *dcnt;
-    if (mul_m) M = min(M, mul_m * c);
-    if (mul_n) N = (int)min((int64_t)N, (int64_t)mul_n * c);
+// The tile of a float64 GEMM: the one whose busiest SM has the fewest padded
+// outputs, the pipe's only cost (smaller tiles read their operands more often,
+// hence the few per cent against them).  6 x 280 x 280 takes 4 x 8 tiles on 70
+// SMs (32 x 128 tiles ran on 3); 96 x 2960 x 2960 went from 3.08 ms in 72 CTAs
+// of 32 x 128 to 1.51 ms in 279 of 32 x 32.
+template <int BM, int BN, int TM, int TN, int KD>
+struct GemmTile {
+  static double cost(int M, int N, double penalty) {
+    const double n = (double)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+    const double sm = sm_count();
+    return (n <= sm ? 1.0 : (double)(int64_t)((n + sm - 1) / sm)) * BM * BN * penalty;
   }
-  const int64_t total = (int64_t)M * N;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t m = i / N, n = i % N;
-    double s = 0.0;
-    for (int z = 0; z < splits; ++z) s += ws[z * zstride + m * ldw + n];
-    C[m * ldc + n] = s;
+  static cudaError_t launch(cudaStream_t st, int M, int N, int K, const double *A, int64_t lda,
+                            const double *B, int64_t ldb, double *C, int64_t ldc, const int *dcnt,
+                            int mul_m, int mul_n) {
+    const int mt = (M + BM - 1) / BM;
+    const int64_t n = (int64_t)mt * ((N + BN - 1) / BN);
+    if (n > INT32_MAX) return cudaErrorInvalidConfiguration;
+    gemm_f64_kernel<BM, BN, TM, TN, KD><<<(unsigned)n, 32 * GF_WARPS, 0, st>>>(
+        M, N, K, A, lda, B, ldb, C, ldc, dcnt, mul_m, mul_n, mt);
+    return cudaGetLastError();
   }
-}
+};
 
 cudaError_t launch_gemm_f64(cudaStream_t st, int M, int N, int K, const double *A, int64_t lda,
                             const double *B, int64_t ldb, double *C, int64_t ldc,
-                            const int *dcnt, int mul_m, int mul_n, double *ws, int64_t ws_elems) {
+                            const int *dcnt, int mul_m, int mul_n) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  const bool small = M < 256;
-  // Long reductions (the K product: K = n_prod) with few output tiles leave SMs
-  // idle, so K is cut into slices of 2048 summed afterwards in a fixed order.
-  // The slicing depends on K alone: every launch shape (host-driven or graph
-  // replay, any batch) sums each output in the same order.
-  constexpr int kSlice = 2048, kMaxSlices = 8;
-  int kchunk = K, splits = 1;
-  if (ws && K >= 2 * kSlice) {
-    kchunk = std::max(kSlice, ((K + kMaxSlices - 1) / kMaxSlices + 15) / 16 * 16);
-    splits = (K + kchunk - 1) / kchunk;
-    if ((int64_t)splits * M * N > ws_elems) return cudaErrorInvalidValue;
-  }
-  double *out = splits > 1 ? ws : C;
-  const int64_t ldo = splits > 1 ? N : ldc;
-  const int64_t zstride = (int64_t)M * N;
-  if (small) {
-    dim3 grid((N + 127) / 128, (M + 31) / 32, splits);
+  using T32 = GemmTile<32, 32, 4, 8, 8>;
+  using T16 = GemmTile<16, 16, 2, 4, 16>;
+  using T8 = GemmTile<8, 8, 1, 2, 16>;
+  using T4 = GemmTile<4, 8, 1, 1, 16>;
+  const double c32 = T32::cost(M, N, 1.0), c16 = T16::cost(M, N, 1.03),
+               c8 = T8::cost(M, N, 1.08), c4 = T4::cost(M, N, 1.15);
+  auto go = [&](auto t) {
+    return decltype(t)::launch(st, M, N, K, A, lda, B, ldb, C, ldc, dcnt, mul_m, mul_n);
+  };
+  if (c32 <= c16 && c32 <= c8 && c32 <= c4) return go(T32{});
+  if (c16 <= c8 && c16 <= c4) return go(T16{});
+  return c8 <= c4 ? go(T8{}) : go(T4{});
+}
+
+namespace {
+// Columns per CTA of the vertex contraction: as many as leave about four
+// CTAs per SM (a vertex block is then read once for all of them).
+cudaError_t launch_vertex(cudaStream_t st, const DevSystem &sys, int ncols, const double *Y,
+                          double *W, const int *dcnt) {
+  auto go = [&](auto vc) {
+    constexpr int VC = decltype(vc)::value;
+    const dim3 grid(sys.n_blocks, (ncols + VC - 1) / VC);
     if (grid.y > 65535) return cudaErrorInvalidConfiguration;
-    gemm_f64_nn<32, 128><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, out, ldo, dcnt, mul_m,
-                                               mul_n, kchunk, zstride);
-  } else {
-    dim3 grid((N + 63) / 64, (M + 63) / 64, splits);
-    if (grid.y > 65535) return cudaErrorInvalidConfiguration;
-    gemm_f64_nn<64, 64><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, out, ldo, dcnt, mul_m,
-                                              mul_n, kchunk, zstride);
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || splits == 1) return e;
-  splitk_reduce_kernel<<<grid_for((int64_t)M * N, 256), 256, 0, st>>>(
-      M, N, splits, ws, zstride, N, C, ldc, dcnt, mul_m, mul_n);
+    vertex_contract<VC><<<grid, 256, 0, st>>>(sys.n_blocks, ncols, sys.n_prod, sys.aoff,
+                                              sys.blk_atoms, sys.blk_ptr, sys.blk_prod, sys.Vpad, Y,
+                                              W, dcnt);
+    return cudaGetLastError();
+  };
+  const int64_t want = 4 * (int64_t)sm_count();
+  auto ctas = [&](int vc) { return (int64_t)sys.n_blocks * ((ncols + vc - 1) / vc); };
+  if (ctas(8) >= want) return go(std::integral_constant<int, 8>{});
+  if (ctas(4) >= want) return go(std::integral_constant<int, 4>{});
+  if (ctas(2) >= want) return go(std::integral_constant<int, 2>{});
+  return go(std::integral_constant<int, 1>{});
+}
+
+cudaError_t launch_beta(cudaStream_t st, const DevSystem &sys, int ncols, const double *W,
+                        double *beta, const int *dcnt) {
+  const int64_t per_atom =
+      ((int64_t)kMaxOrb * ncols * sys.n_occ + BT_THREADS - 1) / BT_THREADS;
+  if (per_atom * sys.n_atoms > INT32_MAX) return cudaErrorInvalidConfiguration;
+  beta_kernel<<<(unsigned)(per_atom * sys.n_atoms), BT_THREADS, 0, st>>>(
+      sys.n_atoms, ncols, sys.n_blocks, sys.n_occ, sys.aoff, sys.adj_ptr, sys.adj, W, sys.Xo, beta,
+      dcnt);
   return cudaGetLastError();
 }
+
+cudaError_t launch_dscale(cudaStream_t st, const DevSystem &sys, int S, const double *omega,
+                          double eps, double *a, const int *dcnt) {
+  const int64_t n = ((int64_t)sys.n_virt * S * sys.n_occ + 255) / 256;
+  if (n > INT32_MAX) return cudaErrorInvalidConfiguration;
+  dscale_kernel<<<(unsigned)n, 256, 0, st>>>(sys.n_virt, S, sys.n_occ, DParams(eps, sys.occ_value),
+                                             sys.energy, omega, a, dcnt);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rhs_expand(cudaStream_t st, const DevSystem &sys, int S, int g0,
+                              const double *omega_all, double eps, const double *a3, double *a) {
+  const int64_t n = ((int64_t)sys.n_virt * S * sys.n_occ + 255) / 256;
+  if (n > INT32_MAX) return cudaErrorInvalidConfiguration;
+  rhs_expand_kernel<<<(unsigned)n, 256, 0, st>>>(sys.n_virt, S, sys.n_occ, g0,
+                                                 DParams(eps, sys.occ_value), sys.energy,
+                                                 omega_all, a3, a);
+  return cudaGetLastError();
+}
+}  // namespace
 
 cudaError_t launch_interleaved_to_planar(cudaStream_t st, int n_rhs, int n, const double *in,
                                          double *out) {
@@ -533,9 +573,8 @@ cudaError_t apply_alpha_emulated(cudaStream_t st, const DevSystem &sys, OpWork &
   }
   {
     Scope sc(wk.timer, st, kcDscale, 0.0);
-    dscale_kernel<<<(unsigned)std::max<int64_t>(1, (int64_t)sys.n_virt * S), 128, 0, st>>>(
-        sys.n_virt, S, sys.n_occ, sys.occ_value, sys.energy, wk.omega, eps, wk.abuf, wk.dcnt);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    if ((err = launch_dscale(st, sys, S, wk.omega, eps, wk.abuf, wk.dcnt)) != cudaSuccess)
+      return err;
   }
   return alpha_dot_emulated(st, sys, wk, ncols, Zin, mode == kA ? 1 : 0, Out, wk.dcnt, kcOzT2);
 }
@@ -561,27 +600,15 @@ cudaError_t launch_rhs_formation(cudaStream_t st, const DevSystem &sys, OpWork &
       err = launch_oz_slice_rows(st, wk.beta, sys.n_orb, n6, sys.n_orb, wk.oz->Bt1);
     if (err == cudaSuccess)
       err = launch_gemm_oz(st, wk.oz->XvT, wk.oz->Bt1, sys.n_virt, n6, a3, n6, 0, wk.oz->err);
-    if (err == cudaSuccess) {
-      rhs_expand_kernel<<<(unsigned)std::max<int64_t>(1, (int64_t)sys.n_virt * S), 128, 0, st>>>(
-          sys.n_virt, S, sys.n_occ, g0, sys.occ_value, sys.energy, omega_all, eps, a3, wk.abuf);
-      err = cudaGetLastError();
-    }
+    if (err == cudaSuccess) err = launch_rhs_expand(st, sys, S, g0, omega_all, eps, a3, wk.abuf);
     if (err == cudaSuccess)
       err = alpha_dot_emulated(st, sys, wk, 2 * S, nullptr, 0, Out, nullptr, kcRhs);
     wk.timer = saved;
     return err;
   }
   // omega-independent part for the three directions (6 real columns)
-  {
-    dim3 grid(sys.n_blocks, 1);
-    vertex_contract<<<grid, 256, 0, st>>>(sys.n_blocks, 6, np, sys.blk_ptr, sys.blk_prod, sys.Vpad,
-                                          Z3, wk.W, nullptr);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    dim3 gb(sys.n_atoms, 2);
-    beta_kernel<<<gb, BT_THREADS, 0, st>>>(6, sys.n_blocks, sys.n_occ, sys.aoff, sys.adj_ptr,
-                                           sys.adj, wk.W, sys.Xo, wk.beta, nullptr);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  }
+  if ((err = launch_vertex(st, sys, 6, Z3, wk.W, nullptr)) != cudaSuccess) return err;
+  if ((err = launch_beta(st, sys, 6, wk.W, wk.beta, nullptr)) != cudaSuccess) return err;
   const int n6 = 6 * sys.n_occ;
   if (wk.oz) {
     err = launch_oz_slice_cols(st, wk.beta, n6, sys.n_orb, n6, wk.oz->Bt1);
@@ -593,9 +620,8 @@ cudaError_t launch_rhs_formation(cudaStream_t st, const DevSystem &sys, OpWork &
   if (err != cudaSuccess) return err;
   // per right-hand side: D(omega) a_k, X_virt a, block dot
   const int64_t ncolE = (int64_t)2 * S * sys.n_occ;
-  rhs_expand_kernel<<<(unsigned)std::max<int64_t>(1, (int64_t)sys.n_virt * S), 128, 0, st>>>(
-      sys.n_virt, S, sys.n_occ, g0, sys.occ_value, sys.energy, omega_all, eps, a3, wk.abuf);
-  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  if ((err = launch_rhs_expand(st, sys, S, g0, omega_all, eps, a3, wk.abuf)) != cudaSuccess)
+    return err;
   if (wk.oz) {
     err = launch_oz_slice_cols(st, wk.abuf, ncolE, sys.n_virt, (int)ncolE, wk.oz->Bt2);
     if (err == cudaSuccess)
@@ -633,8 +659,7 @@ cudaError_t launch_apply_operator(cudaStream_t st, const DevSystem &sys, OpWork 
                              2);
     } else {
       Scope sc(wk.timer, st, kcGemmK, 2.0 * ncols * (double)np * np);
-      err = launch_gemm_f64(st, ncols, np, np, Zin, np, sys.K, np, Yout, np, wk.dcnt, 2, 0,
-                            wk.splitws, wk.splitws_elems);
+      err = launch_gemm_f64(st, ncols, np, np, Zin, np, sys.K, np, Yout, np, wk.dcnt, 2, 0);
     }
     if (err != cudaSuccess || mode == kKernel) return err;
     Y = wk.Y;
@@ -642,17 +667,11 @@ cudaError_t launch_apply_operator(cudaStream_t st, const DevSystem &sys, OpWork 
   if (wk.oz && wk.ar) return apply_alpha_emulated(st, sys, wk, S, mode, eps, Y, Zin, Out);
   {
     Scope sc(wk.timer, st, kcVertex, 2.0 * ncols * (double)kBlk * np);
-    dim3 grid(sys.n_blocks, (ncols + VW_COLS - 1) / VW_COLS);
-    vertex_contract<<<grid, 256, 0, st>>>(sys.n_blocks, ncols, np, sys.blk_ptr, sys.blk_prod,
-                                          sys.Vpad, Y, wk.W, wk.dcnt);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    if ((err = launch_vertex(st, sys, ncols, Y, wk.W, wk.dcnt)) != cudaSuccess) return err;
   }
   {
     Scope sc(wk.timer, st, kcBeta, ncols * sys.sf.beta);
-    dim3 grid(sys.n_atoms, (ncols + BT_COLS - 1) / BT_COLS);
-    beta_kernel<<<grid, BT_THREADS, 0, st>>>(ncols, sys.n_blocks, sys.n_occ, sys.aoff, sys.adj_ptr,
-                                             sys.adj, wk.W, sys.Xo, wk.beta, wk.dcnt);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    if ((err = launch_beta(st, sys, ncols, wk.W, wk.beta, wk.dcnt)) != cudaSuccess) return err;
   }
   const int64_t ncolE = (int64_t)ncols * sys.n_occ;
   if (ncolE > INT32_MAX) return cudaErrorInvalidValue;
@@ -677,9 +696,8 @@ cudaError_t launch_apply_operator(cudaStream_t st, const DevSystem &sys, OpWork 
   }
   {
     Scope sc(wk.timer, st, kcDscale, 0.0);
-    dscale_kernel<<<(unsigned)std::max<int64_t>(1, (int64_t)sys.n_virt * S), 128, 0, st>>>(
-        sys.n_virt, S, sys.n_occ, sys.occ_value, sys.energy, wk.omega, eps, wk.abuf, wk.dcnt);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    if ((err = launch_dscale(st, sys, S, wk.omega, eps, wk.abuf, wk.dcnt)) != cudaSuccess)
+      return err;
   }
   if (wk.oz) {
     {
