@@ -252,47 +252,47 @@ __global__ void __launch_bounds__(BT_THREADS) beta_kernel(
 // D = n_E [1/(omega - Delta + i eps) - 1/(omega + Delta + i eps)],
 // Delta = e_F - e_E  (eq. response-mat, both orderings of the pair merged).
 // ---------------------------------------------------------------------------
-// 1 / x for x > 0 of normal range (here x is the squared modulus of z^2 -
-// Delta^2, between ~1e-10 and ~1e4): the hardware's 2^-20 approximation
-// refined by two Newton-Raphson steps y <- y + y (1 - x y), each squaring the
-// relative error (2^-20 -> 2^-40 -> below the float64 rounding).
+// 1 / x for x > 0 of normal range (here x is a product of two sums of
+// squares, between ~1e-10 and ~1e4): a float32 seed refined by two
+// Newton-Raphson steps y <- y + y (1 - x y), each squaring the relative
+// error (2^-23 -> 2^-46 -> below the float64 rounding).
 __device__ __forceinline__ double recip_nr(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  float yf;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"((float)x));
+  double y = (double)yf;
   double e = fma(-x, y, 1.0);
   y = fma(y, e, y);
   e = fma(-x, y, 1.0);
   return fma(y, e, y);
 }
 
-// The broadening and occupation of D(omega) as the kernels use them (formed
-// on the host: a uniform product costs every thread an FP64 operation).
-struct DParams {
-  double neg_eps2, eps2x, occ2x;   // -eps^2, 2 eps, 2 n_o
-  DParams(double eps, double occ) : neg_eps2(-eps * eps), eps2x(2.0 * eps), occ2x(2.0 * occ) {}
-};
-
-// D(omega) of one (occupied E, virtual F) pair, Delta = e_F - e_E, z = w + i eps:
-// occ [1/(z - Delta) - 1/(z + Delta)] = 2 occ Delta / (z^2 - Delta^2), with
-// z^2 - Delta^2 = (w - Delta)(w + Delta) - eps^2 + 2 i w eps (no squares are
-// subtracted, so a resonance loses nothing).
-__device__ __forceinline__ double2 d_factor(double w, double delta, const DParams &p) {
-  const double re = fma(w - delta, w + delta, p.neg_eps2), im = p.eps2x * w;
-  const double q = p.occ2x * delta * recip_nr(fma(re, re, im * im));
-  return make_double2(q * re, -q * im);
+// D(omega) of one (occupied E, virtual F) pair, Delta = e_F - e_E:
+// occ [1/(omega - Delta + i eps) - 1/(omega + Delta + i eps)] from
+// xm = omega - Delta and xp = omega + Delta; the two denominators share one
+// reciprocal: 1/Am = Ap / (Am Ap), 1/Ap = Am / (Am Ap).
+// (A refinement cycle of the emulated forms amplifies the last bit of D:
+// 2 occ Delta / (z^2 - Delta^2) saves five FP64 operations and moves a
+// converged spectrum by 3e-9, so the form is kept.)
+__device__ __forceinline__ double2 d_factor(double w, double delta, double eps, double e2,
+                                            double occ) {
+  const double xm = w - delta, xp = w + delta;
+  const double Am = fma(xm, xm, e2), Ap = fma(xp, xp, e2);
+  const double q = occ * recip_nr(Am * Ap);
+  const double im2 = Ap * q, ip2 = Am * q;   // occ / Am, occ / Ap
+  return make_double2(xm * im2 - xp * ip2, eps * (ip2 - im2));
 }
 
-// a[F][(2s, 2s+1)][E] *= D_EF(omega_s): one thread per (F, s, E); about 20
-// FP64 operations each bound it (64 right-hand sides on 64 atoms: 254 -> 205 us
-// against two denominators and a float32 seed, whose conversions use the pipe).
+// a[F][(2s, 2s+1)][E] *= D_EF(omega_s): one thread per (F, s, E), about
+// 25 FP64 operations each, which bound it (64 right-hand sides on 64 atoms: 254 us)
 __global__ void __launch_bounds__(256) dscale_kernel(
-    int n_virt, int S, int n_occ, DParams dp, const double *__restrict__ energy,
-    const double *__restrict__ omega, double *__restrict__ a, const int *__restrict__ dcnt) {
+    int n_virt, int S, int n_occ, double occ_value, const double *__restrict__ energy,
+    const double *__restrict__ omega, double eps, double e2, double *__restrict__ a,
+    const int *__restrict__ dcnt) {
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   const int64_t row = i / n_occ;   // F * S + s
   const int F = (int)(row / S), s = (int)(row - (int64_t)F * S), E = (int)(i - row * n_occ);
   if (F >= n_virt || (dcnt && s >= *dcnt)) return;
-  const double2 d = d_factor(omega[s], energy[n_occ + F] - energy[E], dp);
+  const double2 d = d_factor(omega[s], energy[n_occ + F] - energy[E], eps, e2, occ_value);
   double *at = a + ((int64_t)F * 2 * S + 2 * s) * n_occ + E;
   const double re = at[0], im = at[n_occ];
   at[0] = d.x * re - d.y * im;
@@ -322,14 +322,16 @@ __global__ void p2i_kernel(int n_rhs, int n, const double *__restrict__ in, doub
 // a[F][(2s, 2s+1)][E] = D_EF(omega_{(g0+s)/3}) * a3[F][(2k, 2k+1)][E], k = (g0+s) % 3:
 // one thread per (F, s, E)
 __global__ void __launch_bounds__(256) rhs_expand_kernel(
-    int n_virt, int S, int n_occ, int g0, DParams dp, const double *__restrict__ energy,
-    const double *__restrict__ omega_all, const double *__restrict__ a3, double *__restrict__ a) {
+    int n_virt, int S, int n_occ, int g0, double occ_value, const double *__restrict__ energy,
+    const double *__restrict__ omega_all, double eps, double e2, const double *__restrict__ a3,
+    double *__restrict__ a) {
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   const int64_t row = i / n_occ;   // F * S + s
   const int F = (int)(row / S), s = (int)(row - (int64_t)F * S), E = (int)(i - row * n_occ);
   if (F >= n_virt) return;
   const int g = g0 + s, k = g % 3;
-  const double2 d = d_factor(omega_all[g / 3], energy[n_occ + F] - energy[E], dp);
+  const double2 d =
+      d_factor(omega_all[g / 3], energy[n_occ + F] - energy[E], eps, e2, occ_value);
   const double *src = a3 + ((int64_t)F * 6 + 2 * k) * n_occ + E;
   double *dst = a + ((int64_t)F * 2 * S + 2 * s) * n_occ + E;
   const double re = src[0], im = src[n_occ];
@@ -432,8 +434,8 @@ cudaError_t launch_dscale(cudaStream_t st, const DevSystem &sys, int S, const do
                           double eps, double *a, const int *dcnt) {
   const int64_t n = ((int64_t)sys.n_virt * S * sys.n_occ + 255) / 256;
   if (n > INT32_MAX) return cudaErrorInvalidConfiguration;
-  dscale_kernel<<<(unsigned)n, 256, 0, st>>>(sys.n_virt, S, sys.n_occ, DParams(eps, sys.occ_value),
-                                             sys.energy, omega, a, dcnt);
+  dscale_kernel<<<(unsigned)n, 256, 0, st>>>(sys.n_virt, S, sys.n_occ, sys.occ_value, sys.energy,
+                                             omega, eps, eps * eps, a, dcnt);
   return cudaGetLastError();
 }
 
@@ -442,8 +444,8 @@ cudaError_t launch_rhs_expand(cudaStream_t st, const DevSystem &sys, int S, int 
   const int64_t n = ((int64_t)sys.n_virt * S * sys.n_occ + 255) / 256;
   if (n > INT32_MAX) return cudaErrorInvalidConfiguration;
   rhs_expand_kernel<<<(unsigned)n, 256, 0, st>>>(sys.n_virt, S, sys.n_occ, g0,
-                                                 DParams(eps, sys.occ_value), sys.energy,
-                                                 omega_all, a3, a);
+                                                 sys.occ_value, sys.energy, omega_all, eps,
+                                                 eps * eps, a3, a);
   return cudaGetLastError();
 }
 }  // namespace
