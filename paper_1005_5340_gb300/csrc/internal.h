@@ -216,6 +216,12 @@ void tc_init_attributes();
 // with split_ok (the K product): A of M rows and padded K Kp, N columns, N tile bn.
 void tc_split_plan(int Kp, int M, int N, int bn, int *ksplit, int *ncl);
 
+// Stream-ordered scratch from the library's pool of the current device
+// (scratch.cu); freed with cudaFreeAsync on the same stream.  scratch_trim
+// gives back what the pools keep.
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st);
+void scratch_trim();
+
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
 // Warm-started sweep (sweep.cu): frequencies solved per chunk, one solver
@@ -268,9 +274,8 @@ cudaError_t launch_apply_operator_lp(cudaStream_t st, const DevSystem &sys, LpWo
 //   x[r][k] = 2^e[r] * sum_i q_i[r][k] 2^(-7 i),   |q_1| <= 128, |q_i| <= 64,
 // stored as exact bf16 integers [rows][s*Kp] (slice i at column i*Kp).
 struct OzOperand {
-  CUtensorMap map;     // boxes of 64 columns x box_rows rows
-  CUtensorMap map96;   // B role only: boxes of 96 rows (has96)
-  bool has96 = false;
+  CUtensorMap map;       // boxes of 64 columns x box_rows rows
+  CUtensorMap map_wide;  // B role only: boxes of the wide N tile's rows
   __nv_bfloat16 *q = nullptr;
   int *e = nullptr;
   int64_t rows = 0;
@@ -282,7 +287,7 @@ constexpr int kOzDefaultSlices = 6;
 
 // Allocation-free set-up of an operand over caller-owned storage
 // (q: rows * s * Kp bf16, 16-byte aligned; e: rows ints).  box_rows 128 for
-// the A role, 64 for the B role.
+// the A role, 64 for the B role (its N tiles).
 cudaError_t oz_operand(OzOperand &op, __nv_bfloat16 *q, int *e, int64_t rows, int Kdim, int s,
                        int box_rows);
 // Slices of rows r < rows (live rows mul*dcnt) of X [rows][ldx] (first Kdim

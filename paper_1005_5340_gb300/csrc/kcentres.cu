@@ -127,23 +127,21 @@ extern "C" tddft_status tddft_kernel_apply_centres(int32_t n_prod, int32_t n_cen
   std::vector<int> members(n_prod), fill(count.begin(), count.end() - 1);
   for (int mu = 0; mu < n_prod; ++mu) members[fill[prod_centre[mu]]++] = mu;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  std::vector<void *> allocs;
-  auto alloc = [&](size_t bytes, void **p) -> cudaError_t {
-    cudaError_t e = cudaMalloc(p, bytes);
-    if (e == cudaSuccess) allocs.push_back(*p);
-    return e;
-  };
-  void *d_c = nullptr, *d_ptr = nullptr, *d_mem = nullptr, *d_pc = nullptr, *d_Q = nullptr,
-       *d_H = nullptr;
-  cudaError_t e = alloc((size_t)n_centres * 3 * sizeof(double), &d_c);
-  if (e == cudaSuccess) e = alloc(count.size() * sizeof(int), &d_ptr);
-  if (e == cudaSuccess) e = alloc((size_t)n_prod * sizeof(int), &d_mem);
-  if (e == cudaSuccess) e = alloc((size_t)n_prod * sizeof(int), &d_pc);
-  if (e == cudaSuccess) e = alloc((size_t)n_rhs * n_centres * sizeof(double2), &d_Q);
-  if (e == cudaSuccess) e = alloc((size_t)n_rhs * n_centres * sizeof(double2), &d_H);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(d_c, centres, (size_t)n_centres * 3 * sizeof(double),
-                        cudaMemcpyHostToDevice, st);
+  // one scratch block: centres, member lists, charges and potentials
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  const size_t n_c = up((size_t)n_centres * 3 * sizeof(double)),
+               n_ptr = up(count.size() * sizeof(int)), n_mem = up((size_t)n_prod * sizeof(int)),
+               n_q = up((size_t)n_rhs * n_centres * sizeof(double2));
+  char *ws = nullptr;
+  cudaError_t e = tddft::scratch_alloc((void **)&ws, n_c + n_ptr + 2 * n_mem + 2 * n_q, st);
+  if (e != cudaSuccess) {
+    cudaGetLastError();   // not left for a later check
+    return e == cudaErrorMemoryAllocation ? TDDFT_ERR_NOMEM : TDDFT_ERR_CUDA;
+  }
+  char *d_c = ws, *d_ptr = d_c + n_c, *d_mem = d_ptr + n_ptr, *d_pc = d_mem + n_mem,
+       *d_Q = d_pc + n_mem, *d_H = d_Q + n_q;
+  e = cudaMemcpyAsync(d_c, centres, (size_t)n_centres * 3 * sizeof(double), cudaMemcpyHostToDevice,
+                      st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_ptr, count.data(), count.size() * sizeof(int), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
@@ -164,8 +162,9 @@ extern "C" tddft_status tddft_kernel_apply_centres(int32_t n_prod, int32_t n_cen
                                   (const double2 *)z, (const double2 *)d_H, (double2 *)out);
     e = cudaGetLastError();
   }
+  const cudaError_t ef = cudaFreeAsync(ws, st);
+  if (e == cudaSuccess) e = ef;
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  for (void *p : allocs) cudaFree(p);
   if (e == cudaErrorMemoryAllocation) return TDDFT_ERR_NOMEM;
   return e == cudaSuccess ? TDDFT_OK : TDDFT_ERR_CUDA;
 }

@@ -34,15 +34,20 @@
 // Every mbarrier wait is bounded; on expiry the CTA records an error code,
 // stops issuing work, waits (bounded) for its TMA copies in flight and still
 // frees its TMEM.
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
 #include "tc_ptx.h"
+
+namespace cg = cooperative_groups;
 
 namespace tddft {
 namespace {
@@ -52,9 +57,11 @@ constexpr int OZ_BM = 128, OZ_BN = 64, OZ_BK = 64;
 constexpr int OZ_EPI_WARPS = 8;                        // 2 per TMEM lane quadrant
 constexpr int OZ_THREADS = 64 + 32 * OZ_EPI_WARPS;      // producer, MMA, epilogue
 constexpr uint32_t OZ_A_BYTES = OZ_BM * OZ_BK * 2;   // 16 KB
-// The N tile: 96 columns where the s groups fit in tensor memory (s x 96 <=
-// 512, s <= 5), else 64; each MMA then does 1.5x the work for the same A
-// tile read from shared memory.  9 stages of 24 KB, or 8 of 28 KB.
+// The N tile is 64 columns or the widest of 96 and 80 whose s groups fit in
+// tensor memory (s x BN <= 512), chosen per launch (tile_plan): an MMA reads
+// its A tile from shared memory whatever its N, and the operand reads bound
+// it, so a wide tile does more per read and a narrow one pads less.
+// 9 stages of 24 KB, or 8 of 26 or 28 KB.
 template <int BN> struct OzShape {
   static constexpr int EPI_COLS = BN / 2;                      // columns per epilogue thread
   static constexpr uint32_t B_BYTES = BN * OZ_BK * 2;
@@ -62,7 +69,9 @@ template <int BN> struct OzShape {
   static constexpr int STAGES = BN == 64 ? 9 : 8;
   static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + 256;
 };
-__host__ __device__ constexpr int oz_bn(int S) { return S * 96 <= 512 ? 96 : 64; }
+__host__ __device__ constexpr int oz_wide_bn(int S) {
+  return S * 96 <= 512 ? 96 : (S * 80 <= 512 ? 80 : 64);
+}
 
 struct OzArgs {
   int M, N;
@@ -75,6 +84,8 @@ struct OzArgs {
   const GTile *tiles;   // grouped product: one entry per M tile (NULL: plain row tiles)
   int mgroup;           // M tiles per group of the L2-aware tile order
   int Mt, Nt;           // M tiles (rows / 128, or table entries) and N tiles
+  int drop;             // low bits dropped from the integer accumulators (drop_bits)
+  int ksplit;           // > 1: a cluster of ksplit CTAs per tile, each a share of its K chunks
   int *err;
   const int *dcnt;
   int mul_n;
@@ -82,8 +93,15 @@ struct OzArgs {
 
 // Low bits dropped from the integer accumulator for S slices: with u(S) the
 // largest value, 2^(24 + 7(S-1) - u) summed over up to 1024 chunks (and the
-// lower groups, < 1% more) stays below 2^63.
-__host__ __device__ constexpr int oz_drop_bits(int S) { return 7 * S - 35 > 0 ? 7 * S - 35 : 0; }
+// lower groups, < 1% more) stays below 2^63.  With 8 slices the drop's own
+// rounding would exceed the slices' error, so there it follows the product's
+// chunk count (2^10 chunks at most: every halving needs one bit less).
+int drop_bits(int S, int chunks) {
+  int u = std::max(0, 7 * S - 35);
+  if (S == 8)
+    for (int c = 1024; u > 0 && c / 2 >= chunks; c /= 2) --u;
+  return u;
+}
 constexpr int kOzMaxChunks = 1024;
 
 // acc += G_t of every group (t = grp + 2) read from tensor memory (this
@@ -106,18 +124,21 @@ __device__ __forceinline__ void add_group(long long (&acc)[EC], const float *v, 
 
 // tcol: this thread's lane and its first column (h EPI_COLS) in group 0.
 // With 96-wide groups, half h = 0 reads 32 + 16 columns, h = 1 reads 16 +
-// 32, so that every 32-column load starts on a multiple of 32 columns.
+// 32, so that every 32-column load starts on a multiple of 32 columns; the
+// 40 columns of an 80-wide group's half are five 8-column loads.
 template <int S, int BN>
 __device__ __forceinline__ void read_groups(uint32_t tcol, int h,
                                             long long (&acc)[OzShape<BN>::EPI_COLS], int ns,
-                                            uint64_t *tempty) {
+                                            int drop, uint64_t *tempty) {
 #pragma unroll 1
   for (int grp = 0; grp < ns; ++grp) {
-    const int sh = 7 * (S - 1 - grp) - oz_drop_bits(S);
+    const int sh = 7 * (S - 1 - grp) - drop;
     const uint32_t g0 = tcol + (uint32_t)(grp * BN);
-    float v[32], u[16];
-    if (BN == 64) {
+    float v[BN == 80 ? 40 : 32], u[16];
+    if constexpr (BN == 64) {
       tmem_ld32(g0, v);
+    } else if constexpr (BN == 80) {
+      tmem_ld8x5(g0, v);
     } else if (h == 0) {
       tmem_ld32(g0, v);
       tmem_ld16(g0 + 32, u);
@@ -129,8 +150,8 @@ __device__ __forceinline__ void read_groups(uint32_t tcol, int h,
     fence_before();
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(&tempty[grp]);
-    if (BN == 64) {
-      add_group<32>(acc, v, 0, sh);
+    if constexpr (BN == 64 || BN == 80) {
+      add_group<OzShape<BN>::EPI_COLS>(acc, v, 0, sh);
     } else if (h == 0) {
       add_group<32>(acc, v, 0, sh);
       add_group<16>(acc, u, 32, sh);
@@ -147,7 +168,24 @@ __device__ __forceinline__ double pow2(int e) {
   return __longlong_as_double((long long)(e + 1023) << 52);
 }
 
-template <int S, int BN>
+// One output of the split form, C = x 2^(eB[n]) for row m and column n.
+__device__ __forceinline__ void store_one(const OzEpilogue &ep, int atom, int m, int n, double x) {
+  if (ep.mode == kOzC) {
+    ep.C[(int64_t)m * ep.ldc + n] = x;
+  } else if (ep.mode == kOzCT) {
+    ep.C[(int64_t)n * ep.ldc + m] = x;
+  } else if (ep.mode == kOzBetaT) {
+    const int aoA = ep.aoff[atom], nA = ep.aoff[atom + 1] - aoA;
+    const int r = m - aoA * ep.n_occ, E = r / nA, c = r - E * nA;
+    ep.C[((int64_t)n * ep.n_occ + E) * ep.ldc + aoA + c] = x;
+  } else {
+    const int B = ep.orb_atom[m], b = m - ep.aoff[B], jj = n / ep.n_occ, E = n - jj * ep.n_occ;
+    ep.C[(int64_t)jj * ep.ldc + ep.xoff5[B] + (int64_t)b * ep.n_occ + E] = x;
+  }
+}
+
+// SPLIT: the CTAs of a cluster (ksplit of them) share one tile.
+template <int S, int BN, bool SPLIT>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     ozaki_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
                       const __grid_constant__ CUtensorMap mapB, OzArgs a) {
@@ -163,8 +201,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   // that each A panel is read from DRAM about once.  Tiles past the live
   // columns are skipped by every role alike.
   const int Mt = a.Mt, Nt = a.Nt, n_tiles = Mt * Nt;
+  // split form: the CTAs of a cluster share one tile (the launch has a
+  // cluster per tile), CTA `rank` the K chunks [rank c / ks, (rank + 1) c / ks)
+  const int ks = SPLIT ? a.ksplit : 1;
+  const int rank = SPLIT ? (int)(blockIdx.x % ks) : 0;
+  const int tile0 = SPLIT ? (int)(blockIdx.x / ks) : (int)blockIdx.x;
+  const int tstep = SPLIT ? n_tiles : (int)gridDim.x;
   struct Tile {
-    int m0, xoff, nkb, rows_valid, atom, n0;
+    int m0, xoff, kb0, nkb, rows_valid, atom, n0;   // K blocks kb0 .. kb0 + nkb - 1
   };
   auto tile_of = [&](int t, Tile &T) -> bool {
     const int G = a.mgroup;
@@ -186,6 +230,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       T.nkb = a.KpA / OZ_BK;
       T.rows_valid = min(OZ_BM, a.M - T.m0);
       T.atom = -1;
+    }
+    T.kb0 = 0;
+    if constexpr (SPLIT) {
+      const int nch = (T.nkb + a.cb - 1) / a.cb;
+      T.kb0 = rank * nch / ks * a.cb;
+      T.nkb = min(T.nkb, (rank + 1) * nch / ks * a.cb) - T.kb0;
     }
     return true;
   };
@@ -234,7 +284,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       // slice i of K block kb
       int g = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+      for (int t = tile0; t < n_tiles && ok; t += tstep) {
         Tile T;
         if (!tile_of(t, T)) continue;
         for (int kb = 0; kb < T.nkb && ok; ++kb) {
@@ -253,9 +303,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             }
             uint8_t *sa = smem + slot * OZ_STAGE_BYTES;
             mbar_expect_tx(&full[slot], OZ_STAGE_BYTES);
-            tma_load_2d(sa, &mapA, &full[slot], i * a.KpA + kb * OZ_BK, T.m0);
-            tma_load_2d(sa + OZ_A_BYTES, &mapB, &full[slot], i * a.KpB + T.xoff + kb * OZ_BK,
-                        T.n0);
+            const int kx = (T.kb0 + kb) * OZ_BK;
+            tma_load_2d(sa, &mapA, &full[slot], i * a.KpA + kx, T.m0);
+            tma_load_2d(sa + OZ_A_BYTES, &mapB, &full[slot], i * a.KpB + T.xoff + kx, T.n0);
           }
         }
       }
@@ -272,7 +322,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       int g = 0;
       int gc = 0;   // chunks issued by this CTA (over its tiles)
       bool ok = true;
-      for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+      for (int t = tile0; t < n_tiles && ok; t += tstep) {
         Tile T;
         if (!tile_of(t, T)) continue;
         const int nchunks = (T.nkb + cb - 1) / cb;
@@ -351,7 +401,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const int lr = q * 32 + lane;
     const uint32_t tcol = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * OZ_EPI_COLS);
     int gc = 0;   // chunks drained (over this CTA's tiles)
-    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+    for (int t = tile0; t < n_tiles; t += tstep) {
       Tile T;
       if (!tile_of(t, T)) continue;
       const int m = T.m0 + lr;
@@ -372,12 +422,19 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           break;
         }
         fence_after();
-        read_groups<S, BN>(tcol, h, acc, a.ns, tempty);
+        read_groups<S, BN>(tcol, h, acc, a.ns, a.drop, tempty);
       }
       if (!ok) break;
+      if constexpr (SPLIT) {
+        // this CTA's partial sums to its shared memory (the ring is idle: the
+        // last chunk's MMAs, and with them every copy, have completed)
+        long long *part = (long long *)smem;   // [BN][OZ_BM]
+#pragma unroll
+        for (int j = 0; j < OZ_EPI_COLS; ++j) part[(h * OZ_EPI_COLS + j) * OZ_BM + lr] = acc[j];
+      } else
       if (lr < T.rows_valid && nc < N) {
         // C = acc 2^(eA + eB + u - 7(S+1)), as two exact power-of-two factors
-        const double fa = pow2(a.eA[m] + oz_drop_bits(S) - 7 * (S + 1));
+        const double fa = pow2(a.eA[m] + a.drop - 7 * (S + 1));
         const OzEpilogue &ep = a.ep;
         if (ep.mode == kOzC) {
           double *crow = ep.C + (int64_t)m * ep.ldc + nc;
@@ -436,6 +493,28 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols));
   }
+  if constexpr (SPLIT) {
+    // the cluster's integer partial sums added (exact in any order) and
+    // stored, the columns shared out over its CTAs.  Every thread of every
+    // CTA gets here: the roles above end by themselves, after an abort too.
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    Tile T;
+    if (tile0 < n_tiles && tile_of(tile0, T) && !*(volatile int *)&abort_flag) {
+      const int row = threadIdx.x & (OZ_BM - 1);
+      for (int j = rank + ks * (int)(threadIdx.x / OZ_BM); j < BN;
+           j += ks * (OZ_THREADS / OZ_BM)) {
+        const int m = T.m0 + row, n = T.n0 + j;
+        if (threadIdx.x >= OZ_THREADS / OZ_BM * OZ_BM || row >= T.rows_valid || n >= N) continue;
+        long long sum = 0;
+        for (int q = 0; q < ks; ++q)
+          sum += cl.map_shared_rank((const long long *)smem, q)[j * OZ_BM + row];
+        store_one(a.ep, T.atom, m, n,
+                  (double)sum * pow2(a.eA[m] + a.drop - 7 * (S + 1)) * pow2(a.eB[n]));
+      }
+    }
+    cl.sync();   // partial sums stay until every CTA has read them
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -466,86 +545,112 @@ __device__ __forceinline__ long long fixed_point(double x, int e, int s) {
   else F = (M + (1ll << (-sh - 1))) >> (-sh);     // round half up in magnitude
   return b < 0 ? -F : F;
 }
-// bf16 bit pattern of an integer with |q| <= 128 (exact)
-__device__ __forceinline__ unsigned int bf16_bits_small(int q) {
-  if (q == 0) return 0u;
-  const unsigned int sign = q < 0 ? 0x8000u : 0u;
-  const unsigned int a = (unsigned int)(q < 0 ? -q : q);
-  const int p = 31 - __clz(a);                    // 2^p <= a < 2^(p+1), p <= 7
-  return sign | ((unsigned int)(127 + p) << 7) | ((a << (7 - p)) & 0x7Fu);
+// The high half of float32(q) is bf16(q) for |q| <= 128 (8 significant bits at
+// most); q + 1.5 * 2^23 is formed in the integer pipe, the float subtraction
+// is exact.
+__device__ __forceinline__ unsigned int float_bits(int q) {
+  return __float_as_uint(__int_as_float(0x4B400000 + q) - 12582912.0f);
 }
-// slices of two neighbouring entries (x0, x1) of a row with exponent e,
-// stored as bf16 pairs at dst + i*Kp for slice i
-__device__ __forceinline__ void store_slices(double x0, double x1, int e, int s, int Kp,
+// Slices of four neighbouring entries of a row with exponent e, stored as
+// four bf16 at dst + i*Kp for slice i (k a multiple of 4: 8-byte stores).
+// With the offset sum_{t < S-1} 64 128^t added to F, the balanced digit t is
+// the plain base-128 digit minus 64, so the digits are independent 7-bit
+// fields: four of them in the low 28 bits, the others above.
+template <int S>
+__device__ __forceinline__ void store_slices(const double (&x)[4], int e, int Kp,
                                              __nv_bfloat16 *dst) {
-  long long F0 = fixed_point(x0, e, s), F1 = fixed_point(x1, e, s);
-  unsigned int w[kOzMaxSlices];
-  for (int i = s - 1; i >= 1; --i) {
-    const int d0 = (int)(((F0 + 64) & 127) - 64), d1 = (int)(((F1 + 64) & 127) - 64);
-    w[i] = bf16_bits_small(d0) | (bf16_bits_small(d1) << 16);
-    F0 = (F0 - d0) >> 7;
-    F1 = (F1 - d1) >> 7;
+  constexpr long long kOff = [] {
+    long long o = 0;
+    for (int t = 0; t < S - 1; ++t) o = o * 128 + 64;
+    return o;
+  }();
+  int lo[4], hi[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const long long F = fixed_point(x[j], e, S) + kOff;
+    lo[j] = S <= 4 ? (int)F : (int)(F & 0xFFFFFFF);
+    hi[j] = S <= 4 ? 0 : (int)(F >> 28);
   }
-  w[0] = bf16_bits_small((int)F0) | (bf16_bits_small((int)F1) << 16);
-  for (int i = 0; i < s; ++i) *(unsigned int *)(dst + (int64_t)i * Kp) = w[i];
+#pragma unroll
+  for (int i = 0; i < S; ++i) {
+    const int t = S - 1 - i;   // digit of weight 128^t
+    unsigned int f[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int v = t < 4 ? lo[j] >> (7 * (t & 3)) : hi[j] >> (7 * (t & 3));
+      f[j] = float_bits(i == 0 ? v : (v & 127) - 64);
+    }
+    uint2 w;
+    w.x = __byte_perm(f[0], f[1], 0x7632);
+    w.y = __byte_perm(f[2], f[3], 0x7632);
+    *(uint2 *)(dst + (int64_t)i * Kp) = w;
+  }
 }
 
-// Block-wide max of an int (all threads receive it); red holds >= 32 ints.
-__device__ __forceinline__ int block_max_int(int v, int *red) {
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    int t = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0;
-    for (int o = 16; o > 0; o >>= 1) t = max(t, __shfl_xor_sync(0xffffffffu, t, o));
-    if (threadIdx.x == 0) red[0] = t;
-  }
-  __syncthreads();
-  const int r = red[0];
-  __syncthreads();
-  return r;
-}
-
-// Row r of the operand: X[r][k] for k < Kdim, or, with a column map,
-// X[r][cols[k]] (zero where cols[k] < 0).
+// Entry k of row x of the operand: x[k] for k < Kdim, or, with a column map,
+// x[cols[k]] (zero where cols[k] < 0).
 __device__ __forceinline__ double gathered(const double *x, const int *cols, int k, int Kdim) {
   if (k >= Kdim) return 0.0;
   if (!cols) return x[k];
   const int c = cols[k];
   return c >= 0 ? x[c] : 0.0;
 }
+template <int S>
+__device__ __forceinline__ void slice_at(const double *x, const int *cols, int k, int Kdim, int e,
+                                         int Kp, __nv_bfloat16 *qr) {
+  double v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[j] = gathered(x, cols, k + j, Kdim);
+  store_slices<S>(v, e, Kp, qr + k);
+}
 
-__global__ void oz_slice_rows_kernel(int rows, int Kdim, const double *__restrict__ X, int64_t ldx,
-                                     const int *__restrict__ cols, int s, int Kp,
-                                     __nv_bfloat16 *__restrict__ Q, int *__restrict__ E,
-                                     const int *dcnt, int mul) {
-  __shared__ int red[32];
-  int live = rows;
-  if (dcnt) live = min(rows, mul * (*dcnt));
-  for (int r = blockIdx.x; r < live; r += gridDim.x) {
-    const double *x = X + (int64_t)r * ldx;
-    int fm = 0;
-    for (int k = threadIdx.x; k < Kdim; k += blockDim.x) fm = max(fm, exp_field(gathered(x, cols, k, Kdim)));
-    const int e = row_exponent_of_field(block_max_int(fm, red));
-    if (threadIdx.x == 0) E[r] = e;
-    __nv_bfloat16 *qr = Q + (int64_t)r * s * Kp;
-    for (int k = 2 * threadIdx.x; k < Kp; k += 2 * blockDim.x)
-      store_slices(gathered(x, cols, k, Kdim), gathered(x, cols, k + 1, Kdim), e, s, Kp, qr + k);
+// Rows, WPR warps per row (8 rows per CTA, or 1): the exponent of the row's
+// largest entry, then its slices (the second read comes from L1 or L2).
+template <int S, int WPR>
+__global__ void __launch_bounds__(256) oz_slice_rows_kernel(int rows, int Kdim,
+                                                            const double *__restrict__ X,
+                                                            int64_t ldx,
+                                                            const int *__restrict__ cols, int Kp,
+                                                            __nv_bfloat16 *__restrict__ Q,
+                                                            int *__restrict__ E, const int *dcnt,
+                                                            int mul) {
+  __shared__ int red[8];
+  const int live = dcnt ? min(rows, mul * (*dcnt)) : rows;
+  const int warp = threadIdx.x >> 5;
+  const int r = blockIdx.x * (8 / WPR) + warp / WPR;
+  const int t = (warp % WPR) * 32 + (threadIdx.x & 31);
+  const bool on = r < live;
+  const double *x = X + (int64_t)r * ldx;
+  int fm = 0;
+  if (on) {
+#pragma unroll 4
+    for (int k = t; k < Kdim; k += 32 * WPR) fm = max(fm, exp_field(gathered(x, cols, k, Kdim)));
   }
+  for (int o = 16; o > 0; o >>= 1) fm = max(fm, __shfl_xor_sync(0xffffffffu, fm, o));
+  if (WPR > 1) {
+    if ((threadIdx.x & 31) == 0) red[warp] = fm;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < WPR; ++w) fm = max(fm, red[w]);
+  }
+  if (!on) return;
+  const int e = row_exponent_of_field(fm);
+  if (t == 0) E[r] = e;
+  __nv_bfloat16 *qr = Q + (int64_t)r * S * Kp;
+  for (int k = 4 * t; k < Kp; k += 128 * WPR) slice_at<S>(x, cols, k, Kdim, e, Kp, qr);
 }
 
 // Long rows: grid (chunks, rows).  Pass 1 raises E[r] (preset to a large
 // negative value) to the exponent of each chunk's largest entry; pass 2
 // slices every chunk with the row's exponent (a row of zeros keeps the preset
 // value and gives zero slices).
-constexpr int OZ_CHUNK = 4096;
+constexpr int OZ_CHUNK = 2048;
 
 __global__ void __launch_bounds__(256) oz_rowmax_kernel(int rows, int Kdim,
                                                         const double *__restrict__ X, int64_t ldx,
                                                         const int *__restrict__ cols,
                                                         int *__restrict__ E, const int *dcnt,
                                                         int mul) {
-  __shared__ int red[32];
   int live = rows;
   if (dcnt) live = min(rows, mul * (*dcnt));
   const int r = blockIdx.y;
@@ -553,39 +658,64 @@ __global__ void __launch_bounds__(256) oz_rowmax_kernel(int rows, int Kdim,
   const double *x = X + (int64_t)r * ldx;
   const int k0 = blockIdx.x * OZ_CHUNK, k1 = min(Kdim, k0 + OZ_CHUNK);
   int fm = 0;
+#pragma unroll 4
   for (int k = k0 + threadIdx.x; k < k1; k += 256) fm = max(fm, exp_field(gathered(x, cols, k, Kdim)));
-  fm = block_max_int(fm, red);
-  if (threadIdx.x == 0 && fm > 0) atomicMax(E + r, row_exponent_of_field(fm));
+  for (int o = 16; o > 0; o >>= 1) fm = max(fm, __shfl_xor_sync(0xffffffffu, fm, o));
+  if ((threadIdx.x & 31) == 0 && fm > 0) atomicMax(E + r, row_exponent_of_field(fm));
 }
 
+template <int S>
 __global__ void __launch_bounds__(256) oz_slice_chunks_kernel(int rows, int Kdim,
                                                               const double *__restrict__ X,
                                                               int64_t ldx,
-                                                              const int *__restrict__ cols, int s,
-                                                              int Kp, __nv_bfloat16 *__restrict__ Q,
+                                                              const int *__restrict__ cols, int Kp,
+                                                              __nv_bfloat16 *__restrict__ Q,
                                                               const int *__restrict__ E,
                                                               const int *dcnt, int mul) {
   int live = rows;
   if (dcnt) live = min(rows, mul * (*dcnt));
   const int r = blockIdx.y;
   if (r >= live) return;
-  const double *x = X + (int64_t)r * ldx;
   const int e = E[r];   // a row of zeros: every entry gives F = 0 whatever e is
-  __nv_bfloat16 *qr = Q + (int64_t)r * s * Kp;
   const int k0 = blockIdx.x * OZ_CHUNK, k1 = min(Kp, k0 + OZ_CHUNK);
-  for (int k = k0 + 2 * threadIdx.x; k < k1; k += 512)
-    store_slices(gathered(x, cols, k, Kdim), gathered(x, cols, k + 1, Kdim), e, s, Kp, qr + k);
+  for (int k = k0 + 4 * threadIdx.x; k < k1; k += 1024)
+    slice_at<S>(X + (int64_t)r * ldx, cols, k, Kdim, e, Kp, Q + (int64_t)r * S * Kp);
 }
 
-// 32 columns per CTA (256 threads): column exponents, then 64-row tiles staged
-// through shared memory and written as rows of the transposed operand.
+// Columns of a row-major matrix, 32 per CTA: one 64-row tile staged through
+// shared memory and written as rows of the transposed operand.
+template <int S>
+__device__ __forceinline__ void slice_col_tile(int Kdim, int live, const double *X, int64_t ldx,
+                                               int Kp, __nv_bfloat16 *Q, int n0, int k0,
+                                               const int *ecol, double (*tile)[66]) {
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, n = n0 + tx;
+#pragma unroll
+  for (int rr = ty; rr < 64; rr += 8) {
+    const int k = k0 + rr;
+    tile[tx][rr] = (k < Kdim && n < live) ? X[(int64_t)k * ldx + n] : 0.0;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int col = 16 * h + (threadIdx.x >> 4), k4 = 4 * (threadIdx.x & 15);
+    if (n0 + col < live) {
+      const double2 a = *(const double2 *)&tile[col][k4], b = *(const double2 *)&tile[col][k4 + 2];
+      const double v[4] = {a.x, a.y, b.x, b.y};
+      store_slices<S>(v, ecol[col], Kp, Q + (int64_t)(n0 + col) * S * Kp + k0 + k4);
+    }
+  }
+  __syncthreads();
+}
+
+// Short columns: exponents and slices in one launch (grid: column groups).
+template <int S>
 __global__ void __launch_bounds__(256) oz_slice_cols_kernel(int Kdim, int N,
                                                             const double *__restrict__ X,
-                                                            int64_t ldx, int s, int Kp,
+                                                            int64_t ldx, int Kp,
                                                             __nv_bfloat16 *__restrict__ Q,
                                                             int *__restrict__ E, const int *dcnt,
                                                             int mul) {
-  __shared__ double tile[32][65];
+  __shared__ __align__(16) double tile[32][66];
   __shared__ int red[8][32];
   __shared__ int ecol[32];
   int live = N;
@@ -595,8 +725,10 @@ __global__ void __launch_bounds__(256) oz_slice_cols_kernel(int Kdim, int N,
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int n = n0 + tx;
   int fm = 0;
-  if (n < live)
+  if (n < live) {
+#pragma unroll 8
     for (int k = ty; k < Kdim; k += 8) fm = max(fm, exp_field(X[(int64_t)k * ldx + n]));
+  }
   red[ty][tx] = fm;
   __syncthreads();
   if (ty == 0) {
@@ -607,39 +739,154 @@ __global__ void __launch_bounds__(256) oz_slice_cols_kernel(int Kdim, int N,
     ecol[tx] = e;
   }
   __syncthreads();
-  for (int k0 = 0; k0 < Kp; k0 += 64) {
-    for (int rr = ty; rr < 64; rr += 8) {
-      const int k = k0 + rr;
-      tile[tx][rr] = (k < Kdim && n < live) ? X[(int64_t)k * ldx + n] : 0.0;
-    }
-    __syncthreads();
-    for (int cc = 0; cc < 4; ++cc) {
-      const int col = ty * 4 + cc;
-      if (n0 + col < live)
-        store_slices(tile[col][2 * tx], tile[col][2 * tx + 1], ecol[col], s, Kp,
-                     Q + (int64_t)(n0 + col) * s * Kp + k0 + 2 * tx);
-    }
-    __syncthreads();
+  for (int k0 = 0; k0 < Kp; k0 += 64)
+    slice_col_tile<S>(Kdim, live, X, ldx, Kp, Q, n0, k0, ecol, tile);
+}
+
+// Long columns: the same in two passes over a grid (column groups, K chunks),
+// the exponents by atomic maximum into a preset E as for long rows.
+constexpr int OZ_CCHUNK = 256;
+
+__global__ void __launch_bounds__(256) oz_colmax_kernel(int Kdim, int N,
+                                                        const double *__restrict__ X, int64_t ldx,
+                                                        int *__restrict__ E, const int *dcnt,
+                                                        int mul) {
+  __shared__ int red[8][32];
+  int live = N;
+  if (dcnt) live = (int)min((int64_t)N, (int64_t)mul * (*dcnt));
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, n = blockIdx.x * 32 + tx;
+  if (blockIdx.x * 32 >= live) return;
+  const int k0 = blockIdx.y * OZ_CCHUNK, k1 = min(Kdim, k0 + OZ_CCHUNK);
+  int fm = 0;
+  if (n < live) {
+#pragma unroll 8
+    for (int k = k0 + ty; k < k1; k += 8) fm = max(fm, exp_field(X[(int64_t)k * ldx + n]));
+  }
+  red[ty][tx] = fm;
+  __syncthreads();
+  if (ty == 0 && n < live) {
+    int v = 0;
+    for (int i = 0; i < 8; ++i) v = max(v, red[i][tx]);
+    if (v > 0) atomicMax(E + n, row_exponent_of_field(v));
+  }
+}
+
+template <int S>
+__global__ void __launch_bounds__(256) oz_slice_col_chunks_kernel(
+    int Kdim, int N, const double *__restrict__ X, int64_t ldx, int Kp,
+    __nv_bfloat16 *__restrict__ Q, const int *__restrict__ E, const int *dcnt, int mul) {
+  __shared__ __align__(16) double tile[32][66];
+  __shared__ int ecol[32];
+  int live = N;
+  if (dcnt) live = (int)min((int64_t)N, (int64_t)mul * (*dcnt));
+  const int n0 = blockIdx.x * 32;
+  if (n0 >= live) return;
+  if (threadIdx.x < 32) ecol[threadIdx.x] = n0 + threadIdx.x < live ? E[n0 + threadIdx.x] : 0;
+  const int k1 = min(Kp, (int)(blockIdx.y + 1) * OZ_CCHUNK);
+  for (int k0 = blockIdx.y * OZ_CCHUNK; k0 < k1; k0 += 64)   // (the tile's barrier covers ecol)
+    slice_col_tile<S>(Kdim, live, X, ldx, Kp, Q, n0, k0, ecol, tile);
+}
+
+// f(integral_constant<S>) for the slice count s of an operand
+template <class F>
+cudaError_t with_slices(int s, F &&f) {
+  switch (s) {
+    case 3: return f(std::integral_constant<int, 3>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    case 5: return f(std::integral_constant<int, 5>{});
+    case 6: return f(std::integral_constant<int, 6>{});
+    case 7: return f(std::integral_constant<int, 7>{});
+    case 8: return f(std::integral_constant<int, 8>{});
+    default: return cudaErrorInvalidValue;
   }
 }
 
 int chunk_blocks(int s) { return std::max(1, 4096 / (s + 2) / OZ_BK); }
 
-template <int S>
-cudaError_t launch_oz_kernel(cudaStream_t st, dim3 grid, const CUtensorMap &mA,
-                             const OzOperand &B, const OzArgs &a) {
-  constexpr int BN = oz_bn(S);
-  ozaki_gemm_kernel<S, BN><<<grid, OZ_THREADS, OzShape<BN>::SMEM, st>>>(
-      mA, BN == 64 ? B.map : B.map96, a);
-  return cudaGetLastError();
+template <int S, int BN>
+cudaError_t launch_oz_kernel(cudaStream_t st, int ctas, const CUtensorMap &mA,
+                             const CUtensorMap &mB, const OzArgs &a) {
+  if (a.ksplit <= 1) {
+    ozaki_gemm_kernel<S, BN, false><<<ctas, OZ_THREADS, OzShape<BN>::SMEM, st>>>(mA, mB, a);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(OZ_THREADS);
+  cfg.dynamicSmemBytes = OzShape<BN>::SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = a.ksplit;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, ozaki_gemm_kernel<S, BN, true>, mA, mB, a);
 }
 
-template <int S>
+template <int S, int BN>
 cudaError_t set_smem_attr() {
-  constexpr int BN = oz_bn(S);
-  return cudaFuncSetAttribute(ozaki_gemm_kernel<S, BN>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)OzShape<BN>::SMEM);
+  constexpr int bytes = (int)OzShape<BN>::SMEM;
+  const cudaError_t e = cudaFuncSetAttribute(ozaki_gemm_kernel<S, BN, false>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(ozaki_gemm_kernel<S, BN, true>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
+// Clusters of c CTAs (one CTA per SM) that run at once.  GPCs hold 16 to 20
+// SMs, so 152 SMs take 76 clusters of 2, 36 of 4, 23 of 6, but 15 of 7 or 8.
+int active_clusters(int c) {
+  static int fit[9] = {};
+  if (fit[c] == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c * 256);
+    cfg.blockDim = dim3(OZ_THREADS);
+    cfg.dynamicSmemBytes = OzShape<64>::SMEM;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = c;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, ozaki_gemm_kernel<6, 64, true>, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    fit[c] = n > 0 ? n : -1;
+  }
+  return fit[c];
+}
+
+// N tile and K split of a product of Mt row tiles, N columns and nch K chunks:
+// the least of waves x chunks per CTA x clocks per MMA (measured: 55 at N =
+// 64, 65 at 80, 66 at 96, the reads of the A tile among them), with half a
+// chunk for the sum over a cluster and a third for a tile's start.  Exact
+// integer sums: every plan gives the same bits.
+// (1000 x 129 x 9080, 6 slices: 24 CTAs 455 us -> 16 clusters of 6, 101 us.)
+struct TilePlan {
+  int bn, ks;
+};
+TilePlan tile_plan(int S, int Mt, int N, int nch) {
+  TilePlan best{64, 1};
+  double least = 1e300;
+  for (int bn : {64, oz_wide_bn(S)}) {
+    const double tiles = (double)Mt * ((N + bn - 1) / bn);
+    for (int ks = 1; ks <= std::min(8, nch); ++ks) {
+      const int fit = active_clusters(ks);
+      if (fit < 1) continue;
+      const double cost = std::ceil(tiles / fit) * ((nch + ks - 1) / ks + (ks > 1 ? 0.83 : 0.33)) *
+                          (bn == 64 ? 55.0 : (bn == 80 ? 65.0 : 66.0));
+      if (cost < least) {
+        least = cost;
+        best = TilePlan{bn, ks};
+      }
+    }
+  }
+  return best;
 }
 }  // namespace
 
@@ -648,12 +895,13 @@ cudaError_t set_smem_attr() {
 cudaError_t oz_init_attributes() {
   static cudaError_t done = cudaErrorNotReady;
   if (done == cudaSuccess) return done;
-  cudaError_t e = set_smem_attr<3>();
-  if (e == cudaSuccess) e = set_smem_attr<4>();
-  if (e == cudaSuccess) e = set_smem_attr<5>();
-  if (e == cudaSuccess) e = set_smem_attr<6>();
-  if (e == cudaSuccess) e = set_smem_attr<7>();
-  if (e == cudaSuccess) e = set_smem_attr<8>();
+  cudaError_t e = cudaSuccess;
+  for (int n = kOzMinSlices; n <= kOzMaxSlices && e == cudaSuccess; ++n)
+    e = with_slices(n, [](auto sc) {
+      constexpr int S = decltype(sc)::value, W = oz_wide_bn(S);
+      const cudaError_t r = set_smem_attr<S, 64>();
+      return W == 64 || r != cudaSuccess ? r : set_smem_attr<S, W>();
+    });
   done = e;
   return e;
 }
@@ -666,43 +914,61 @@ cudaError_t oz_operand(OzOperand &op, __nv_bfloat16 *q, int *e, int64_t rows, in
   op.rows = rows;
   op.Kp = round_up(Kdim, OZ_BK);
   op.s = s;
-  cudaError_t r = encode_bf16_map(&op.map, q, rows, (int64_t)s * op.Kp, box_rows);
-  // the B role also gets 96-row boxes (the N tile of 3 to 5 slices)
-  op.has96 = false;
-  if (r == cudaSuccess && box_rows == OZ_BN) {
-    r = encode_bf16_map(&op.map96, q, rows, (int64_t)s * op.Kp, 96);
-    op.has96 = r == cudaSuccess;
-  }
-  return r;
+  const cudaError_t r = encode_bf16_map(&op.map, q, rows, (int64_t)s * op.Kp, box_rows);
+  // the B role (box_rows OZ_BN) also takes boxes of the wide N tile
+  if (r != cudaSuccess || box_rows != OZ_BN) return r;
+  return encode_bf16_map(&op.map_wide, q, rows, (int64_t)s * op.Kp, oz_wide_bn(s));
 }
+
+// Rows up to this length take one warp each, then one CTA; from OZ_LONG_ROW on
+// (and for columns from OZ_LONG_COL on) chunks go to separate CTAs, with the
+// exponent by atomic maximum in a pass of its own.
+constexpr int OZ_WARP_ROW = 2048, OZ_LONG_ROW = 8192, OZ_LONG_COL = 512;
 
 cudaError_t launch_oz_slice_rows(cudaStream_t st, const double *X, int64_t ldx, int rows, int Kdim,
                                  OzOperand &op, const int *dcnt, int mul, const int *cols) {
   if (rows <= 0) return cudaSuccess;
   if (rows > op.rows || Kdim > op.Kp) return cudaErrorInvalidValue;
-  if (op.Kp >= 2 * OZ_CHUNK && rows <= 65535) {
-    // long rows: chunks of a row on separate CTAs (exponent by atomic max)
-    cudaError_t e = cudaMemsetAsync(op.e, 0x80, (size_t)rows * sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    dim3 g1((Kdim + OZ_CHUNK - 1) / OZ_CHUNK, rows), g2((op.Kp + OZ_CHUNK - 1) / OZ_CHUNK, rows);
-    oz_rowmax_kernel<<<g1, 256, 0, st>>>(rows, Kdim, X, ldx, cols, op.e, dcnt, mul);
-    oz_slice_chunks_kernel<<<g2, 256, 0, st>>>(rows, Kdim, X, ldx, cols, op.s, op.Kp, op.q, op.e,
-                                               dcnt, mul);
+  return with_slices(op.s, [&](auto sc) {
+    constexpr int S = decltype(sc)::value;
+    if (op.Kp >= OZ_LONG_ROW && rows <= 65535) {
+      cudaError_t e = cudaMemsetAsync(op.e, 0x80, (size_t)rows * sizeof(int), st);
+      if (e != cudaSuccess) return e;
+      dim3 g1((Kdim + OZ_CHUNK - 1) / OZ_CHUNK, rows), g2((op.Kp + OZ_CHUNK - 1) / OZ_CHUNK, rows);
+      oz_rowmax_kernel<<<g1, 256, 0, st>>>(rows, Kdim, X, ldx, cols, op.e, dcnt, mul);
+      oz_slice_chunks_kernel<S><<<g2, 256, 0, st>>>(rows, Kdim, X, ldx, cols, op.Kp, op.q, op.e,
+                                                    dcnt, mul);
+    } else if (op.Kp <= OZ_WARP_ROW) {
+      oz_slice_rows_kernel<S, 1><<<(rows + 7) / 8, 256, 0, st>>>(rows, Kdim, X, ldx, cols, op.Kp,
+                                                                 op.q, op.e, dcnt, mul);
+    } else {
+      oz_slice_rows_kernel<S, 8><<<rows, 256, 0, st>>>(rows, Kdim, X, ldx, cols, op.Kp, op.q, op.e,
+                                                       dcnt, mul);
+    }
     return cudaGetLastError();
-  }
-  const int grid = std::min(rows, 152 * 8);
-  oz_slice_rows_kernel<<<grid, 256, 0, st>>>(rows, Kdim, X, ldx, cols, op.s, op.Kp, op.q, op.e,
-                                             dcnt, mul);
-  return cudaGetLastError();
+  });
 }
 
 cudaError_t launch_oz_slice_cols(cudaStream_t st, const double *X, int64_t ldx, int Kdim, int N,
                                  OzOperand &op, const int *dcnt, int mul) {
   if (N <= 0) return cudaSuccess;
   if (N > op.rows || Kdim > op.Kp) return cudaErrorInvalidValue;
-  oz_slice_cols_kernel<<<(N + 31) / 32, 256, 0, st>>>(Kdim, N, X, ldx, op.s, op.Kp, op.q, op.e,
-                                                      dcnt, mul);
-  return cudaGetLastError();
+  return with_slices(op.s, [&](auto sc) {
+    constexpr int S = decltype(sc)::value;
+    const int chunks = (op.Kp + OZ_CCHUNK - 1) / OZ_CCHUNK;
+    if (op.Kp >= OZ_LONG_COL && chunks <= 65535) {
+      cudaError_t e = cudaMemsetAsync(op.e, 0x80, (size_t)N * sizeof(int), st);
+      if (e != cudaSuccess) return e;
+      const dim3 grid((N + 31) / 32, chunks);
+      oz_colmax_kernel<<<grid, 256, 0, st>>>(Kdim, N, X, ldx, op.e, dcnt, mul);
+      oz_slice_col_chunks_kernel<S><<<grid, 256, 0, st>>>(Kdim, N, X, ldx, op.Kp, op.q, op.e, dcnt,
+                                                          mul);
+    } else {
+      oz_slice_cols_kernel<S><<<(N + 31) / 32, 256, 0, st>>>(Kdim, N, X, ldx, op.Kp, op.q, op.e,
+                                                             dcnt, mul);
+    }
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t launch_gemm_oz_ex(cudaStream_t st, const OzOperand &A, const OzOperand &B, int M,
@@ -737,30 +1003,22 @@ cudaError_t launch_gemm_oz_ex(cudaStream_t st, const OzOperand &A, const OzOpera
   a.err = err;
   a.dcnt = dcnt;
   a.mul_n = mul_n;
-  const int bn = oz_bn(A.s);
-  if (bn == 96 && !B.has96) return cudaErrorInvalidValue;
-  // persistent grid: one CTA per SM at most, each walking its share of the tiles
   a.Mt = tiles ? n_tiles : (M + OZ_BM - 1) / OZ_BM;
-  a.Nt = (N + bn - 1) / bn;
-  if ((int64_t)a.Mt * a.Nt > INT32_MAX) return cudaErrorInvalidConfiguration;
-  static int n_sm = 0;
-  if (n_sm == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        n_sm < 1)
-      n_sm = 1;
-  }
-  dim3 grid((unsigned)std::min<int64_t>((int64_t)a.Mt * a.Nt, n_sm));
-  switch (A.s) {
-    case 3: return launch_oz_kernel<3>(st, grid, A.map, B, a);
-    case 4: return launch_oz_kernel<4>(st, grid, A.map, B, a);
-    case 5: return launch_oz_kernel<5>(st, grid, A.map, B, a);
-    case 6: return launch_oz_kernel<6>(st, grid, A.map, B, a);
-    case 7: return launch_oz_kernel<7>(st, grid, A.map, B, a);
-    case 8: return launch_oz_kernel<8>(st, grid, A.map, B, a);
-    default: return cudaErrorInvalidValue;
-  }
+  const int nch = (nkb + a.cb - 1) / a.cb;
+  a.drop = drop_bits(A.s, nch);
+  const TilePlan plan = tile_plan(A.s, a.Mt, N, nch);
+  a.Nt = (N + plan.bn - 1) / plan.bn;
+  a.ksplit = plan.ks;
+  const int64_t all = (int64_t)a.Mt * a.Nt;
+  if (all * plan.ks > INT32_MAX) return cudaErrorInvalidConfiguration;
+  // unsplit: a persistent grid, one CTA per SM at most, each walking its share
+  // of the tiles; split: one cluster per tile
+  const int ctas = (int)(plan.ks > 1 ? all * plan.ks : std::min<int64_t>(all, active_clusters(1)));
+  return with_slices(A.s, [&](auto sc) {
+    constexpr int S = decltype(sc)::value, W = oz_wide_bn(S);
+    if (plan.bn == 64) return launch_oz_kernel<S, 64>(st, ctas, A.map, B.map, a);
+    return launch_oz_kernel<S, W>(st, ctas, A.map, B.map_wide, a);
+  });
 }
 
 cudaError_t launch_gemm_oz(cudaStream_t st, const OzOperand &A, const OzOperand &B, int M, int N,
@@ -834,29 +1092,32 @@ extern "C" tddft_status tddft_gemm_f64_emulated(int32_t M, int32_t N, int32_t K,
   if (lda < K || ldb < N || ldc < N) return TDDFT_ERR_SHAPE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int Kp = round_up(K, OZ_BK);
-  std::vector<void *> allocs;
-  auto alloc = [&](size_t bytes, void **p) -> cudaError_t {
-    cudaError_t e = cudaMalloc(p, bytes + 16);
-    if (e == cudaSuccess) allocs.push_back(*p);
-    return e;
-  };
-  void *qa = nullptr, *qb = nullptr, *ea = nullptr, *eb = nullptr, *err = nullptr;
-  cudaError_t e = alloc((size_t)M * slices * Kp * sizeof(__nv_bfloat16), &qa);
-  if (e == cudaSuccess) e = alloc((size_t)N * slices * Kp * sizeof(__nv_bfloat16), &qb);
-  if (e == cudaSuccess) e = alloc((size_t)M * sizeof(int), &ea);
-  if (e == cudaSuccess) e = alloc((size_t)N * sizeof(int), &eb);
-  if (e == cudaSuccess) e = alloc(ptx::kErrInts * sizeof(int), &err);
+  // one scratch block: error ints, exponents, the two sliced operands
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  const size_t n_err = up(ptx::kErrInts * sizeof(int)), n_e = up(((size_t)M + N) * sizeof(int)),
+               n_qa = up((size_t)M * slices * Kp * sizeof(__nv_bfloat16)),
+               n_qb = up((size_t)N * slices * Kp * sizeof(__nv_bfloat16));
+  char *ws = nullptr;
+  cudaError_t e = scratch_alloc((void **)&ws, n_err + n_e + n_qa + n_qb, st);
+  if (e != cudaSuccess) {
+    cudaGetLastError();   // not left for a later check
+    return e == cudaErrorMemoryAllocation ? TDDFT_ERR_NOMEM : TDDFT_ERR_CUDA;
+  }
+  int *err = (int *)ws, *ea = (int *)(ws + n_err), *eb = ea + M;
+  __nv_bfloat16 *qa = (__nv_bfloat16 *)(ws + n_err + n_e),
+                *qb = (__nv_bfloat16 *)(ws + n_err + n_e + n_qa);
   OzOperand oa, ob;
-  if (e == cudaSuccess) e = oz_operand(oa, (__nv_bfloat16 *)qa, (int *)ea, M, K, slices, OZ_BM);
-  if (e == cudaSuccess) e = oz_operand(ob, (__nv_bfloat16 *)qb, (int *)eb, N, K, slices, OZ_BN);
+  e = oz_operand(oa, qa, ea, M, K, slices, OZ_BM);
+  if (e == cudaSuccess) e = oz_operand(ob, qb, eb, N, K, slices, OZ_BN);
   if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, ptx::kErrInts * sizeof(int), st);
   if (e == cudaSuccess) e = launch_oz_slice_rows(st, A, lda, M, K, oa);
   if (e == cudaSuccess) e = launch_oz_slice_cols(st, B, ldb, K, N, ob);
-  if (e == cudaSuccess) e = launch_gemm_oz(st, oa, ob, M, N, C, ldc, 0, (int *)err);
+  if (e == cudaSuccess) e = launch_gemm_oz(st, oa, ob, M, N, C, ldc, 0, err);
   int herr = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
+  const cudaError_t ef = cudaFreeAsync(ws, st);
+  if (e == cudaSuccess) e = ef;
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  for (void *p : allocs) cudaFree(p);
   if (e == cudaErrorMemoryAllocation) return TDDFT_ERR_NOMEM;
   if (e != cudaSuccess) return TDDFT_ERR_CUDA;
   return herr ? TDDFT_ERR_TIMEOUT : TDDFT_OK;

@@ -544,6 +544,7 @@ void tddft_destroy(tddft_ctx *c) {
   cudaStreamSynchronize(c->st);
   release(c);
   delete c;
+  scratch_trim();
 }
 
 const char *tddft_last_error(const tddft_ctx *c) {
