@@ -452,34 +452,36 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      // MMA issuer
-      const uint32_t idesc = TF ? idesc_tf32(TC_BM, tn) : idesc_bf16(TC_BM, tn);
-      const uint32_t base = smem_u32(smem);
-      int g = 0, lt = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++lt) {
-        int m0, xa, xoff, nkb, rv, at, n0;
-        tile_of(t, m0, xa, xoff, nkb, rv, at, n0);
-        const int buf = lt & 1, use = lt >> 1;
-        if (use > 0) {
-          // the epilogue has drained this buffer's previous tile
-          if (!mbar_wait(&tempty[buf], (uint32_t)(use - 1) & 1u, lim)) {
-            atomicExch(err, 2);
-            abort_flag = 1;
-            ok = false;
-            break;
-          }
-          fence_after();
+    // MMA issuer: the whole warp runs the loop, the elected lane issues
+    const uint32_t leader = elect_one();
+    const uint32_t idesc = TF ? idesc_tf32(TC_BM, tn) : idesc_bf16(TC_BM, tn);
+    const uint32_t lo0 = desc_lo(smem_u32(smem));
+    int slot = 0;          // ring slot and phase of the next stage
+    uint32_t phase = 0;
+    int lt = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++lt) {
+      int m0, xa, xoff, nkb, rv, at, n0;
+      tile_of(t, m0, xa, xoff, nkb, rv, at, n0);
+      const int buf = lt & 1, use = lt >> 1;
+      if (use > 0) {
+        // the epilogue has drained this buffer's previous tile
+        if (!warp_wait(&tempty[buf], (uint32_t)(use - 1) & 1u, lim)) {
+          if (lane == 0) atomicExch(err, 2);
+          abort_flag = 1;
+          ok = false;
+          break;
         }
-        const uint32_t d0 = tmem + (uint32_t)(buf * ACC);
-        // M2: the second M block (accumulator d + TC_BN) only where the
-        // table entry has rows there
-        const int nblk = (kM2 && rv > TC_BM) ? 2 : 1;
-        // step 2: one K loop per part, into the part's own columns
-        // (c16 start x 16, N = 16 x its orbitals) with its own descriptor
-        const int nparts = kPart ? nkb : 1;
-        for (int p = 0; p < nparts && ok; ++p) {
+        fence_after();
+      }
+      const uint32_t d0 = tmem + (uint32_t)(buf * ACC);
+      // M2: the second M block (accumulator d + TC_BN) only where the
+      // table entry has rows there
+      const int nblk = (kM2 && rv > TC_BM) ? 2 : 1;
+      // step 2: one K loop per part, into the part's own columns
+      // (c16 start x 16, N = 16 x its orbitals) with its own descriptor
+      const int nparts = kPart ? nkb : 1;
+      for (int p = 0; p < nparts && ok; ++p) {
         int pnkb = nkb;
         uint32_t pidesc = idesc, d = d0;
         if (kPart) {
@@ -489,19 +491,22 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           d = d0 + (uint32_t)((pi.x & 255) * 16);
           pidesc = TF ? idesc_tf32(TC_BM, ncol) : idesc_bf16(TC_BM, ncol);
         }
-        for (int kb = 0; kb < pnkb; ++kb, ++g) {
-          const int s = g % NS;
-          if (!mbar_wait(&full[s], (uint32_t)(g / NS) & 1u, lim)) {
-            atomicExch(err, 2);
+        for (int kb = 0; kb < pnkb; ++kb) {
+          if (!warp_wait(&full[slot], phase, lim)) {
+            if (lane == 0) atomicExch(err, 2);
             abort_flag = 1;
             ok = false;
             break;
           }
           fence_after();
-          const uint32_t bhi = base + (uint32_t)s * SB + B_OFF, blo = bhi + B_BYTES;
-          for (int blk = 0; blk < nblk; ++blk) {
-            const uint32_t ahi = base + (uint32_t)s * SB + (uint32_t)blk * 2 * TC_A_BYTES,
-                           alo = ahi + TC_A_BYTES;
+          const uint32_t st = lo0 + (uint32_t)slot * (SB >> 4);
+          const uint32_t bhi = st + (B_OFF >> 4), blo = bhi + (B_BYTES >> 4);
+          const uint32_t more = kb > 0 ? 1u : 0u;
+#pragma unroll
+          for (int blk = 0; blk < (kM2 ? 2 : 1); ++blk) {
+            if (blk >= nblk) continue;
+            const uint32_t ahi = st + (uint32_t)blk * 2 * (TC_A_BYTES >> 4),
+                           alo = ahi + (TC_A_BYTES >> 4);
             const uint32_t db = d + (uint32_t)(blk * TC_BN);
             if (TF) {
 #pragma unroll
@@ -509,29 +514,32 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 const uint32_t a0 = h ? alo : ahi, b0 = h ? blo : bhi;
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                  mma_tf32(db, desc_sw128(a0 + 32 * k), desc_sw128(b0 + 32 * k), pidesc,
-                           (kb > 0 || h > 0 || k > 0) ? 1u : 0u);
+                  mma_tf32_if(leader, db, desc_of(a0 + 2 * k), desc_of(b0 + 2 * k), pidesc,
+                              (h > 0 || k > 0) ? 1u : more);
               }
             } else {
 #pragma unroll
               for (int k = 0; k < TC_BK / 16; ++k) {
-                mma_bf16(db, desc_sw128(ahi + 32 * k), desc_sw128(bhi + 32 * k), pidesc,
-                         (kb > 0 || k > 0) ? 1u : 0u);
-                mma_bf16(db, desc_sw128(ahi + 32 * k), desc_sw128(blo + 32 * k), pidesc, 1u);
-                mma_bf16(db, desc_sw128(alo + 32 * k), desc_sw128(bhi + 32 * k), pidesc, 1u);
+                mma_bf16_if(leader, db, desc_of(ahi + 2 * k), desc_of(bhi + 2 * k), pidesc,
+                            k > 0 ? 1u : more);
+                mma_bf16_if(leader, db, desc_of(ahi + 2 * k), desc_of(blo + 2 * k), pidesc, 1u);
+                mma_bf16_if(leader, db, desc_of(alo + 2 * k), desc_of(bhi + 2 * k), pidesc, 1u);
               }
             }
           }
-          mma_commit(&empty[s]);
+          mma_commit_if(leader, &empty[slot]);
+          if (++slot == NS) {
+            slot = 0;
+            phase ^= 1u;
+          }
         }
-        }
-        if (ok) mma_commit(&tfull[buf]);
       }
-      // every MMA issued here (also after an abort) completes before the
-      // tensor memory is freed
-      mma_commit(drain);
-      mbar_wait(drain, 0u);
+      if (ok) mma_commit_if(leader, &tfull[buf]);
     }
+    // every MMA issued here (also after an abort) completes before the
+    // tensor memory is freed
+    mma_commit_if(leader, drain);
+    mbar_wait(drain, 0u);
     __syncwarp();
   } else {
     // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (rows of the tile)

@@ -316,83 +316,93 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16(OZ_BM, BN);
-      const uint32_t base = smem_u32(smem);
-      int g = 0;
-      int gc = 0;   // chunks issued by this CTA (over its tiles)
-      bool ok = true;
-      for (int t = tile0; t < n_tiles && ok; t += tstep) {
-        Tile T;
-        if (!tile_of(t, T)) continue;
-        const int nchunks = (T.nkb + cb - 1) / cb;
-        for (int c = 0; c < nchunks && ok; ++c, ++gc) {
-          const int kb1 = min(T.nkb, (c + 1) * cb);
-          for (int kb = c * cb; kb < kb1 && ok; ++kb) {
-            const bool first_kb = kb == c * cb;
-            // slice pairs (i, j), i >= j, i + j <= S - 1, in the order i, then
-            // j; the unrolled schedule is fixed by S.  (i, j) is the first
-            // pair of its group (i + j) in that order exactly when i - j <= 1.
+    // the whole warp runs the schedule; the elected lane issues
+    constexpr uint32_t idesc = idesc_bf16(OZ_BM, BN);
+    const uint32_t leader = elect_one();
+    const uint32_t lo0 = desc_lo(smem_u32(smem));
+    int slot0 = 0;        // ring slot and phase of the K block's slice 0
+    uint32_t phase0 = 0;
+    int gc = 0;   // chunks issued by this CTA (over its tiles)
+    bool ok = true;
+    for (int t = tile0; t < n_tiles && ok; t += tstep) {
+      Tile T;
+      if (!tile_of(t, T)) continue;
+      const int nchunks = (T.nkb + cb - 1) / cb;
+      for (int c = 0; c < nchunks && ok; ++c, ++gc) {
+        const int kb1 = min(T.nkb, (c + 1) * cb);
+        for (int kb = c * cb; kb < kb1 && ok; ++kb) {
+          const bool first_kb = kb == c * cb;
+          // slot of slice i, and the descriptor words of its A and B tiles
+          auto slot_of = [&](int i) {
+            return slot0 + i >= OZ_STAGES ? slot0 + i - OZ_STAGES : slot0 + i;
+          };
+          auto lo_of = [&](int i) { return lo0 + (uint32_t)slot_of(i) * (OZ_STAGE_BYTES >> 4); };
+          constexpr uint32_t kB = OZ_A_BYTES >> 4;
+          // slice pairs (i, j), i >= j, i + j <= S - 1, in the order i, then
+          // j; the unrolled schedule is fixed by S.  (i, j) is the first
+          // pair of its group (i + j) in that order exactly when i - j <= 1.
 #pragma unroll
-            for (int i = 0; i < S; ++i) {
-              const int gi = g + i;
-              if (!mbar_wait(&full[gi % OZ_STAGES], (uint32_t)(gi / OZ_STAGES) & 1u, lim)) {
-                atomicExch(a.err, 23);
-                abort_flag = 1;
-                ok = false;
-                break;
-              }
-              // each group of the previous chunk (of this tile or the one
-              // before) drained by the epilogue, which drains them in order,
-              // before its first MMA of this chunk: the groups first used at
-              // step i are 2i - 1 and 2i, so the MMAs of the first groups
-              // overlap the drain of the later ones
-              if (first_kb && gc > 0) {
+          for (int i = 0; i < S; ++i) {
+            const uint32_t ph = slot0 + i >= OZ_STAGES ? phase0 ^ 1u : phase0;
+            if (!warp_wait(&full[slot_of(i)], ph, lim)) {
+              if (lane == 0) atomicExch(a.err, 23);
+              abort_flag = 1;
+              ok = false;
+              break;
+            }
+            // each group of the previous chunk (of this tile or the one
+            // before) drained by the epilogue, which drains them in order,
+            // before its first MMA of this chunk: the groups first used at
+            // step i are 2i - 1 and 2i, so the MMAs of the first groups
+            // overlap the drain of the later ones
+            if (first_kb && gc > 0) {
 #pragma unroll
-                for (int grp = (i == 0 ? 0 : 2 * i - 1); grp <= 2 * i && grp < S; ++grp)
-                  if (ok && !mbar_wait(&tempty[grp], (uint32_t)(gc - 1) & 1u, lim)) {
-                    atomicExch(a.err, 22);
-                    abort_flag = 1;
-                    ok = false;
-                  }
-                if (!ok) break;
-              }
-              fence_after();
-              const uint32_t si = base + (uint32_t)(gi % OZ_STAGES) * OZ_STAGE_BYTES;
+              for (int grp = (i == 0 ? 0 : 2 * i - 1); grp <= 2 * i && grp < S; ++grp)
+                if (ok && !warp_wait(&tempty[grp], (uint32_t)(gc - 1) & 1u, lim)) {
+                  if (lane == 0) atomicExch(a.err, 22);
+                  abort_flag = 1;
+                  ok = false;
+                }
+              if (!ok) break;
+            }
+            fence_after();
+            const uint32_t si = lo_of(i);
 #pragma unroll
-              for (int j = 0; j <= (i < S - 1 - i ? i : S - 1 - i); ++j) {
-                const uint32_t sj = base + (uint32_t)((g + j) % OZ_STAGES) * OZ_STAGE_BYTES;
-                const uint32_t d = tmem + (uint32_t)((i + j) * BN);
-                const bool overwrite = first_kb && (i - j <= 1);
-                // A slice i x B slice j
+            for (int j = 0; j <= (i < S - 1 - i ? i : S - 1 - i); ++j) {
+              const uint32_t sj = lo_of(j);
+              const uint32_t d = tmem + (uint32_t)((i + j) * BN);
+              const bool overwrite = first_kb && (i - j <= 1);
+              // A slice i x B slice j (32 bytes per K step)
+#pragma unroll
+              for (int k = 0; k < OZ_BK / 16; ++k)
+                mma_bf16_if(leader, d, desc_of(si + 2 * k), desc_of(sj + kB + 2 * k), idesc,
+                            (overwrite && k == 0) ? 0u : 1u);
+              if (j < i) {
+                // A slice j x B slice i
 #pragma unroll
                 for (int k = 0; k < OZ_BK / 16; ++k)
-                  mma_bf16(d, desc_sw128(si + 32 * k), desc_sw128(sj + OZ_A_BYTES + 32 * k),
-                           idesc, (overwrite && k == 0) ? 0u : 1u);
-                if (j < i) {
-                  // A slice j x B slice i
-#pragma unroll
-                  for (int k = 0; k < OZ_BK / 16; ++k)
-                    mma_bf16(d, desc_sw128(sj + 32 * k), desc_sw128(si + OZ_A_BYTES + 32 * k),
-                             idesc, 1u);
-                }
+                  mma_bf16_if(leader, d, desc_of(sj + 2 * k), desc_of(si + kB + 2 * k), idesc, 1u);
               }
-              // slice q is last used at step max(q, S-1-q): release what step i
-              // finished (the stage frees once these MMAs complete)
-              if (i >= S - 1 - i) mma_commit(&empty[gi % OZ_STAGES]);
-              if (S - 1 - i < i) mma_commit(&empty[(g + S - 1 - i) % OZ_STAGES]);
             }
-            if (!ok) break;
-            g += S;
+            // slice q is last used at step max(q, S-1-q): release what step i
+            // finished (the stage frees once these MMAs complete)
+            if (i >= S - 1 - i) mma_commit_if(leader, &empty[slot_of(i)]);
+            if (S - 1 - i < i) mma_commit_if(leader, &empty[slot_of(S - 1 - i)]);
           }
-          if (ok) mma_commit(tfull);
+          if (!ok) break;
+          slot0 += S;
+          if (slot0 >= OZ_STAGES) {
+            slot0 -= OZ_STAGES;
+            phase0 ^= 1u;
+          }
         }
+        if (ok) mma_commit_if(leader, tfull);
       }
-      // every MMA issued here (also after an abort) completes before the
-      // tensor memory is freed
-      mma_commit(drain);
-      mbar_wait(drain, 0u);
     }
+    // every MMA issued here (also after an abort) completes before the
+    // tensor memory is freed
+    mma_commit_if(leader, drain);
+    mbar_wait(drain, 0u);
     __syncwarp();
   } else {
     // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (rows of the tile)

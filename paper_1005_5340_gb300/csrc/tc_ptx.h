@@ -117,6 +117,59 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar) {
           smem_u32(bar))
       : "memory");
 }
+// One lane of a converged warp (the same one at every call).  A role that
+// issues MMAs runs as a whole warp, with warp-uniform loop state, and only the
+// MMAs and commits are predicated on the elected lane: descriptors are then
+// formed in uniform registers.  Inside a one-lane branch every operand is
+// moved to a uniform register first, about 80 clocks per MMA whatever its N
+// (an M = 128, N = 96, K = 16 MMA takes 48).
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t is;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(is));
+  return is;
+}
+// Low word of desc_sw128 of a shared address (the 14-bit address field never
+// carries: shared memory ends below 2^18), and the descriptor at a low word.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return (saddr >> 4) | (1u << 16); }
+__device__ __forceinline__ uint64_t desc_of(uint32_t lo) {
+  constexpr uint32_t kHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+  return ((uint64_t)kHi << 32) | lo;
+}
+__device__ __forceinline__ void mma_bf16_if(uint32_t leader, uint32_t dtmem, uint64_t ad,
+                                            uint64_t bd, uint32_t idesc, uint32_t accum) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
+      "l"(ad), "l"(bd), "r"(idesc), "r"(accum), "r"(leader));
+}
+__device__ __forceinline__ void mma_tf32_if(uint32_t leader, uint32_t dtmem, uint64_t ad,
+                                            uint64_t bd, uint32_t idesc, uint32_t accum) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
+      "l"(ad), "l"(bd), "r"(idesc), "r"(accum), "r"(leader));
+}
+__device__ __forceinline__ void mma_commit_if(uint32_t leader, uint64_t *bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
+          smem_u32(bar)),
+      "r"(leader)
+      : "memory");
+}
+// A wait of the whole warp, one answer for all lanes.
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, uint64_t limit_ns) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit_ns));
+}
 // Sixteen 4-column loads at columns taddr + 16 c (c = 0..15), then the wait:
 // v[c][j] = column 16 c + j of this thread's lane.
 __device__ __forceinline__ void tmem_ld4x16(uint32_t taddr, float (&v)[16][4]) {
