@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "mlp_tc.h"
 
 struct tddft_mlp {
   int n_in = 0, width = 0, n_out = 0;
@@ -26,6 +27,8 @@ struct tddft_mlp {
   float *params = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
   __nv_bfloat16 *params_bf16 = nullptr;
   float *H1 = nullptr, *H2 = nullptr, *dH1 = nullptr, *dH2 = nullptr, *Y = nullptr;
+  bool use_tc = false;   // the tensor-core kernels take this network's shape
+  tddft::MlpTc tc;
   cudaStream_t st = nullptr;
   std::vector<void *> allocs;
   std::string err;
@@ -293,16 +296,36 @@ __global__ void combine_kernel(int64_t n, const float *__restrict__ Y, const dou
   }
 }
 
+tddft_status mfail(tddft_mlp *p, tddft_status s, const std::string &msg);
+
+// After a synchronisation: a wait of the tensor-core kernels that gave up.
+tddft_status check_waits(tddft_mlp *p) {
+  if (!p->use_tc) return TDDFT_OK;
+  int code = 0;
+  cudaError_t e = cudaMemcpy(&code, p->tc.err, sizeof(int), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return mfail(p, TDDFT_ERR_CUDA, cudaGetErrorString(e));
+  if (code == 0) return TDDFT_OK;
+  cudaMemset(p->tc.err, 0, sizeof(int));
+  return mfail(p, TDDFT_ERR_TIMEOUT, "a network kernel's wait gave up (code " +
+                                         std::to_string(code) + ")");
+}
+
 tddft_status mfail(tddft_mlp *p, tddft_status s, const std::string &msg) {
   if (p) p->err = msg;
   else g_mlp_error = msg;
   return s;
 }
 
-cudaError_t forward(tddft_mlp *p, int64_t rows, const float *F, float *Y, bool bf16) {
+// keep: H1 and H2 of every row stay for a backward pass
+cudaError_t forward(tddft_mlp *p, int64_t rows, const float *F, float *Y, bool bf16, bool keep) {
   const int W = p->width, R = (int)rows;
   cudaError_t e;
+  if (p->use_tc)
+    return mlp_tc_forward(p->st, p->tc, p->params, rows, F, keep ? p->H1 : nullptr,
+                          keep ? p->H2 : nullptr, Y, bf16);
   if (bf16) {
+    to_bf16_kernel<<<grid1(p->n_params), 256, 0, p->st>>>(p->n_params, p->params, p->params_bf16);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const __nv_bfloat16 *q = p->params_bf16;
     e = gemm<kBiasTanh>(p->st, R, W, p->n_in, F, p->n_in, 1, q + p->oW1, 1, p->n_in, p->H1, W,
                         p->params + p->ob1);
@@ -326,6 +349,8 @@ cudaError_t forward(tddft_mlp *p, int64_t rows, const float *F, float *Y, bool b
 // grad = d/dparams of sum_rows dY . Y(rows), using H1, H2 of the last forward
 cudaError_t backward(tddft_mlp *p, int64_t rows, const float *F, const float *dY) {
   const int W = p->width, R = (int)rows, no = p->n_out, ni = p->n_in;
+  if (p->use_tc)
+    return mlp_tc_backward(p->st, p->tc, rows, F, dY, p->H1, p->H2, p->dH1, p->grad);
   const float *q = p->params;
   float *g = p->grad;
   cudaError_t e = cudaMemsetAsync(g, 0, p->n_params * sizeof(float), p->st);
@@ -421,8 +446,13 @@ tddft_status tddft_mlp_create(int32_t n_in, int32_t width, int32_t n_out, int64_
   al(&p->H1, (size_t)max_rows * width * sizeof(float));
   al(&p->H2, (size_t)max_rows * width * sizeof(float));
   al(&p->dH1, (size_t)max_rows * width * sizeof(float));
-  al(&p->dH2, (size_t)max_rows * width * sizeof(float));
+  p->use_tc = mlp_tc_fits(n_in, width, n_out);
+  void *tc_mem = nullptr;
+  if (p->use_tc) al((char **)&tc_mem, mlp_tc_bytes(max_rows));
+  else al(&p->dH2, (size_t)max_rows * width * sizeof(float));
   al(&p->Y, (size_t)max_rows * n_out * sizeof(float));
+  if (e == cudaSuccess && p->use_tc)
+    e = mlp_tc_init(p->tc, n_in, width, n_out, max_rows, tc_mem, p->st);
   if (e == cudaSuccess) {
     init_params_kernel<<<grid1(p->n_params), 256, 0, p->st>>>(
         p->n_params, p->params, p->oW1, p->ob1, p->oW2, p->ob2, p->oW3,
@@ -464,7 +494,7 @@ tddft_status tddft_mlp_params(tddft_mlp *p, float *host, int64_t n, int32_t set)
   if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);
   if (e != cudaSuccess) return mfail(p, TDDFT_ERR_CUDA, cudaGetErrorString(e));
   if (set) p->step = 0;
-  return TDDFT_OK;
+  return check_waits(p);
 }
 
 tddft_status tddft_mlp_save(tddft_mlp *p, const char *path) {
@@ -516,12 +546,7 @@ tddft_status tddft_mlp_load(tddft_mlp *p, const char *path) {
 tddft_status tddft_mlp_forward(tddft_mlp *p, int64_t rows, const float *F, float *Y, int32_t bf16) {
   if (!p || !F || !Y) return mfail(p, TDDFT_ERR_INVALID_ARG, "null pointer");
   if (rows < 1 || rows > p->cap_rows) return mfail(p, TDDFT_ERR_SHAPE, "rows beyond max_rows");
-  cudaError_t e = cudaSuccess;
-  if (bf16) {
-    to_bf16_kernel<<<grid1(p->n_params), 256, 0, p->st>>>(p->n_params, p->params, p->params_bf16);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = forward(p, rows, F, Y, bf16 != 0);
+  const cudaError_t e = forward(p, rows, F, Y, bf16 != 0, false);
   if (e != cudaSuccess) return mfail(p, TDDFT_ERR_CUDA, cudaGetErrorString(e));
   return TDDFT_OK;
 }
@@ -530,13 +555,13 @@ tddft_status tddft_mlp_backward(tddft_mlp *p, int64_t rows, const float *F, cons
                                 float *grad_host) {
   if (!p || !F || !dY) return mfail(p, TDDFT_ERR_INVALID_ARG, "null pointer");
   if (rows < 1 || rows > p->cap_rows) return mfail(p, TDDFT_ERR_SHAPE, "rows beyond max_rows");
-  cudaError_t e = forward(p, rows, F, p->Y, false);
+  cudaError_t e = forward(p, rows, F, p->Y, false, true);
   if (e == cudaSuccess) e = backward(p, rows, F, dY);
   if (e == cudaSuccess && grad_host)
     e = cudaMemcpyAsync(grad_host, p->grad, p->n_params * sizeof(float), cudaMemcpyDeviceToHost, p->st);
   if (e == cudaSuccess && grad_host) e = cudaStreamSynchronize(p->st);
   if (e != cudaSuccess) return mfail(p, TDDFT_ERR_CUDA, cudaGetErrorString(e));
-  return TDDFT_OK;
+  return grad_host ? check_waits(p) : TDDFT_OK;
 }
 
 tddft_status tddft_mlp_train_step(tddft_mlp *p, int32_t n_target, int32_t n_prod, const float *F,
@@ -548,7 +573,7 @@ tddft_status tddft_mlp_train_step(tddft_mlp *p, int32_t n_target, int32_t n_prod
   const int64_t rows = (int64_t)n_target * n_prod;
   if (n_target < 1 || n_prod < 1 || rows > p->cap_rows)
     return mfail(p, TDDFT_ERR_SHAPE, "rows beyond max_rows");
-  cudaError_t e = forward(p, rows, F, p->Y, false);
+  cudaError_t e = forward(p, rows, F, p->Y, false, true);
   if (e == cudaSuccess) {
     // dY reuses dH1's storage (rows x 2 <= rows x width)
     guess_loss_kernel<<<n_target, 256, 0, p->st>>>(n_prod, n_target, p->Y, lin, xstar, scale,
