@@ -36,12 +36,6 @@
 namespace tddft {
 namespace {
 
-int grid_for(int64_t total, int threads) {
-  int64_t g = (total + threads - 1) / threads;
-  if (g > 152 * 32) g = 152 * 32;
-  return (int)(g < 1 ? 1 : g);
-}
-
 // One CTA per product (Vpad row q): every (side, c, E) of alpha_mu, written
 // to the step-2 operand (row (ao_X n_occ + E n_X + c), column pos_X) and to
 // the step-5 operand (row rowoff5_X + pos_X, column c n_occ + E).
@@ -132,44 +126,104 @@ __global__ void alpha_part_kernel(int64_t rows, int K2max, int n_occ, int n_orb,
   }
 }
 
-// Ycat[c][k] = Y[c][lcat[k]] (0 where lcat[k] < 0), split bf16 (or tf32)
+// Ycat[c][k] = Y[c][lcat[k]] (0 where lcat[k] < 0), split bf16 (or tf32): two
+// neighbouring k per thread (4-byte stores), their list entries read once for
+// kGatherCols columns.  Y: rows c of ld, or, interleaved, complex vectors of ld.
+constexpr int kGatherCols = 8;
 template <class T>
-__global__ void gather_split_kernel(int ncols, int kcat, const int *__restrict__ lcat,
-                                    const T *__restrict__ Y, int64_t ld,
-                                    void *__restrict__ dstv, bool tf32, const int *dcnt) {
+__global__ void __launch_bounds__(256) gather_split_kernel(int ncols, int kcat,
+                                                           const int *__restrict__ lcat,
+                                                           const T *__restrict__ Y, int64_t ld,
+                                                           bool inter, void *__restrict__ dstv,
+                                                           bool tf32, const int *dcnt) {
   if (dcnt) ncols = min(ncols, 2 * *dcnt);
-  const int64_t total = (int64_t)ncols * kcat;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = i / kcat;
-    const int k = (int)(i - c * kcat);
-    const int mu = lcat[k];
-    const float x = mu >= 0 ? (float)Y[c * ld + mu] : 0.f;
+  const int k = 2 * (blockIdx.x * 256 + threadIdx.x);
+  if (k >= kcat) return;
+  const int2 mu = *(const int2 *)(lcat + k);
+  const int c1 = min(ncols, ((int)blockIdx.y + 1) * kGatherCols);
+#pragma unroll 4
+  for (int c = blockIdx.y * kGatherCols; c < c1; ++c) {
+    const T *y = inter ? Y + (int64_t)(c >> 1) * 2 * ld + (c & 1) : Y + c * ld;
+    const int st = inter ? 2 : 1;
+    const float x0 = mu.x >= 0 ? (float)y[(int64_t)mu.x * st] : 0.f;
+    const float x1 = mu.y >= 0 ? (float)y[(int64_t)mu.y * st] : 0.f;
     if (tf32) {
-      ((float *)dstv)[i] = ptx::tf32_round(x);
+      *(float2 *)((float *)dstv + (int64_t)c * kcat + k) =
+          make_float2(ptx::tf32_round(x0), ptx::tf32_round(x1));
       continue;
     }
-    __nv_bfloat16 *dst = (__nv_bfloat16 *)dstv;
-    const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-    dst[c * 2 * kcat + k] = hi;
-    dst[c * 2 * kcat + kcat + k] = __float2bfloat16_rn(x - __bfloat162float(hi));
+    __nv_bfloat16 *dst = (__nv_bfloat16 *)dstv + (int64_t)c * 2 * kcat + k;
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+    *(__nv_bfloat162 *)dst = h;
+    *(__nv_bfloat162 *)(dst + kcat) =
+        __floats2bfloat162_rn(x0 - __bfloat162float(h.x), x1 - __bfloat162float(h.y));
   }
 }
 
+// float32 -> float64 in the integer pipe (a conversion would take the FP64
+// pipe's time); subnormals, infinities and NaN convert.
+__device__ __forceinline__ double to_f64(float x) {
+  const unsigned int u = __float_as_uint(x), e = (u >> 23) & 0xFF;
+  if (e == 0xFF || (e == 0 && (u << 1) != 0)) return (double)x;
+  const unsigned int top = (u & 0x80000000u) | (e == 0 ? 0u : ((u & 0x7FFFFFFFu) >> 3) + 0x38000000u);
+  return __hiloint2double((int)top, (int)(u << 29));
+}
+__device__ __forceinline__ double to_f64(double x) { return x; }
+
+// Out = Zin - n or n, n_mu the sum of product mu's one or two partials (first
+// the smaller atom's): tiles of 32 products x 32 columns, the partials read
+// along the columns (their rows) and passed through shared memory.  Zin and Out:
+// rows c of n_prod, or, interleaved, complex vectors.
 template <class TP>
-__global__ void combine_kernel(int ncols, int n_prod, const int2 *__restrict__ pos5,
-                               const TP *__restrict__ P2, int ldp, const double *__restrict__ Zin,
-                               int subtract, double *__restrict__ Out, const int *dcnt) {
+__global__ void __launch_bounds__(256) combine_kernel(int ncols, int n_prod,
+                                                      const int2 *__restrict__ pos5,
+                                                      const TP *__restrict__ P2, int ldp,
+                                                      const double *__restrict__ Zin, int subtract,
+                                                      double *__restrict__ Out, bool inter,
+                                                      const int *dcnt) {
+  __shared__ TP ta[32][33], tb[32][33];
   if (dcnt) ncols = min(ncols, 2 * *dcnt);
-  const int64_t total = (int64_t)ncols * n_prod;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = i / n_prod;
-    const int mu = (int)(i - c * n_prod);
-    const int2 p = pos5[mu];
-    double n = (double)P2[(int64_t)p.x * ldp + c];
-    if (p.y >= 0) n += (double)P2[(int64_t)p.y * ldp + c];
-    Out[i] = subtract ? Zin[i] - n : n;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int mu0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
+  if (c0 >= ncols) return;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int m = warp + 8 * i, c = c0 + lane;
+    TP a = 0, b = 0;
+    if (mu0 + m < n_prod && c < ncols) {
+      const int2 p = pos5[mu0 + m];
+      a = P2[(int64_t)p.x * ldp + c];
+      if (p.y >= 0) b = P2[(int64_t)p.y * ldp + c];
+    }
+    ta[m][lane] = a;
+    tb[m][lane] = b;
+  }
+  __syncthreads();
+  const int mu = mu0 + lane;
+  if (mu >= n_prod) return;
+  if (inter) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int v = warp + 8 * i, c = c0 + 2 * v;   // vector c / 2
+      if (c >= ncols) continue;
+      double2 n = make_double2(to_f64(ta[lane][2 * v]) + to_f64(tb[lane][2 * v]),
+                               to_f64(ta[lane][2 * v + 1]) + to_f64(tb[lane][2 * v + 1]));
+      const int64_t at = (int64_t)(c >> 1) * n_prod + mu;
+      if (subtract) {
+        const double2 z = ((const double2 *)Zin)[at];
+        n = make_double2(z.x - n.x, z.y - n.y);
+      }
+      ((double2 *)Out)[at] = n;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int v = warp + 8 * i, c = c0 + v;
+      if (c >= ncols) continue;
+      const double n = to_f64(ta[lane][v]) + to_f64(tb[lane][v]);
+      const int64_t at = (int64_t)c * n_prod + mu;
+      Out[at] = subtract ? Zin[at] - n : n;
+    }
   }
 }
 
@@ -213,7 +267,7 @@ cudaError_t alpha_setup(cudaStream_t st, const tddft_system *h, const DevSystem 
   ar.kcat2 = std::max((int)lcat.size(), 64);
   while ((int)lcat.size() < ar.kcat2) lcat.push_back(-1);
   ar.kcat5 = kcat5;
-  ar.ldp = 2 * std::max(slots, 3);
+  ar.ldp = round_up(2 * std::max(slots, 3), 4);   // rows of 16-byte stores
   // tiles (128 rows of the per-atom operands), atom by atom
   std::vector<GTile> t2, t5, t5lp;   // t5lp: 256-row entries (two M blocks per tile)
   ar.flops2 = ar.flops5 = 0.0;
@@ -387,28 +441,30 @@ cudaError_t alpha_setup(cudaStream_t st, const tddft_system *h, const DevSystem 
 }
 
 cudaError_t launch_alpha_gather_lp(cudaStream_t st, const AlphaRoute &ar, int ncols, const void *Y,
-                                   bool y_f64, int64_t ld, const int *dcnt) {
-  const int g = grid_for((int64_t)ncols * ar.kcat2, 256);
+                                   bool y_f64, bool inter, int64_t ld, const int *dcnt) {
+  const dim3 grid((ar.kcat2 / 2 + 255) / 256, (ncols + kGatherCols - 1) / kGatherCols);
+  if (grid.y > 65535) return cudaErrorInvalidConfiguration;
   __nv_bfloat16 *dst = ar.ycat_q;
   if (y_f64)
-    gather_split_kernel<double><<<g, 256, 0, st>>>(ncols, ar.kcat2, ar.lcat, (const double *)Y, ld,
-                                                   dst, ar.tf32, dcnt);
+    gather_split_kernel<double><<<grid, 256, 0, st>>>(ncols, ar.kcat2, ar.lcat, (const double *)Y,
+                                                      ld, inter, dst, ar.tf32, dcnt);
   else
-    gather_split_kernel<float><<<g, 256, 0, st>>>(ncols, ar.kcat2, ar.lcat, (const float *)Y, ld,
-                                                  dst, ar.tf32, dcnt);
+    gather_split_kernel<float><<<grid, 256, 0, st>>>(ncols, ar.kcat2, ar.lcat, (const float *)Y, ld,
+                                                     false, dst, ar.tf32, dcnt);
   return cudaGetLastError();
 }
 
 cudaError_t launch_alpha_combine(cudaStream_t st, const AlphaRoute &ar, int ncols, int n_prod,
                                  bool p_f64, const double *Zin, int subtract, double *Out,
-                                 const int *dcnt) {
-  const int g = grid_for((int64_t)ncols * n_prod, 256);
+                                 const int *dcnt, bool inter) {
+  const dim3 grid((n_prod + 31) / 32, (ncols + 31) / 32);
+  if (grid.y > 65535) return cudaErrorInvalidConfiguration;
   if (p_f64)
-    combine_kernel<double><<<g, 256, 0, st>>>(ncols, n_prod, ar.pos5, ar.P2d, ar.ldp, Zin,
-                                              subtract, Out, dcnt);
+    combine_kernel<double><<<grid, 256, 0, st>>>(ncols, n_prod, ar.pos5, ar.P2d, ar.ldp, Zin,
+                                                 subtract, Out, inter, dcnt);
   else
-    combine_kernel<float><<<g, 256, 0, st>>>(ncols, n_prod, ar.pos5, ar.P2f, ar.ldp, Zin, subtract,
-                                             Out, dcnt);
+    combine_kernel<float><<<grid, 256, 0, st>>>(ncols, n_prod, ar.pos5, ar.P2f, ar.ldp, Zin,
+                                                subtract, Out, inter, dcnt);
   return cudaGetLastError();
 }
 

@@ -45,6 +45,7 @@ using namespace ptx;
 
 constexpr int TC_BM = 128, TC_BK = 64;
 constexpr int TC_EPI_WARPS = 8;                     // two per TMEM lane quadrant
+constexpr int TC_EPI_GROUPS = TC_EPI_WARPS / 4;     // warps per lane quadrant, sharing the columns
 constexpr int TC_THREADS = 64 + 32 * TC_EPI_WARPS;   // producer, MMA issuer, epilogue
 constexpr uint32_t TC_A_BYTES = TC_BM * TC_BK * 2;    // 16 KB per plane
 constexpr int TC_EOCC_MAX = 1024;   // occupied energies staged in shared memory (D(omega) epilogue)
@@ -111,17 +112,20 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
-// kDscaleSplit: the (omega -+ e_F) terms of the chunk's first slot (loaded
-// before the chunk's TMEM read) and the occupied energies (shared memory)
-struct DscaleIn {
-  float4 dt;
+// Inputs of a 16-column piece beside the accumulator: kDscaleSplit the
+// (omega -+ e_F) terms of its eight slots (loaded together, ahead of the TMEM
+// read: one load after the other would cost its latency per pair) and the
+// occupied energies (shared memory); kGammaCatSplit the row's Gcat offset.
+struct EpiIn {
+  float4 dt[8];
   const float2 *eocc;
+  int64_t xo;
 };
 
 template <int EPI, bool TF>
 __device__ __forceinline__ void epilogue16(const float (&v)[16], int m, int lr, int rows_valid,
                                            int atom, int M, int N, int n0, int j0,
-                                           const TcEpilogue &ep, const DscaleIn &di) {
+                                           const TcEpilogue &ep, const EpiIn &di) {
   if (EPI == kStoreF32) {
     if (m < M) {
       if (ep.ksplit > 1) {
@@ -139,9 +143,14 @@ __device__ __forceinline__ void epilogue16(const float (&v)[16], int m, int lr, 
         }
       }
     }
-  } else if (EPI == kPartialF32) {
+  } else if (EPI == kPartialF32 || EPI == kPartialOneF32) {
     // C layout, rows of the grouped operand
-    if (lr < rows_valid) {
+    if (lr < rows_valid && (ep.ldo & 3) == 0 && n0 + j0 + 16 <= N) {
+      float4 *dst = (float4 *)(ep.outF + (int64_t)m * ep.ldo + n0 + j0);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+    } else if (lr < rows_valid) {
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         const int n = n0 + j0 + j;
@@ -154,8 +163,7 @@ __device__ __forceinline__ void epilogue16(const float (&v)[16], int m, int lr, 
     // row m = orbital (atom B, b); column n = (s n_occ + E) 2 + p, j = 2 s + p:
     // Gcat[j][xoff5_B + b n_occ + E]
     if (m < M) {
-      const int B = ep.orb_atom[m], b = m - ep.aoff[B];
-      const int64_t xo = ep.xoff5[B] + (int64_t)b * ep.n_occ;
+      const int64_t xo = di.xo;
       const int pair0 = (n0 + j0) >> 1;
       if (ep.n_occ % 8 == 0 && n0 + j0 + 16 <= N) {
         // the 16 columns are E0 .. E0+7 of one slot, both planes: four
@@ -181,14 +189,43 @@ __device__ __forceinline__ void epilogue16(const float (&v)[16], int m, int lr, 
           }
         }
       } else {
+        // eight states E from pair0 on, over one slot's end if need be; with an
+        // even n_occ two neighbours at a time (4-byte stores: every offset is
+        // even, and a slot holds an even number of states)
+        int sl = pair0 / ep.n_occ, E = pair0 - sl * ep.n_occ;
+        if (!TF && ep.n_occ % 2 == 0) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int n = n0 + j0 + j;
-          if (n < N) {
-            const int pair = n >> 1, p = n & 1;
-            const int sl = pair / ep.n_occ, E = pair - sl * ep.n_occ;
-            put_operand<TF>(ep.outB, (int64_t)(2 * sl + p) * operand_ld<TF>(ep) + xo + E, ep.lo_off,
-                            v[j]);
+          for (int e = 0; e < 8; e += 2) {
+            if (n0 + j0 + 2 * e < N) {
+#pragma unroll
+              for (int p = 0; p < 2; ++p) {
+                __nv_bfloat162 h, l;
+                split_bf16(v[2 * e + p], h.x, l.x);
+                split_bf16(v[2 * e + 2 + p], h.y, l.y);
+                __nv_bfloat16 *dst = (__nv_bfloat16 *)ep.outB +
+                                     (int64_t)(2 * sl + p) * operand_ld<TF>(ep) + xo + E;
+                *(__nv_bfloat162 *)dst = h;
+                *(__nv_bfloat162 *)(dst + ep.lo_off) = l;
+              }
+            }
+            if ((E += 2) == ep.n_occ) {
+              E = 0;
+              ++sl;
+            }
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            if (n0 + j0 + 2 * e < N) {
+#pragma unroll
+              for (int p = 0; p < 2; ++p)
+                put_operand<TF>(ep.outB, (int64_t)(2 * sl + p) * operand_ld<TF>(ep) + xo + E,
+                                ep.lo_off, v[2 * e + p]);
+            }
+            if (++E == ep.n_occ) {
+              E = 0;
+              ++sl;
+            }
           }
         }
       }
@@ -209,21 +246,15 @@ __device__ __forceinline__ void epilogue16(const float (&v)[16], int m, int lr, 
       const int hs = max(1, N / (2 * ep.n_occ));
       const int pair0 = (n0 + j0) >> 1;
       int E = pair0 / hs, sl = pair0 - E * hs;
-      // (omega -+ e_F) of each pair's slot as float (hi, lo) pairs,
-      // precomputed per (slot, F) for this product; the first is loaded
-      // before the chunk's TMEM read
-      float4 dt = di.dt;
-      int dsl = sl;
+      // di.dt: (omega -+ e_F) of each pair's slot as float (hi, lo) pairs,
+      // precomputed per (slot, F) for this product
 #pragma unroll
       for (int j = 0; j < 16; j += 2) {
         const int n = n0 + j0 + j;
         if (n >= N) continue;
         float re = 0.f, im = 0.f;
         if (live) {
-          if (sl != dsl) {
-            dt = ep.dterm[(int64_t)sl * M + m];
-            dsl = sl;
-          }
+          const float4 dt = di.dt[j >> 1];
           const float2 eE = di.eocc[E];
           const float xm = (dt.x + eE.x) + (dt.y + eE.y);
           const float xp = (dt.z - eE.x) + (dt.w - eE.y);
@@ -567,15 +598,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         break;
       }
       fence_after();
-      // the two warps of a lane quadrant take the two halves of the columns
-      // (M2: the two M blocks, all columns each)
-      const int blk = (kM2 && warp >= 6) ? 1 : 0;
+      // the warps of a lane quadrant share the columns (M2: first the two M
+      // blocks, then the columns of each)
+      const int grp = (warp - 2) >> 2;
+      constexpr int kShare = kM2 ? TC_EPI_GROUPS / 2 : TC_EPI_GROUPS;   // warps per M block
+      const int blk = kM2 ? grp / kShare : 0, part = grp % kShare;
       const int m = m0 + blk * TC_BM + lr;
       const int rv_blk = kM2 ? min(TC_BM, rows_valid - blk * TC_BM) : rows_valid;
       const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * ACC + blk * TC_BN);
-      const int half = ((tn >> 4) + 1) / 2 * 16;
-      const int j_lo = kM2 ? 0 : ((warp >= 6) ? half : 0);
-      const int j_hi = kM2 ? tn : ((warp >= 6) ? tn : half);
+      const int per = ((tn >> 4) + kShare - 1) / kShare * 16;
+      const int j_lo = min(tn, part * per), j_hi = min(tn, j_lo + per);
       if (kPart) {
         // step 2: tensor-memory column c16 16 + e holds orbital 16 k + c16
         // (k = atom, the chunk) and occupied state E = 16 eb + e of column
@@ -585,8 +617,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const int eb = n0 / 256 - atom * ((ep.n_occ + 15) / 16);
         const int mm = m0 + lr;
 #pragma unroll 1
-        for (int r = 0; r < 2; ++r) {
-          const int e0 = ((warp >= 6) ? 8 : 0) + 4 * r;
+        for (int r = 0; r < 4 / TC_EPI_GROUPS; ++r) {
+          const int e0 = 16 / TC_EPI_GROUPS * grp + 4 * r;
           float v[16][4];
           tmem_ld4x16(trow + (uint32_t)e0, v);
 #pragma unroll
@@ -613,14 +645,22 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           }
         }
       }
+      EpiIn di;
+      di.eocc = eocc;
+      if (EPI == kGammaCatSplit && m < M) {
+        const int B = ep.orb_atom[m], b = m - ep.aoff[B];
+        di.xo = ep.xoff5[B] + (int64_t)b * ep.n_occ;
+      }
+      const int hs = EPI == kDscaleSplit ? max(1, N / (2 * ep.n_occ)) : 1;   // live slots
       for (int j0 = j_lo; j0 < j_hi && !kPart; j0 += 16) {
-        DscaleIn di;
-        di.eocc = eocc;
         if (EPI == kDscaleSplit) {
-          const int hs = max(1, N / (2 * ep.n_occ));   // live slots (E-major columns)
-          const int sl0 = ((n0 + j0) >> 1) % hs;
-          di.dt = (m < M && n0 + j0 < N) ? ep.dterm[(int64_t)sl0 * M + m]
-                                         : make_float4(0.f, 0.f, 0.f, 0.f);
+          int sl = ((n0 + j0) >> 1) % hs;   // E-major columns: consecutive slots
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            di.dt[i] = (m < M && n0 + j0 + 2 * i < N) ? ep.dterm[(int64_t)sl * M + m]
+                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (++sl == hs) sl = 0;
+          }
         }
         float v[16];
         tmem_ld16(trow + (uint32_t)j0, v);
@@ -734,6 +774,7 @@ void set_attr_all() {
   set_attr<kBetaPartSplit, BN>();
   set_attr<kGammaCatSplit, BN>();
   set_attr<kPartialF32, BN>();
+  set_attr<kPartialOneF32, BN>();
 }
 }  // namespace
 
@@ -822,6 +863,9 @@ cudaError_t launch_tc_epi(cudaStream_t st, int epi, int M, int N, const CUtensor
     case kPartialF32:
       return launch_tc<kPartialF32, BN, TF>(st, grid, mA, mB, mB64, mB128, M, N, KpA, KpB, ep, err,
                                     dcnt, mul_n, tiles, n_mtiles);
+    case kPartialOneF32:
+      return launch_tc<kPartialOneF32, BN, TF>(st, grid, mA, mB, mB64, mB128, M, N, KpA, KpB, ep,
+                                               err, dcnt, mul_n, tiles, n_mtiles);
     default:
       return cudaErrorInvalidValue;
   }
@@ -877,7 +921,7 @@ cudaError_t launch_gemm_tc(cudaStream_t st, const TcOperand &A, const TcOperand 
   e.ksplit = 1;
   if (epi == kStoreF32 && ep.split_ok) {
     tc_split_plan(A.Kp, M, N, bn, &e.ksplit, &e.ncl);
-    if (e.ksplit > 1) {
+    if (e.ksplit > 1 && !ep.cleared) {
       cudaError_t r = cudaMemsetAsync(ep.outF, 0, (size_t)N * ep.ldo * sizeof(float), st);
       if (r != cudaSuccess) return r;
     }

@@ -23,8 +23,10 @@
 // ||R_j^-1||_F^2; ||H_j^-1||_F follows because H_j and R_j differ by a unitary
 // factor except in the last diagonal entry (before the last rotation in H_j).
 #include <cooperative_groups.h>
+#include <cuda_bf16.h>
 
 #include "internal.h"
+#include "tc_ptx.h"
 
 namespace cg = cooperative_groups;
 
@@ -266,25 +268,86 @@ __global__ void __launch_bounds__(1024) gmres_select_kernel(const int *__restric
   }
 }
 
-// Operator input of each active right-hand side: v_j (Arnoldi) or x (residual).
+// The reduced-precision operator's copy of its input, written by the gather
+// (the basis is float32 there, so the split needs no float64 operation).
+struct GatherSplit {
+  void *Zb = nullptr;      // rows c: [hi | lo] bf16 of Kp entries, or Kp tf32 floats
+  int Kp = 0;
+  bool tf32 = false;
+  float *zero = nullptr;   // rows to clear (lp_cleared_output)
+};
+
+__device__ __forceinline__ void put_split(const GatherSplit &g, int64_t row, int e, float x) {
+  if (g.tf32) {
+    ((float *)g.Zb)[row * g.Kp + e] = ptx::tf32_round(x);
+    return;
+  }
+  __nv_bfloat16 *d = (__nv_bfloat16 *)g.Zb + row * 2 * g.Kp + e;
+  const __nv_bfloat16 h = __float2bfloat16_rn(x);
+  d[0] = h;
+  d[g.Kp] = __float2bfloat16_rn(x - __bfloat162float(h));
+}
+__device__ __forceinline__ void put_split4(const GatherSplit &g, int64_t row, int e, float4 x) {
+  if (g.tf32) {
+    *(float4 *)((float *)g.Zb + row * g.Kp + e) =
+        make_float4(ptx::tf32_round(x.x), ptx::tf32_round(x.y), ptx::tf32_round(x.z),
+                    ptx::tf32_round(x.w));
+    return;
+  }
+  __nv_bfloat16 *d = (__nv_bfloat16 *)g.Zb + row * 2 * g.Kp + e;
+  __nv_bfloat162 h[2] = {__floats2bfloat162_rn(x.x, x.y), __floats2bfloat162_rn(x.z, x.w)};
+  __nv_bfloat162 l[2] = {__floats2bfloat162_rn(x.x - __bfloat162float(h[0].x),
+                                               x.y - __bfloat162float(h[0].y)),
+                         __floats2bfloat162_rn(x.z - __bfloat162float(h[1].x),
+                                               x.w - __bfloat162float(h[1].y))};
+  *(uint2 *)d = *(const uint2 *)h;
+  *(uint2 *)(d + g.Kp) = *(const uint2 *)l;
+}
+
+// Operator input of each active right-hand side: v_j (Arnoldi) or x
+// (residual); blockIdx.y the plane.  With gs.Zb also its split.
 template <class T>
 __global__ void __launch_bounds__(NT) gmres_gather_kernel(Gs G, const int *__restrict__ list,
                                                           double *__restrict__ Zc,
                                                           double *__restrict__ slot_omega,
-                                                          const int *__restrict__ dcnt) {
-  const int s = blockIdx.x;
+                                                          const int *__restrict__ dcnt,
+                                                          GatherSplit gs) {
+  const int s = blockIdx.x, p = blockIdx.y;
   if (dcnt && s >= *dcnt) return;
   const int r = list[s];
   const int N = G.n_prod;
-  double *dst = Zc + (int64_t)2 * s * N;
+  const int64_t row = 2 * (int64_t)s + p;
+  double *dst = Zc + row * N;
+  float *zero = gs.zero ? gs.zero + row * N : nullptr;
   if (G.state[r] == kStateArnoldi) {
-    const T *src = basis<T>(G) + ((int64_t)r * (G.m + 1) + G.jcur[r]) * 2 * N;
-    for (int e = threadIdx.x; e < 2 * N; e += NT) dst[e] = (double)src[e];
+    const T *src = basis<T>(G) + (((int64_t)r * (G.m + 1) + G.jcur[r]) * 2 + p) * N;
+    if constexpr (sizeof(T) == 4) {
+      if ((N & 3) == 0) {
+        // four entries per thread and access (every row starts on 16 bytes)
+        for (int e = 4 * threadIdx.x; e < N; e += 4 * NT) {
+          const float4 v = *(const float4 *)(src + e);
+          *(double2 *)(dst + e) = make_double2((double)v.x, (double)v.y);
+          *(double2 *)(dst + e + 2) = make_double2((double)v.z, (double)v.w);
+          if (gs.Zb) put_split4(gs, row, e, v);
+          if (zero) *(float4 *)(zero + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      } else {
+        for (int e = threadIdx.x; e < N; e += NT) {
+          const float v = src[e];
+          dst[e] = (double)v;
+          if (gs.Zb) put_split(gs, row, e, v);
+          if (zero) zero[e] = 0.f;
+        }
+      }
+    } else {
+      for (int e = threadIdx.x; e < N; e += NT) dst[e] = (double)src[e];
+    }
   } else {
-    const double *src = G.x + (int64_t)2 * r * N;
-    for (int e = threadIdx.x; e < 2 * N; e += NT) dst[e] = src[e];
+    // (never with gs.Zb: residuals take the float64 operator)
+    const double *src = G.x + ((int64_t)2 * r + p) * N;
+    for (int e = threadIdx.x; e < N; e += NT) dst[e] = src[e];
   }
-  if (threadIdx.x == 0) slot_omega[s] = G.omega[r];
+  if (threadIdx.x == 0 && p == 0) slot_omega[s] = G.omega[r];
 }
 
 // Sum of NV values over the P CTAs of the cluster (after the block sums), in
@@ -1187,13 +1250,22 @@ cudaError_t launch_gmres_select(cudaStream_t st, GmresState &gs, int n, int spli
 
 cudaError_t launch_gmres_gather(cudaStream_t st, const DevSystem &sys, GmresState &gs,
                                 const int *list, int S, double *Zc, double *slot_omega,
-                                const int *dcnt) {
+                                const int *dcnt, const LpWork *lp) {
   if (S <= 0) return cudaSuccess;
   if (!gs.V && !gs.Vf) return cudaErrorInvalidValue;
+  GatherSplit sp;
+  if (lp) {
+    if (!gs.Vf) return cudaErrorInvalidValue;
+    sp.Zb = lp->Zb;
+    sp.Kp = lp->KpK;
+    sp.tf32 = lp->tf32;
+    sp.zero = lp_cleared_output(sys, *lp, 2 * S);
+  }
+  const dim3 grid(S, 2);
   if (gs.Vf)
-    gmres_gather_kernel<float><<<S, NT, 0, st>>>(view(gs, sys), list, Zc, slot_omega, dcnt);
+    gmres_gather_kernel<float><<<grid, NT, 0, st>>>(view(gs, sys), list, Zc, slot_omega, dcnt, sp);
   else
-    gmres_gather_kernel<double><<<S, NT, 0, st>>>(view(gs, sys), list, Zc, slot_omega, dcnt);
+    gmres_gather_kernel<double><<<grid, NT, 0, st>>>(view(gs, sys), list, Zc, slot_omega, dcnt, sp);
   return cudaGetLastError();
 }
 

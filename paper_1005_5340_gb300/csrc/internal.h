@@ -144,7 +144,7 @@ struct GTile {
   int row0, xoff, nkb, rows, atom, pad0, pad1, pad2;
 };
 
-enum TcEpi { kStoreF32 = 0, kDscaleSplit = 1, kBetaPartSplit = 2, kGammaCatSplit = 3, kPartialF32 = 4 };
+enum TcEpi { kStoreF32 = 0, kDscaleSplit = 1, kBetaPartSplit = 2, kGammaCatSplit = 3, kPartialF32 = 4, kPartialOneF32 = 5 };
 
 // A bf16 operand [rows][2*Kp] ([hi | lo] planes) with its TMA descriptor.
 struct TcOperand {
@@ -167,11 +167,11 @@ struct TcEpilogue {
   const double *energy = nullptr;  // [n_orb]
   const float2 *eocc2 = nullptr;   // [n_occ] occupied energies as float (hi, lo)
   const float4 *dterm = nullptr;   // [S][M] omega_s -+ e_F as float (hi, lo, hi, lo)
-  const double *omega = nullptr;   // [S]
   double eps = 0.0;
   double occ_value = 0.0;
   int n_occ = 0;
   int split_ok = 0;                // kStoreF32: the launch may split K in two (adds into outF)
+  int cleared = 0;                 // kStoreF32: the caller has cleared outF for that
   int ksplit = 1;                  // set by the launcher
   int ncl = 1;                     // set by the launcher: > 1, clusters of ncl CTAs, one per N tile
   const int *aoff = nullptr;       // kGammaCatSplit
@@ -204,6 +204,7 @@ cudaError_t launch_gemm_tc(cudaStream_t st, const TcOperand &A, const TcOperand 
 //   kPartialF32     one table entry per tile (A rows, up to 256: two M
 //                   blocks sharing the B tile; B K offset and length);
 //                   outF[m*ldo + n] for the valid rows
+//   kPartialOneF32  the same over entries of up to 128 rows, one M block
 // (the plain launch_gemm_tc also takes kGammaCatSplit: row m = orbital (B, b),
 // column n = (s n_occ + E) 2 + p -> Gcat split at row 2 s + p, column
 // xoff5_B + b n_occ + E.)
@@ -263,9 +264,17 @@ cudaError_t lp_prepare_constants(cudaStream_t st, const DevSystem &sys, LpWork &
 // Time the N tiles (64, 128, 256) on this context's three products (the full batch; the
 // K product also at half of it) and keep the fastest, best of four runs each.
 cudaError_t lp_autotune(cudaStream_t st, const DevSystem &sys, LpWork &lp);
-// Out[c][mu] (float64) = Zin - chi0 K Zin (kA) or chi0 Zin (kChi0), reduced precision.
+// Out (float64) = Zin - chi0 K Zin (kA) or chi0 Zin (kChi0), reduced precision.
+// Zin and Out are planar rows c, interleaved complex vectors (kInterleaved),
+// or planar with the K product's operand already in lp.Zb (kSplitDone: written,
+// and lp_cleared_output's rows cleared, by launch_gmres_gather).  omega: the
+// frequency of each slot (NULL: lp.omega).
+enum LpInput { kPlanar = 0, kInterleaved = 1, kSplitDone = 2 };
 cudaError_t launch_apply_operator_lp(cudaStream_t st, const DevSystem &sys, LpWork &lp, int S,
-                                     OpMode mode, double eps, const double *Zin, double *Out);
+                                     OpMode mode, double eps, const double *Zin, double *Out,
+                                     LpInput input = kPlanar, const double *omega = nullptr);
+// The rows to clear before the K product of ncols columns, or NULL.
+float *lp_cleared_output(const DevSystem &sys, const LpWork &lp, int ncols);
 
 // ---------------------------------------------------------------------------
 // Float64 products emulated on the tensor cores (ozaki.cu)
@@ -393,11 +402,11 @@ cudaError_t alpha_setup(cudaStream_t st, const tddft_system *host, const DevSyst
                         std::vector<void *> &allocs);
 // Ycat split bf16 from rows of Y (float32 or float64, row stride ld)
 cudaError_t launch_alpha_gather_lp(cudaStream_t st, const AlphaRoute &ar, int ncols, const void *Y,
-                                   bool y_f64, int64_t ld, const int *dcnt);
+                                   bool y_f64, bool inter, int64_t ld, const int *dcnt);
 // Out[c][mu] = Zin - n (subtract) or n, n_mu summed from the per-atom partials
 cudaError_t launch_alpha_combine(cudaStream_t st, const AlphaRoute &ar, int ncols, int n_prod,
                                  bool p_f64, const double *Zin, int subtract, double *Out,
-                                 const int *dcnt);
+                                 const int *dcnt, bool inter = false);
 
 // GMRES state of a group of right-hand sides (one per (omega, direction)).
 struct GmresState {
@@ -451,7 +460,7 @@ cudaError_t launch_gmres_prepare(cudaStream_t st, const DevSystem &sys, GmresSta
 cudaError_t launch_gmres_select(cudaStream_t st, GmresState &gs, int n, int split, int min_b = 1);
 cudaError_t launch_gmres_gather(cudaStream_t st, const DevSystem &sys, GmresState &gs,
                                 const int *list, int S, double *Zc, double *slot_omega,
-                                const int *dcnt = nullptr);
+                                const int *dcnt = nullptr, const LpWork *lp = nullptr);
 cudaError_t launch_gmres_step(cudaStream_t st, const DevSystem &sys, GmresState &gs,
                               const int *list, int S, const double *Wout,
                               const int *dcnt = nullptr);

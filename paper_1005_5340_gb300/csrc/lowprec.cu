@@ -15,6 +15,8 @@
 //   aT     [2 S n_occ][2 Kp2]   (D . X_virt^T beta)^T split
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "internal.h"
 #include "tc_ptx.h"
 
@@ -44,9 +46,7 @@ struct Scope {
 // dst[r][k] = hi(src[r, k]), dst[r][Kp + k] = lo(src[r, k]); zero for k >= cols.
 // With tf32: dst is float [r][Kp], the value rounded to tf32 (same bytes per row).
 __global__ void split_rows_kernel(const double *__restrict__ src, int64_t rs, int64_t cs, int rows,
-                                  int cols, int Kp, void *__restrict__ dstv, bool tf32,
-                                  const int *__restrict__ dcnt = nullptr, int mul_r = 0) {
-  if (dcnt) rows = min(rows, mul_r * *dcnt);
+                                  int cols, int Kp, void *__restrict__ dstv, bool tf32) {
   const int64_t total = (int64_t)rows * Kp;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -62,6 +62,100 @@ __global__ void split_rows_kernel(const double *__restrict__ src, int64_t rs, in
     const __nv_bfloat16 lo = __double2bfloat16(x - (double)__bfloat162float(hi));
     dst[r * 2 * Kp + k] = hi;
     dst[r * 2 * Kp + Kp + k] = lo;
+  }
+}
+
+// The split of a float64 value as __double2bfloat16 gives it, hi = bf16(x) and
+// lo = bf16(x - hi), to nearest even, in integer arithmetic on the mantissa
+// (the conversions and the subtraction would run on the FP64 pipe, one
+// operation per 15 clocks and warp on an SM).  Exponents far from 1, zeros,
+// infinities and NaN take the conversions.
+__device__ __forceinline__ void split_f64(double x, __nv_bfloat16 &hi, __nv_bfloat16 &lo) {
+  const long long b = __double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7FF);
+  if (e < 1023 - 64 || e > 1023 + 64) {
+    hi = __double2bfloat16(x);
+    lo = __double2bfloat16(x - (double)__bfloat162float(hi));
+    return;
+  }
+  const unsigned int sign = (unsigned int)((unsigned long long)b >> 63) << 31;
+  const long long m = (b & 0xFFFFFFFFFFFFFll) | (1ll << 52);   // |x| = m 2^(e - 1075)
+  const long long h = (m + ((1ll << 44) - 1) + ((m >> 45) & 1)) >> 45;   // 128 .. 256
+  const long long r = m - (h << 45);                           // |r| <= 2^44
+  // float32(h) 2^(e - 1030): h has 8 significant bits
+  const unsigned int fh = __float_as_uint((float)(int)h) + ((unsigned int)(e - 1030) << 23);
+  hi = __ushort_as_bfloat16((unsigned short)((fh | sign) >> 16));
+  const unsigned long long q = (unsigned long long)(r < 0 ? -r : r);
+  const int sh = max(0, 63 - __clzll((long long)(q | 1)) - 7);   // bits below the 8 kept
+  const unsigned int l = sh == 0 ? (unsigned int)q
+                                 : (unsigned int)((q + ((1ull << (sh - 1)) - 1) + ((q >> sh) & 1)) >> sh);
+  // float32(l) 2^(sh + e - 1075), zero for r = 0
+  const unsigned int fl = __float_as_uint((float)(int)l) + ((unsigned int)(sh + e - 1075) << 23);
+  lo = __ushort_as_bfloat16(
+      (unsigned short)(l == 0 ? 0u : ((fl | (r < 0 ? sign ^ 0x80000000u : sign)) >> 16)));
+}
+
+// Four consecutive entries of an operand row: split bf16 (hi at p, lo at p +
+// Kp) or tf32 floats.
+__device__ __forceinline__ void put_operand4(void *base, int64_t row, int Kp, int k, bool tf32,
+                                             const double (&x)[4]) {
+  if (tf32) {
+    *(float4 *)((float *)base + row * Kp + k) =
+        make_float4(ptx::tf32_round((float)x[0]), ptx::tf32_round((float)x[1]),
+                    ptx::tf32_round((float)x[2]), ptx::tf32_round((float)x[3]));
+    return;
+  }
+  __align__(8) __nv_bfloat16 h[4], l[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) split_f64(x[j], h[j], l[j]);
+  __nv_bfloat16 *dst = (__nv_bfloat16 *)base + row * 2 * Kp + k;
+  *(uint2 *)dst = *(const uint2 *)h;
+  *(uint2 *)(dst + Kp) = *(const uint2 *)l;
+}
+
+// The operator's input as the K product's operand, four entries per thread,
+// rows on blockIdx.y: planar rows c, or interleaved complex vectors (both
+// planes of vector s = blockIdx.y).  zero (may be NULL): float32 rows of n
+// entries cleared on the way (the output of a K product in two K halves).
+template <bool INTER>
+__global__ void __launch_bounds__(256) split_input_kernel(const double *__restrict__ Z, int rows,
+                                                          int n, int Kp, void *__restrict__ dst,
+                                                          bool tf32, float *__restrict__ zero,
+                                                          const int *__restrict__ dcnt, int mul) {
+  if (dcnt) rows = min(rows, mul * *dcnt);
+  const int k = 4 * (blockIdx.x * 256 + threadIdx.x);
+  if (k >= Kp) return;
+  for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+    if (INTER) {
+      const double2 *z = (const double2 *)Z + (int64_t)r * n + k;
+      double re[4], im[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const double2 v = k + j < n ? z[j] : make_double2(0.0, 0.0);
+        re[j] = v.x;
+        im[j] = v.y;
+      }
+      put_operand4(dst, 2 * (int64_t)r, Kp, k, tf32, re);
+      put_operand4(dst, 2 * (int64_t)r + 1, Kp, k, tf32, im);
+    } else {
+      const double *z = Z + (int64_t)r * n + k;
+      double x[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[j] = k + j < n ? z[j] : 0.0;
+      put_operand4(dst, r, Kp, k, tf32, x);
+    }
+    if (zero) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (k + j < n) {
+          if (INTER) {
+            zero[2 * (int64_t)r * n + k + j] = 0.f;
+            zero[(2 * (int64_t)r + 1) * n + k + j] = 0.f;
+          } else {
+            zero[(int64_t)r * n + k + j] = 0.f;
+          }
+        }
+    }
   }
 }
 
@@ -143,7 +237,6 @@ cudaError_t lp_autotune(cudaStream_t st, const DevSystem &sys, LpWork &lp) {
         ep.energy = sys.energy;
         ep.eocc2 = lp.eocc2;
         ep.dterm = lp.dterm;
-        ep.omega = lp.omega;
         ep.eps = 0.01;
         ep.occ_value = sys.occ_value;
         ep.n_occ = sys.n_occ;
@@ -197,21 +290,38 @@ cudaError_t lp_autotune(cudaStream_t st, const DevSystem &sys, LpWork &lp) {
   return e;
 }
 
+// Whether the K product of ncols columns adds K halves into a cleared output
+// (which the kernel that writes its operand clears).
+float *lp_cleared_output(const DevSystem &sys, const LpWork &lp, int ncols) {
+  int ks = 1, ncl = 1;
+  tc_split_plan(lp.KpK, sys.n_prod, ncols, lp.bnK, &ks, &ncl);
+  return ks > 1 ? lp.Yt : nullptr;
+}
+
 cudaError_t launch_apply_operator_lp(cudaStream_t st, const DevSystem &sys, LpWork &lp, int S,
-                                     OpMode mode, double eps, const double *Zin, double *Out) {
+                                     OpMode mode, double eps, const double *Zin, double *Out,
+                                     LpInput input, const double *omega) {
   if (S <= 0) return cudaSuccess;
   if (S > lp.slots || mode == kKernel) return cudaErrorInvalidValue;
   const int ncols = 2 * S;
   const int np = sys.n_prod;
+  const bool inter = input == kInterleaved;
+  if (!omega) omega = lp.omega;
   cudaError_t err;
   const int64_t N1 = (int64_t)ncols * sys.n_occ;
   if (N1 > INT32_MAX) return cudaErrorInvalidValue;
   TcEpilogue ep;
   if (mode == kA) {
-    {
+    if (input != kSplitDone) {
       Scope sc(lp.timer, st, kcLpSplit, 0.0);
-      split_rows_kernel<<<grid_for((int64_t)ncols * lp.KpK, 256), 256, 0, st>>>(
-          Zin, np, 1, ncols, np, lp.KpK, lp.Zb, lp.tf32, lp.dcnt, 2);
+      const dim3 grid((lp.KpK / 4 + 255) / 256, std::min(inter ? S : ncols, 32768));
+      float *zero = lp_cleared_output(sys, lp, ncols);
+      if (inter)
+        split_input_kernel<true><<<grid, 256, 0, st>>>(Zin, S, np, lp.KpK, lp.Zb, lp.tf32, zero,
+                                                       lp.dcnt, 1);
+      else
+        split_input_kernel<false><<<grid, 256, 0, st>>>(Zin, ncols, np, lp.KpK, lp.Zb, lp.tf32,
+                                                        zero, lp.dcnt, 2);
       if ((err = cudaGetLastError()) != cudaSuccess) return err;
     }
     {
@@ -219,6 +329,7 @@ cudaError_t launch_apply_operator_lp(cudaStream_t st, const DevSystem &sys, LpWo
       ep.outF = lp.Yt;
       ep.ldo = np;
       ep.split_ok = 1;
+      ep.cleared = 1;
       err = launch_gemm_tc(st, lp.opK, lp.opZ, np, ncols, kStoreF32, ep, lp.err, lp.dcnt, 2,
                            lp.bnK);
       if (err != cudaSuccess) return err;
@@ -231,7 +342,7 @@ cudaError_t launch_apply_operator_lp(cudaStream_t st, const DevSystem &sys, LpWo
   {
     Scope sc(lp.timer, st, kcAlphaGather, 0.0);
     err = launch_alpha_gather_lp(st, ar, ncols, mode == kA ? (const void *)lp.Yt : Zin,
-                                 mode != kA, np, lp.dcnt);
+                                 mode != kA, inter, np, lp.dcnt);
     if (err != cudaSuccess) return err;
   }
   {
@@ -250,7 +361,7 @@ cudaError_t launch_apply_operator_lp(cudaStream_t st, const DevSystem &sys, LpWo
   {
     Scope sc(lp.timer, st, kcDterm, 0.0);
     dterm_kernel<<<grid_for((int64_t)S * sys.n_virt, 256), 256, 0, st>>>(
-        S, sys.n_virt, sys.n_occ, sys.energy, lp.omega, lp.dterm, lp.dcnt);
+        S, sys.n_virt, sys.n_occ, sys.energy, omega, lp.dterm, lp.dcnt);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
   {
@@ -263,7 +374,6 @@ cudaError_t launch_apply_operator_lp(cudaStream_t st, const DevSystem &sys, LpWo
     e1.energy = sys.energy;
     e1.eocc2 = lp.eocc2;
     e1.dterm = lp.dterm;
-    e1.omega = lp.omega;
     e1.eps = eps;
     e1.occ_value = sys.occ_value;
     e1.n_occ = sys.n_occ;
@@ -292,13 +402,21 @@ cudaError_t launch_apply_operator_lp(cudaStream_t st, const DevSystem &sys, LpWo
     TcEpilogue e5;
     e5.outF = ar.P2f;
     e5.ldo = ar.ldp;
-    err = launch_gemm_tc_grouped(st, ar.a5, ar.gcat, ar.tiles5lp, ar.n_tiles5lp, ncols, kPartialF32,
-                                 e5, lp.err, lp.dcnt, 2);
+    // two M blocks per tile halve the reads of Gcat; where that leaves SMs
+    // without a tile, one M block and 64 columns (an output's K order is the
+    // same: same bits)
+    if ((int64_t)ar.n_tiles5lp * ((ncols + 127) / 128) >= 152)
+      err = launch_gemm_tc_grouped(st, ar.a5, ar.gcat, ar.tiles5lp, ar.n_tiles5lp, ncols,
+                                   kPartialF32, e5, lp.err, lp.dcnt, 2);
+    else
+      err = launch_gemm_tc_grouped(st, ar.a5, ar.gcat, ar.tiles5, ar.n_tiles5, ncols,
+                                   kPartialOneF32, e5, lp.err, lp.dcnt, 2, 64);
     if (err != cudaSuccess) return err;
   }
   {
     Scope sc(lp.timer, st, kcCombine, 0.0);
-    err = launch_alpha_combine(st, ar, ncols, np, false, Zin, mode == kA ? 1 : 0, Out, lp.dcnt);
+    err = launch_alpha_combine(st, ar, ncols, np, false, Zin, mode == kA ? 1 : 0, Out, lp.dcnt,
+                               inter);
     if (err != cudaSuccess) return err;
   }
   return cudaSuccess;

@@ -609,23 +609,35 @@ static tddft_status boundary_apply(tddft_ctx *c, OpMode mode, int32_t n_rhs, con
   const int np = c->sys.n_prod;
   const size_t bytes = (size_t)n_rhs * np * 2 * sizeof(double);
   cudaStream_t st = c->st;
-  if (mode != kKernel)
-    CUDA_TRY(c, cudaMemcpyAsync(c->wk.omega, omega, n_rhs * sizeof(double),
+  const bool lp = c->lowprec && mode != kKernel;
+  // the reduced-precision operator reads device frequencies where they are
+  if (mode != kKernel && !(lp && dev))
+    CUDA_TRY(c, cudaMemcpyAsync(lp ? c->lp.omega : c->wk.omega, omega, n_rhs * sizeof(double),
                                 dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
   const double *zin = z;
   if (!dev) {
     CUDA_TRY(c, cudaMemcpyAsync(c->stage, z, bytes, cudaMemcpyHostToDevice, st));
     zin = c->stage;
   }
-  CUDA_TRY(c, launch_interleaved_to_planar(st, n_rhs, np, zin, c->Zc));
-  if (c->lowprec && mode != kKernel) {
-    CUDA_TRY(c, cudaMemcpyAsync(c->lp.omega, c->wk.omega, n_rhs * sizeof(double),
-                                cudaMemcpyDeviceToDevice, st));
-    CUDA_TRY(c, launch_apply_operator_lp(st, c->sys, c->lp, n_rhs, mode, eps, c->Zc, c->Wout));
+  double *dst = dev ? out : c->stage;
+  // It also takes the interleaved vectors as they are, where complex entries
+  // are aligned and the result does not run into an input it still reads
+  // (z == out is fine: every entry is read and written by one thread).
+  const char *z0 = (const char *)zin, *o0 = (const char *)dst;
+  const bool direct = lp && (((uintptr_t)zin | (uintptr_t)dst) & 15) == 0 &&
+                      (z0 == o0 || z0 + bytes <= o0 || o0 + bytes <= z0);
+  if (direct) {
+    CUDA_TRY(c, launch_apply_operator_lp(st, c->sys, c->lp, n_rhs, mode, eps, zin, dst,
+                                         kInterleaved, dev ? omega : nullptr));
   } else {
-    CUDA_TRY(c, launch_apply_operator(st, c->sys, c->wk, n_rhs, mode, eps, c->Zc, c->Wout));
+    CUDA_TRY(c, launch_interleaved_to_planar(st, n_rhs, np, zin, c->Zc));
+    if (lp)
+      CUDA_TRY(c, launch_apply_operator_lp(st, c->sys, c->lp, n_rhs, mode, eps, c->Zc, c->Wout,
+                                           kPlanar, dev ? omega : nullptr));
+    else
+      CUDA_TRY(c, launch_apply_operator(st, c->sys, c->wk, n_rhs, mode, eps, c->Zc, c->Wout));
+    CUDA_TRY(c, launch_planar_to_interleaved(st, n_rhs, np, c->Wout, dst));
   }
-  CUDA_TRY(c, launch_planar_to_interleaved(st, n_rhs, np, c->Wout, dev ? out : c->stage));
   if (!dev) {
     CUDA_TRY(c, cudaMemcpyAsync(out, c->stage, bytes, cudaMemcpyDeviceToHost, st));
     CUDA_TRY(c, cudaStreamSynchronize(st));
@@ -750,8 +762,10 @@ static cudaError_t enqueue_iteration(tddft_ctx *c, cudaStream_t gs, int n, doubl
     e = cudaGetLastError();
   }
   if (split) {
-    if (e == cudaSuccess) e = launch_gmres_gather(gs, c->sys, g, g.act, n, c->Zc, lp.omega, g.count);
-    if (e == cudaSuccess) e = launch_apply_operator_lp(gs, c->sys, lp, n, kA, eps, c->Zc, c->Wout);
+    if (e == cudaSuccess)
+      e = launch_gmres_gather(gs, c->sys, g, g.act, n, c->Zc, lp.omega, g.count, &lp);
+    if (e == cudaSuccess)
+      e = launch_apply_operator_lp(gs, c->sys, lp, n, kA, eps, c->Zc, c->Wout, kSplitDone);
     if (e == cudaSuccess) e = launch_gmres_step(gs, c->sys, g, g.act, n, c->Wout, g.count);
     if (e == cudaSuccess)
       e = launch_gmres_gather(gs, c->sys, g, g.act2, n, c->Zc, wk.omega, g.count + 1);
@@ -926,10 +940,12 @@ static tddft_status polarizability_impl(tddft_ctx *c, int32_t n_omega, const dou
           {
             TimedLaunch tl(c->timer, st, kcGmresGather);
             CUDA_TRY(c, launch_gmres_gather(st, c->sys, g, g.act, cntA, c->Zc,
-                                            split ? c->lp.omega : c->wk.omega));
+                                            split ? c->lp.omega : c->wk.omega, nullptr,
+                                            split ? &c->lp : nullptr));
           }
           if (split)
-            CUDA_TRY(c, launch_apply_operator_lp(st, c->sys, c->lp, cntA, kA, eps, c->Zc, c->Wout));
+            CUDA_TRY(c, launch_apply_operator_lp(st, c->sys, c->lp, cntA, kA, eps, c->Zc, c->Wout,
+                                                 kSplitDone));
           else
             CUDA_TRY(c, launch_apply_operator(st, c->sys, c->wk, cntA, kA, eps, c->Zc, c->Wout));
           {
