@@ -53,6 +53,24 @@ __device__ inline double2 cdiv(double2 a, double2 b) {
   }
 }
 
+// n / d, correctly rounded, from inv = 1 / d (itself correctly rounded):
+// remainders correct the product n inv twice, first to within one unit in the
+// last place, then to the rounded quotient (Markstein, IBM J. Res. Dev. 34,
+// 1990); five dependent operations instead of a whole division.  The theorem
+// needs its products clear of under- and overflow and a denominator whose
+// significand is not all ones; others divide.
+__device__ inline double quotient(double n, double d, double inv) {
+  const unsigned en = (unsigned)(__double2hiint(n) >> 20) & 0x7FFu,
+                 ed = (unsigned)(__double2hiint(d) >> 20) & 0x7FFu;
+  const bool plain = en - 400u < 1247u && ed - 400u < 1247u &&
+                     (__double_as_longlong(d) & 0xFFFFFFFFFFFFFll) != 0xFFFFFFFFFFFFFll;
+  const int gap = (int)en - (int)ed;
+  if (!plain || gap > 500 || gap < -500) return n / d;
+  double q = n * inv;
+  q = fma(fma(-q, d, n), inv, q);
+  return fma(fma(-q, d, n), inv, q);
+}
+
 // Sum of NV values over the CTA; every thread receives the totals.
 template <int NV>
 __device__ void block_sum(double (&v)[NV], double *red /* [NV][NT/32] */) {
@@ -372,15 +390,49 @@ __device__ void cluster_sum(double (&v)[NV], double *red, double *clx) {
   cl.sync();   // clx may be reused once every CTA has read it
 }
 
+// Sum over the cluster of one value per warp (lane 0), for every thread: the
+// same additions as cluster_sum of a value that is zero on the other lanes,
+// once per CTA instead of in every warp (an FP64 instruction takes 15 clocks
+// of the SM's pipe however few lanes are live).
+template <int P>
+__device__ double cluster_warp_sum(double v, double *red, double *clx, double *bcast) {
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) t += red[w];
+    clx[0] = t;
+  }
+  if constexpr (P == 1) {
+    __syncthreads();
+    return clx[0];
+  } else {
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int rk = 0; rk < P; ++rk) t += cl.map_shared_rank(clx, rk)[0];
+      *bcast = t;
+    }
+    cl.sync();   // clx may be reused once every CTA has read it
+    return *bcast;
+  }
+}
+
 // One GMRES step of the right-hand side in slot blockIdx.y, its vectors split
 // over the P CTAs of a cluster (element range per CTA); dot products and norms
-// are reduced across the cluster through distributed shared memory.  Every
-// CTA takes the same decisions from the same totals; rank 0 writes the
+// are reduced across the cluster through distributed shared memory.  With the
+// residual rule the scalar work is done once per cluster: the coefficients'
+// rows are shared out over the CTAs, rank 0 alone rotates the column and
+// solves the triangle, and the others read its decision and solution (done by
+// every CTA it took a third of the FP64 pipe's time).  With the error
+// estimates every CTA does it all, from the same totals.  Rank 0 writes the
 // per-right-hand-side scalars.
 // EST: 0 the residual rule; 1 and 2 the error estimates (eps_P; eps_P and
 // eps_X), the latter also needing <x0|v_i>.
 template <int P, class T, int EST>
-__global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__restrict__ list,
+__global__ void __launch_bounds__(NT, 3) gmres_step_kernel(Gs G, const int *__restrict__ list,
                                                         const double *__restrict__ Wout,
                                                         const int *__restrict__ dcnt,
                                                         int h_smem) {
@@ -390,6 +442,9 @@ __global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__re
   __shared__ float2 hT[257];   // coefficients in float32 for the float32 basis
   __shared__ int finish_flag;
   __shared__ double2 s_gj;
+  __shared__ double s_tot, s_hn;
+  __shared__ float s_inv;
+  constexpr bool kOnce = P > 1 && EST == 0;   // scalar work once per cluster
   // error estimates: this step's <d|A v_j>, <d|w>, <x0|w>, |a|^2 and |rho|^2
   // of the last diagonal before and after its rotation, |g_{j+1}|, the
   // cycle's scalars read at entry, and the updated Frobenius sums
@@ -580,27 +635,64 @@ __global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__re
   } else {
     aw = win;
   }
-  for (int i = warp; i <= j; i += NT / 32) {
-    const T *vi_ = Vr + (int64_t)i * 2 * N;
-    T pr = 0, pim = 0, gr = 0, gim = 0;
-    if (vec4) {
-      // four elements per lane and load (float32 basis)
-      const float4 *v_r = (const float4 *)(vi_ + lo), *v_i = (const float4 *)(vi_ + N + lo);
-      const float4 *w_r = (const float4 *)(aw + lo), *w_i = (const float4 *)(aw + N + lo);
-      const float4 *j_r = (const float4 *)(vj + lo), *j_i = (const float4 *)(vj + N + lo);
+  if (vec4) {
+    // four elements per lane and load (float32 basis), kDotRows basis vectors
+    // at a time (warp q: q, q + 8, ...): w and v_j are loaded once for them,
+    // and their loads are in flight together (an L2 load takes about 1400
+    // clocks here; one vector at a time made this pass 40000 clocks at j = 20)
+    constexpr int kDotRows = 3;
+    const float4 *w_r = (const float4 *)(aw + lo), *w_i = (const float4 *)(aw + N + lo);
+    const float4 *j_r = (const float4 *)(vj + lo), *j_i = (const float4 *)(vj + N + lo);
+    for (int i0 = warp; i0 <= j; i0 += kDotRows * (NT / 32)) {
+      const float *vb[kDotRows];
+      float pr[kDotRows], pim[kDotRows], gr[kDotRows], gim[kDotRows];
+#pragma unroll
+      for (int t = 0; t < kDotRows; ++t) {
+        vb[t] = (const float *)(Vr + (int64_t)min(j, i0 + t * (NT / 32)) * 2 * N);
+        pr[t] = pim[t] = gr[t] = gim[t] = 0.f;
+      }
 #pragma unroll 1
       for (int q = lane; q < n4; q += 32) {
-        const float4 a = v_r[q], b = v_i[q], c = w_r[q], d = w_i[q], f = j_r[q], g = j_i[q];
-        pr = fmaf(a.x, c.x, fmaf(b.x, d.x, fmaf(a.y, c.y, fmaf(b.y, d.y,
-             fmaf(a.z, c.z, fmaf(b.z, d.z, fmaf(a.w, c.w, fmaf(b.w, d.w, pr))))))));
-        pim = fmaf(a.x, d.x, fmaf(-b.x, c.x, fmaf(a.y, d.y, fmaf(-b.y, c.y,
-              fmaf(a.z, d.z, fmaf(-b.z, c.z, fmaf(a.w, d.w, fmaf(-b.w, c.w, pim))))))));
-        gr = fmaf(a.x, f.x, fmaf(b.x, g.x, fmaf(a.y, f.y, fmaf(b.y, g.y,
-             fmaf(a.z, f.z, fmaf(b.z, g.z, fmaf(a.w, f.w, fmaf(b.w, g.w, gr))))))));
-        gim = fmaf(a.x, g.x, fmaf(-b.x, f.x, fmaf(a.y, g.y, fmaf(-b.y, f.y,
-              fmaf(a.z, g.z, fmaf(-b.z, f.z, fmaf(a.w, g.w, fmaf(-b.w, f.w, gim))))))));
+        const float4 c = w_r[q], d = w_i[q], f = j_r[q], g = j_i[q];
+        float4 va[kDotRows], vc[kDotRows];
+#pragma unroll
+        for (int t = 0; t < kDotRows; ++t) {
+          va[t] = ((const float4 *)(vb[t] + lo))[q];
+          vc[t] = ((const float4 *)(vb[t] + N + lo))[q];
+        }
+#pragma unroll
+        for (int t = 0; t < kDotRows; ++t) {
+          const float4 a = va[t], b = vc[t];
+          pr[t] = fmaf(a.x, c.x, fmaf(b.x, d.x, fmaf(a.y, c.y, fmaf(b.y, d.y,
+                  fmaf(a.z, c.z, fmaf(b.z, d.z, fmaf(a.w, c.w, fmaf(b.w, d.w, pr[t]))))))));
+          pim[t] = fmaf(a.x, d.x, fmaf(-b.x, c.x, fmaf(a.y, d.y, fmaf(-b.y, c.y,
+                   fmaf(a.z, d.z, fmaf(-b.z, c.z, fmaf(a.w, d.w, fmaf(-b.w, c.w, pim[t]))))))));
+          gr[t] = fmaf(a.x, f.x, fmaf(b.x, g.x, fmaf(a.y, f.y, fmaf(b.y, g.y,
+                  fmaf(a.z, f.z, fmaf(b.z, g.z, fmaf(a.w, f.w, fmaf(b.w, g.w, gr[t]))))))));
+          gim[t] = fmaf(a.x, g.x, fmaf(-b.x, f.x, fmaf(a.y, g.y, fmaf(-b.y, f.y,
+                   fmaf(a.z, g.z, fmaf(-b.z, f.z, fmaf(a.w, g.w, fmaf(-b.w, f.w, gim[t]))))))));
+        }
       }
-    } else {
+#pragma unroll
+      for (int t = 0; t < kDotRows; ++t) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+          pr[t] += __shfl_xor_sync(0xffffffffu, pr[t], off);
+          pim[t] += __shfl_xor_sync(0xffffffffu, pim[t], off);
+          gr[t] += __shfl_xor_sync(0xffffffffu, gr[t], off);
+          gim[t] += __shfl_xor_sync(0xffffffffu, gim[t], off);
+        }
+        const int i = i0 + t * (NT / 32);
+        if (lane == 0 && i <= j) {
+          hq[i] = make_double2((double)pr[t], (double)pim[t]);
+          gq[i] = make_double2((double)gr[t], (double)gim[t]);
+        }
+      }
+    }
+  } else {
+    for (int i = warp; i <= j; i += NT / 32) {
+      const T *vi_ = Vr + (int64_t)i * 2 * N;
+      T pr = 0, pim = 0, gr = 0, gim = 0;
 #pragma unroll 4
       for (int e = lo + lane; e < hi; e += 32) {
         const T wr = aw[e], wi = aw[N + e];
@@ -611,19 +703,19 @@ __global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__re
         gr = fma(vr, ar, fma(vi, ai, gr));
         gim = fma(vr, ai, fma(-vi, ar, gim));
       }
-    }
-    // across the warp in type T (the float32 basis: float64 shuffles would load
-    // the FP64 pipe with every vector), then float64 per warp
+      // across the warp in type T (the float32 basis: float64 shuffles would load
+      // the FP64 pipe with every vector), then float64 per warp
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      pr += __shfl_xor_sync(0xffffffffu, pr, off);
-      pim += __shfl_xor_sync(0xffffffffu, pim, off);
-      gr += __shfl_xor_sync(0xffffffffu, gr, off);
-      gim += __shfl_xor_sync(0xffffffffu, gim, off);
-    }
-    if (lane == 0) {
-      hq[i] = make_double2((double)pr, (double)pim);
-      gq[i] = make_double2((double)gr, (double)gim);
+      for (int off = 16; off > 0; off >>= 1) {
+        pr += __shfl_xor_sync(0xffffffffu, pr, off);
+        pim += __shfl_xor_sync(0xffffffffu, pim, off);
+        gr += __shfl_xor_sync(0xffffffffu, gr, off);
+        gim += __shfl_xor_sync(0xffffffffu, gim, off);
+      }
+      if (lane == 0) {
+        hq[i] = make_double2((double)pr, (double)pim);
+        gq[i] = make_double2((double)gr, (double)gim);
+      }
     }
   }
   if (P == 1) {
@@ -654,7 +746,10 @@ __global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__re
   // h_i = 2 h1_i - sum_k G_ik h1_k (warp per row i, lanes over k); column k
   // of G (entries i <= k) is stored at Gr[k (m+1) + i], column j is gp
   double2 *Gr = G.Gm + (int64_t)r * (m + 1) * (m + 1);
-  for (int i = warp; i <= j; i += NT / 32) {
+  // (rows shared out over the cluster: row i belongs to CTA (i / 8) % P, which
+  // leaves it in hq)
+  for (int i = kOnce ? rank * (NT / 32) + warp : warp; i <= j;
+       i += kOnce ? P * (NT / 32) : NT / 32) {
     double sr = 0.0, si = 0.0;
     for (int k = lane; k <= j; k += 32) {
       double2 gik;
@@ -671,7 +766,15 @@ __global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__re
       sr += __shfl_xor_sync(0xffffffffu, sr, off);
       si += __shfl_xor_sync(0xffffffffu, si, off);
     }
-    if (lane == 0) hs[i] = make_double2(2.0 * hp[i].x - sr, 2.0 * hp[i].y - si);
+    if (lane == 0)
+      (kOnce ? hq : hs)[i] = make_double2(2.0 * hp[i].x - sr, 2.0 * hp[i].y - si);
+  }
+  if constexpr (kOnce) {
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    for (int i = tid; i <= j; i += NT)
+      hs[i] = cl.map_shared_rank(hq, (i / (NT / 32)) % P)[i];
+    // (hq is rewritten only after the next cluster synchronisation)
   }
   __syncthreads();
   if (rank == 0)
@@ -784,16 +887,22 @@ __global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__re
       s_dw = make_double2(q7[3], q7[4]);
       s_xw = make_double2(q7[5], q7[6]);
     }
+  } else if (vec4) {
+    q7[0] = cluster_warp_sum<P>(q7[0], red, clx, &s_tot);   // synchronises: w complete
   } else {
     double n1[1] = {q7[0]};
     cluster_sum<P, 1>(n1, red, clx);   // synchronises: w complete
     q7[0] = n1[0];
   }
-  const double hn = sqrt(q7[0]);
+  if (tid == 0) {
+    s_hn = sqrt(q7[0]);
+    s_inv = (float)(1.0 / s_hn);
+  }
 
-  // the earlier rotations to shared memory (all threads), then thread 0
+  // the earlier rotations to shared memory (all threads), then warp 0
   // applies them to the new column in order
-  {
+  const bool scalar = !kOnce || rank == 0;   // this CTA does the scalar work
+  if (scalar) {
     const double *csg = G.cs + (int64_t)r * m;
     const double2 *sng = G.sn + (int64_t)r * m;
     for (int i = tid; i < j; i += NT) {
@@ -802,20 +911,22 @@ __global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__re
     }
   }
   __syncthreads();
-  if (tid == 0) {
-    // every CTA rotates its own copy of the new column (identical inputs)
+  const double hn = s_hn;
+  if (scalar && warp == 0) {
+    // the rotated entry is carried in registers from one rotation to the next
+    double2 a = hs[0];
+#pragma unroll 4
     for (int i = 0; i < j; ++i) {
       const double csi = gq[i].x;
-      const double2 sni = hq[i];
-      const double2 a = hs[i], bb = hs[i + 1];
+      const double2 sni = hq[i], bb = hs[i + 1];
       const double2 t = make_double2(csi * a.x + (sni.x * bb.x - sni.y * bb.y),
                                      csi * a.y + (sni.x * bb.y + sni.y * bb.x));
       const double2 cb = cmul(cconj(sni), a);
-      hs[i + 1] = make_double2(-cb.x + csi * bb.x, -cb.y + csi * bb.y);
-      hs[i] = t;
+      if (lane == 0) hs[i] = t;
+      a = make_double2(-cb.x + csi * bb.x, -cb.y + csi * bb.y);
     }
-    // new rotation mapping (hs[j], hn) to (rho, 0)
-    const double2 a = hs[j];
+    // new rotation mapping (a, hn) to (rho, 0); its three quotients, then the
+    // last two, are one division each on three lanes
     const double aa = cabs2(a);
     double c;
     double2 sv;
@@ -823,9 +934,12 @@ __global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__re
     else if (aa == 0.0) { c = 0.0; sv = make_double2(1.0, 0.0); }
     else {
       const double rr = hypot(aa, hn);
-      c = aa / rr;
-      sv = make_double2(a.x / aa * hn / rr, a.y / aa * hn / rr);
+      const double q = (lane == 0 ? a.x : (lane == 1 ? a.y : aa)) / (lane < 2 ? aa : rr);
+      const double q2 = q * hn / rr;
+      c = __shfl_sync(0xffffffffu, q, 2);
+      sv = make_double2(__shfl_sync(0xffffffffu, q2, 0), __shfl_sync(0xffffffffu, q2, 1));
     }
+    if (lane == 0) {
     hs[j] = make_double2(c * a.x + sv.x * hn, c * a.y + sv.y * hn);
     const double2 t = cmul(cconj(sv), gj0);
     const double2 gnext = make_double2(-t.x, -t.y);
@@ -844,6 +958,12 @@ __global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__re
     gq[0] = make_double2(c, 0.0);   // the new rotation, kept for the writes below
     hq[0] = sv;
     hq[1] = gnext;
+    }
+  }
+  if constexpr (kOnce) {
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    if (rank != 0 && tid == 0) finish_flag = *cl.map_shared_rank(&finish_flag, 0);
   }
   __syncthreads();
   const double c_new = gq[0].x;
@@ -966,7 +1086,7 @@ __global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__re
     }
   }
   __syncthreads();
-  if (finish_flag && !EST) {
+  if (finish_flag && !EST && scalar) {
     // back substitution R y = g (with the error estimates, ys holds y already) with the rotated (upper triangular)
     // Hessenberg matrix: its earlier columns (shared memory when they fit)
     // and g_0..g_{j-1} staged by all threads, column j and g_j from this
@@ -981,34 +1101,64 @@ __global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__re
       }
     }
     for (int i = tid; i < j; i += NT) hp[i] = gg[i];
+    // the parts of the quotients that depend on the diagonal alone (cdiv's
+    // ratio and denominator, and the denominator's reciprocal), off the chain
+    for (int i = tid; i < k; i += NT) {
+      const double2 b = (i == j) ? hs[j] : Hr[(int64_t)i * (m + 1) + i];
+      const bool wide = fabs(b.x) >= fabs(b.y);
+      const double r = wide ? b.y / b.x : b.x / b.y;
+      const double d = wide ? b.x + r * b.y : b.y + r * b.x;
+      gq[i] = make_double2(r, d);
+      gp[i] = make_double2(1.0 / d, wide ? 1.0 : 0.0);
+    }
     __syncthreads();
     const double2 *Hs = h_smem ? hdyn : Hr;
     if (warp == 0) {
+      double2 yn = make_double2(0.0, 0.0);   // lane 0: y_{i+1}
       for (int i = k - 1; i >= 0; --i) {
         double sr = 0.0, si = 0.0;
+        const int n = k - 1 - i;             // terms, on lanes 0 .. n - 1
         for (int l = i + 1 + lane; l < k; l += 32) {
           const double2 hil = (l == j) ? hs[i] : Hs[(int64_t)l * (m + 1) + i];
-          const double2 p = cmul(hil, ys[l]);
+          const double2 p = cmul(hil, l == i + 1 ? yn : ys[l]);
           sr += p.x;
           si += p.y;
         }
+        // (lanes from n on hold zeros: the wider steps would add only those)
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-          sr += __shfl_xor_sync(0xffffffffu, sr, off);
-          si += __shfl_xor_sync(0xffffffffu, si, off);
-        }
+        for (int off = 16; off > 0; off >>= 1)
+          if (off < n) {
+            sr += __shfl_xor_sync(0xffffffffu, sr, off);
+            si += __shfl_xor_sync(0xffffffffu, si, off);
+          }
         if (lane == 0) {
           const double2 gi = (i == j) ? s_gj : hp[i];
-          const double2 hii = (i == j) ? hs[j] : Hs[(int64_t)i * (m + 1) + i];
-          ys[i] = cdiv(make_double2(gi.x - sr, gi.y - si), hii);
+          const double2 a = make_double2(gi.x - sr, gi.y - si);
+          const double r = gq[i].x, d = gq[i].y, inv = gp[i].x;
+          const bool wide = gp[i].y != 0.0;
+          const double nx = wide ? a.x + a.y * r : a.x * r + a.y;
+          const double ny = wide ? a.y - a.x * r : a.y * r - a.x;
+          yn = make_double2(quotient(nx, d, inv), quotient(ny, d, inv));
+          ys[i] = yn;
         }
         __syncwarp();
       }
     }
     __syncthreads();
   }
+  if constexpr (kOnce) {
+    if (finish_flag) {
+      cg::cluster_group cl = cg::this_cluster();
+      cl.sync();
+      if (rank != 0)
+        for (int i = tid; i <= j; i += NT) ys[i] = cl.map_shared_rank(ys, 0)[i];
+      __syncthreads();
+    }
+  }
   if (!finish_flag) {
-    const T inv = (T)(1.0 / hn);
+    T inv;
+    if constexpr (sizeof(T) == 4) inv = s_inv;
+    else inv = (T)(1.0 / hn);
     if (vec4) {
       float4 *w_r = (float4 *)(w + lo), *w_i = (float4 *)(w + N + lo);
       const float fi = (float)inv;
@@ -1086,6 +1236,7 @@ __global__ void __launch_bounds__(NT, 4) gmres_step_kernel(Gs G, const int *__re
       }
     }
   }
+  if constexpr (kOnce) cg::this_cluster().sync();   // rank 0's shared memory has been read
 }
 
 // Initial guesses: x = x0 (interleaved complex rows g0..g0+n-1), and the first
