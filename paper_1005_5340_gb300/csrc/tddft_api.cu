@@ -728,9 +728,13 @@ tddft_status tddft_set_guess(tddft_ctx *c, int32_t guess) {
 // Loop control of the device-driven GMRES loop (one WHILE node per group):
 // right after the selection of each iteration, keep the node repeating while
 // some right-hand side is live and the iteration bound holds; ctl[0] counts
-// the iterations, ctl[1] = 1 records that the bound stopped the loop.
-__global__ void loop_control_kernel(cudaGraphConditionalHandle h, const int *__restrict__ count,
-                                    int *__restrict__ ctl, int max_iter) {
+// the iterations, ctl[1] = 1 records that the bound stopped the loop.  In the
+// refinement forms (resid) the IF node with the float64 residuals runs only in
+// iterations that have some.
+__global__ void loop_control_kernel(cudaGraphConditionalHandle loop,
+                                    cudaGraphConditionalHandle resid_if, int resid,
+                                    const int *__restrict__ count, int *__restrict__ ctl,
+                                    int max_iter) {
   const bool live = count[0] > 0 || count[1] > 0;
   const int it = ++ctl[0];
   bool go = live;
@@ -738,44 +742,59 @@ __global__ void loop_control_kernel(cudaGraphConditionalHandle h, const int *__r
     ctl[1] = 1;
     go = false;
   }
-  cudaGraphSetConditional(h, go ? 1u : 0u);
+  cudaGraphSetConditional(loop, go ? 1u : 0u);
+  if (resid) cudaGraphSetConditional(resid_if, count[1] > 0 ? 1u : 0u);
 }
 
+// The conditions that the loop control of a captured iteration sets.
+struct LoopHandles {
+  cudaGraphConditionalHandle loop, resid_if;
+  int max_iter;
+};
+
 // Enqueue one device-driven GMRES iteration of context c's current group of
-// n right-hand sides on stream gs (no host decision, no synchronisation).
-// With loop: the body of a WHILE node, whose condition the control kernel
-// sets after the selection (the rest of the iteration then finds no live
-// right-hand side and does no work).
-static cudaError_t enqueue_iteration(tddft_ctx *c, cudaStream_t gs, int n, double eps, int split,
-                                     int min_b, const cudaGraphConditionalHandle *loop = nullptr,
-                                     int max_iter = 0) {
+// n right-hand sides on stream gs (no host decision, no synchronisation): the
+// selection and the Arnoldi steps, and, in the refinement forms (split), the
+// float64 residuals, apart.  With loop: the body of a WHILE node, whose
+// conditions the control kernel sets after the selection (the rest of a last
+// iteration then finds no live right-hand side and does no work).
+static cudaError_t enqueue_arnoldi(tddft_ctx *c, cudaStream_t gs, int n, double eps, int split,
+                                   int min_b, const LoopHandles *loop = nullptr) {
   GmresState &g = c->gs;
-  OpWork wk = c->wk;
-  LpWork lp = c->lp;
-  wk.timer = nullptr;
-  lp.timer = nullptr;
-  wk.dcnt = g.count + (split ? 1 : 0);
-  lp.dcnt = g.count;
   cudaError_t e = launch_gmres_select(gs, g, n, split, min_b);
   if (e == cudaSuccess && loop) {
-    loop_control_kernel<<<1, 1, 0, gs>>>(*loop, g.count, g.loopctl, max_iter);
+    loop_control_kernel<<<1, 1, 0, gs>>>(loop->loop, loop->resid_if, split, g.count, g.loopctl,
+                                         loop->max_iter);
     e = cudaGetLastError();
   }
   if (split) {
+    LpWork lp = c->lp;
+    lp.timer = nullptr;
+    lp.dcnt = g.count;
     if (e == cudaSuccess)
       e = launch_gmres_gather(gs, c->sys, g, g.act, n, c->Zc, lp.omega, g.count, &lp);
     if (e == cudaSuccess)
       e = launch_apply_operator_lp(gs, c->sys, lp, n, kA, eps, c->Zc, c->Wout, kSplitDone);
-    if (e == cudaSuccess) e = launch_gmres_step(gs, c->sys, g, g.act, n, c->Wout, g.count);
-    if (e == cudaSuccess)
-      e = launch_gmres_gather(gs, c->sys, g, g.act2, n, c->Zc, wk.omega, g.count + 1);
-    if (e == cudaSuccess) e = launch_apply_operator(gs, c->sys, wk, n, kA, eps, c->Zc, c->Wout);
-    if (e == cudaSuccess) e = launch_gmres_step(gs, c->sys, g, g.act2, n, c->Wout, g.count + 1);
   } else {
-    if (e == cudaSuccess) e = launch_gmres_gather(gs, c->sys, g, g.act, n, c->Zc, wk.omega, g.count);
+    OpWork wk = c->wk;
+    wk.timer = nullptr;
+    wk.dcnt = g.count;
+    if (e == cudaSuccess)
+      e = launch_gmres_gather(gs, c->sys, g, g.act, n, c->Zc, wk.omega, g.count);
     if (e == cudaSuccess) e = launch_apply_operator(gs, c->sys, wk, n, kA, eps, c->Zc, c->Wout);
-    if (e == cudaSuccess) e = launch_gmres_step(gs, c->sys, g, g.act, n, c->Wout, g.count);
   }
+  if (e == cudaSuccess) e = launch_gmres_step(gs, c->sys, g, g.act, n, c->Wout, g.count);
+  return e;
+}
+
+static cudaError_t enqueue_residuals(tddft_ctx *c, cudaStream_t gs, int n, double eps) {
+  GmresState &g = c->gs;
+  OpWork wk = c->wk;
+  wk.timer = nullptr;
+  wk.dcnt = g.count + 1;
+  cudaError_t e = launch_gmres_gather(gs, c->sys, g, g.act2, n, c->Zc, wk.omega, g.count + 1);
+  if (e == cudaSuccess) e = launch_apply_operator(gs, c->sys, wk, n, kA, eps, c->Zc, c->Wout);
+  if (e == cudaSuccess) e = launch_gmres_step(gs, c->sys, g, g.act2, n, c->Wout, g.count + 1);
   return e;
 }
 
@@ -786,27 +805,59 @@ static int residual_batch(int split, int n) {
   return split ? std::max(1, std::min(64, n / 3)) : 1;
 }
 
-// Add to graph `parent` a WHILE node (no dependencies) whose body, captured
-// on stream cs, is one device-driven GMRES iteration of context c's group.
-static cudaError_t add_device_loop(tddft_ctx *c, cudaGraph_t parent, cudaStream_t cs, int n,
-                                   double eps, int split, int min_b, int max_iter) {
-  cudaGraphConditionalHandle h;
-  cudaError_t e = cudaGraphConditionalHandleCreate(&h, parent, 1, cudaGraphCondAssignDefault);
-  if (e != cudaSuccess) return e;
+// Add a conditional node to `parent` after the nodes deps; *body receives its
+// (empty) graph.
+static cudaError_t add_conditional(cudaGraph_t parent, cudaGraphConditionalHandle h,
+                                   cudaGraphConditionalNodeType type,
+                                   const std::vector<cudaGraphNode_t> &deps, cudaGraph_t *body) {
   cudaGraphNodeParams p = {};
   p.type = cudaGraphNodeTypeConditional;
   p.conditional.handle = h;
-  p.conditional.type = cudaGraphCondTypeWhile;
+  p.conditional.type = type;
   p.conditional.size = 1;
   cudaGraphNode_t node;
-  e = cudaGraphAddNode(&node, parent, nullptr, nullptr, 0, &p);
+  const cudaError_t e =
+      cudaGraphAddNode(&node, parent, deps.empty() ? nullptr : deps.data(), nullptr, deps.size(), &p);
+  if (e == cudaSuccess) *body = p.conditional.phGraph_out[0];
+  return e;
+}
+
+// Add to graph `parent` a WHILE node (no dependencies) whose body, captured
+// on stream cs, is one device-driven GMRES iteration of context c's group; in
+// the refinement forms the float64 residuals are an IF node at its end (empty
+// launches of their twenty kernels took 35 us of an iteration of 140 us on 10
+// atoms).
+static cudaError_t add_device_loop(tddft_ctx *c, cudaGraph_t parent, cudaStream_t cs, int n,
+                                   double eps, int split, int min_b, int max_iter) {
+  LoopHandles h = {};
+  h.max_iter = max_iter;
+  cudaGraph_t body = nullptr, resid = nullptr, captured = nullptr;
+  cudaError_t e = cudaGraphConditionalHandleCreate(&h.loop, parent, 1, cudaGraphCondAssignDefault);
+  if (e == cudaSuccess) e = add_conditional(parent, h.loop, cudaGraphCondTypeWhile, {}, &body);
+  if (e == cudaSuccess && split)
+    e = cudaGraphConditionalHandleCreate(&h.resid_if, body, 0, cudaGraphCondAssignDefault);
+  if (e == cudaSuccess)
+    e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
-  cudaGraph_t body = p.conditional.phGraph_out[0];
-  e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+  cudaError_t e1 = enqueue_arnoldi(c, cs, n, eps, split, min_b, &h);
+  std::vector<cudaGraphNode_t> last;   // what the iteration's end depends on
+  if (e1 == cudaSuccess && split) {
+    cudaStreamCaptureStatus status;
+    const cudaGraphNode_t *deps = nullptr;
+    const cudaGraphEdgeData *edges = nullptr;
+    size_t nd = 0;
+    e1 = cudaStreamGetCaptureInfo(cs, &status, nullptr, nullptr, &deps, &edges, &nd);
+    if (e1 == cudaSuccess) last.assign(deps, deps + nd);
+  }
+  cudaError_t e2 = cudaStreamEndCapture(cs, &captured);
+  if (e1 != cudaSuccess || e2 != cudaSuccess) return e1 != cudaSuccess ? e1 : e2;
+  if (!split) return cudaSuccess;
+  e = add_conditional(body, h.resid_if, cudaGraphCondTypeIf, last, &resid);
+  if (e == cudaSuccess)
+    e = cudaStreamBeginCaptureToGraph(cs, resid, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
-  const cudaError_t e1 = enqueue_iteration(c, cs, n, eps, split, min_b, &h, max_iter);
-  cudaGraph_t captured = nullptr;
-  const cudaError_t e2 = cudaStreamEndCapture(cs, &captured);
+  e1 = enqueue_residuals(c, cs, n, eps);
+  e2 = cudaStreamEndCapture(cs, &captured);
   return e1 != cudaSuccess ? e1 : e2;
 }
 
@@ -851,7 +902,8 @@ static tddft_status run_group_graph(tddft_ctx *c, int n, double eps, int split, 
     ~Cleanup() { if (e) cudaGraphExecDestroy(e); if (g) cudaGraphDestroy(g); }
   } cleanup{graph, exec};
   CUDA_TRY(c, cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal));
-  cudaError_t e = enqueue_iteration(c, gs, n, eps, split, min_b);
+  cudaError_t e = enqueue_arnoldi(c, gs, n, eps, split, min_b);
+  if (e == cudaSuccess && split) e = enqueue_residuals(c, gs, n, eps);
   cudaError_t e2 = cudaStreamEndCapture(gs, &graph);
   if (e != cudaSuccess || e2 != cudaSuccess)
     return fail(c, TDDFT_ERR_CUDA, std::string("graph capture failed: ") +
