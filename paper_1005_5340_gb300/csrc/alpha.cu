@@ -267,7 +267,7 @@ cudaError_t alpha_setup(cudaStream_t st, const tddft_system *h, const DevSystem 
   ar.kcat2 = std::max((int)lcat.size(), 64);
   while ((int)lcat.size() < ar.kcat2) lcat.push_back(-1);
   ar.kcat5 = kcat5;
-  ar.ldp = round_up(2 * std::max(slots, 3), 4);   // rows of 16-byte stores
+  ar.ldp = round_up(2 * std::max(slots, 3), 8);   // rows of 32-byte stores
   // tiles (128 rows of the per-atom operands), atom by atom
   std::vector<GTile> t2, t5, t5lp;   // t5lp: 256-row entries (two M blocks per tile)
   ar.flops2 = ar.flops5 = 0.0;

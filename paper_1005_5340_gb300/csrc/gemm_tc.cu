@@ -104,6 +104,22 @@ __device__ __forceinline__ void put_operand(void *base, int64_t idx, int64_t lo_
     store_split((__nv_bfloat16 *)base + idx, lo_off, x);
 }
 
+// 32 bytes by one store (one full L2 sector per lane); dst 32-byte aligned
+__device__ __forceinline__ void store32(void *dst, const uint32_t (&r)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+
+// two neighbours' (hi, lo) planes, packed
+__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t &hi, uint32_t &lo) {
+  __nv_bfloat162 h, l;
+  split_bf16(x0, h.x, l.x);
+  split_bf16(x1, h.y, l.y);
+  hi = *(const uint32_t *)&h;
+  lo = *(const uint32_t *)&l;
+}
+
 // One 16-column chunk of the epilogue: row m (local row lr of the tile),
 // columns n0 + j0 .. n0 + j0 + 15, fused per use.
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -121,6 +137,23 @@ struct EpiIn {
   const float2 *eocc;
   int64_t xo;
 };
+
+// Transform 2, n_occ a multiple of 16: the 32 columns from n on are 16 states of
+// one slot and both planes p; one sector per lane, plane and half of the split.
+__device__ __forceinline__ void store_states16(const float (&v)[32], int n, const TcEpilogue &ep,
+                                               int64_t xo) {
+  const int pair0 = n >> 1, sl = pair0 / ep.n_occ, E0 = pair0 - sl * ep.n_occ;
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    uint32_t h[8], l[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) split_pair(v[4 * e + p], v[4 * e + 2 + p], h[e], l[e]);
+    __nv_bfloat16 *dst =
+        (__nv_bfloat16 *)ep.outB + (int64_t)(2 * sl + p) * ep.ldo + xo + E0;
+    store32(dst, h);
+    store32(dst + ep.lo_off, l);
+  }
+}
 
 template <int EPI, bool TF>
 __device__ __forceinline__ void epilogue16(const float (&v)[16], int m, int lr, int rows_valid,
@@ -146,10 +179,20 @@ __device__ __forceinline__ void epilogue16(const float (&v)[16], int m, int lr, 
   } else if (EPI == kPartialF32 || EPI == kPartialOneF32) {
     // C layout, rows of the grouped operand
     if (lr < rows_valid && (ep.ldo & 3) == 0 && n0 + j0 + 16 <= N) {
-      float4 *dst = (float4 *)(ep.outF + (int64_t)m * ep.ldo + n0 + j0);
+      float *dst = ep.outF + (int64_t)m * ep.ldo + n0 + j0;
+      if ((ep.ldo & 7) == 0) {   // (outF is an allocation's start, n0 + j0 a multiple of 16)
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        for (int j = 0; j < 16; j += 8) {
+          uint32_t r[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) r[i] = __float_as_uint(v[j + i]);
+          store32(dst + j, r);
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          ((float4 *)dst)[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+      }
     } else if (lr < rows_valid) {
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
@@ -336,7 +379,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // tile t: M tile fastest, then the K slice (split K), then the N tile of
   // tn columns (the small A of the transforms stays in L2 while each B tile
-  // is read once); in a cluster launch (ep.ncl > 1) and in a grouped product
+  // is read once); in the K product (ep.n_fast) and in a grouped product
   // (per-atom A operands, the large operand of steps 2 and 5) the N tile is
   // fastest, so consecutive CTAs (in a cluster: one GPC, one L2 partition)
   // read the same A tile, which DRAM then supplies once;
@@ -359,7 +402,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       return;
     }
     int mt, ks, nt;
-    if (ep.ncl > 1 || tiles) {
+    if (ep.n_fast || tiles) {
       nt = t % n_ntiles;
       const int rest = t / n_ntiles;
       mt = rest % n_mtiles;
@@ -633,14 +676,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 dst[c] = make_float4(tf32_round(v[4 * c][e]), tf32_round(v[4 * c + 1][e]),
                                      tf32_round(v[4 * c + 2][e]), tf32_round(v[4 * c + 3][e]));
             } else {
-              __align__(16) __nv_bfloat16 hh[16], ll[16];
+              uint32_t hh[8], ll[8];
 #pragma unroll
-              for (int c = 0; c < 16; ++c) split_bf16(v[c][e], hh[c], ll[c]);
+              for (int c = 0; c < 8; ++c) split_pair(v[2 * c][e], v[2 * c + 1][e], hh[c], ll[c]);
               __nv_bfloat16 *dst = (__nv_bfloat16 *)ep.outB + at;
-              *(uint4 *)dst = *(const uint4 *)hh;
-              *(uint4 *)(dst + 8) = *(const uint4 *)(hh + 8);
-              *(uint4 *)(dst + ep.lo_off) = *(const uint4 *)ll;
-              *(uint4 *)(dst + ep.lo_off + 8) = *(const uint4 *)(ll + 8);
+              store32(dst, hh);
+              store32(dst + ep.lo_off, ll);
             }
           }
         }
@@ -652,7 +693,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         di.xo = ep.xoff5[B] + (int64_t)b * ep.n_occ;
       }
       const int hs = EPI == kDscaleSplit ? max(1, N / (2 * ep.n_occ)) : 1;   // live slots
-      for (int j0 = j_lo; j0 < j_hi && !kPart; j0 += 16) {
+      int j_from = j_lo;
+      if (EPI == kGammaCatSplit && !TF) {
+        // 32 columns at a time where they are 16 states of one slot
+        if (ep.n_occ % 16 == 0 && ((n0 + j_lo) & 31) == 0) {
+          for (; j_from + 32 <= j_hi && n0 + j_from + 32 <= N; j_from += 32) {
+            float v[32];
+            tmem_ld32(trow + (uint32_t)j_from, v);
+            if (m < M) store_states16(v, n0 + j_from, ep, di.xo);
+          }
+        }
+      }
+      for (int j0 = j_from; j0 < j_hi && !kPart; j0 += 16) {
         if (EPI == kDscaleSplit) {
           int sl = ((n0 + j0) >> 1) % hs;   // E-major columns: consecutive slots
 #pragma unroll
@@ -800,15 +852,18 @@ int sm_count() {
 }
 
 template <int EPI, int BN, bool TF>
-cudaError_t launch_tc(cudaStream_t st, int grid, const CUtensorMap &mA, const CUtensorMap &mB,
+cudaError_t launch_tc(cudaStream_t st, int64_t work, const CUtensorMap &mA, const CUtensorMap &mB,
                       const CUtensorMap &mB64, const CUtensorMap &mB128, int M, int N, int KpA,
                       int KpB, const TcEpilogue &ep, int *err, const int *dcnt, int mul_n,
                       const GTile *tiles, int n_mtiles) {
-  if (ep.ncl <= 1) {
+  // persistent: one CTA per SM at most, each walking its share of the tiles
+  const int sms = sm_count(), grid = (int)std::min<int64_t>(work, sms);
+  auto plain = [&]() {
     gemm_tc_kernel<EPI, BN, TF><<<grid, TC_THREADS, TcCfg<EPI, BN>::SMEM, st>>>(
         mA, mB, mB64, mB128, M, N, KpA, KpB, ep, err, dcnt, mul_n, tiles, n_mtiles);
     return cudaGetLastError();
-  }
+  };
+  if (ep.ncl <= 1) return plain();
   // clusters of ncl CTAs; the grid is at most the clusters that fit at once
   // (a persistent CTA that waited for a slot would run its tiles last)
   cudaLaunchConfig_t cfg = {};
@@ -832,6 +887,13 @@ cudaError_t launch_tc(cudaStream_t st, int grid, const CUtensorMap &mA, const CU
       return cudaErrorInvalidConfiguration;
     fit[ep.ncl] = n;
   }
+  // Clusters of 3 or 4 leave SMs without one (46 and 36 clusters fit on 152
+  // SMs): where that costs a fifth more waves or above, single CTAs in the
+  // same tile order instead.  64 atoms, 384 columns: 142 clusters, 4 waves
+  // against 3, 160 us against 127; 128 atoms: 7 against 6, 702 us against 710
+  // (without the cluster an A tile is fetched by both dies).
+  const int64_t wc = (work / ep.ncl + fit[ep.ncl] - 1) / fit[ep.ncl], wp = (work + sms - 1) / sms;
+  if (5 * wp <= 4 * wc) return plain();
   cfg.gridDim = dim3(std::min(grid / ep.ncl, fit[ep.ncl]) * ep.ncl);
   return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<EPI, BN, TF>, mA, mB, mB64, mB128, M, N, KpA, KpB,
                             ep, err, dcnt, mul_n, tiles, n_mtiles);
@@ -842,29 +904,27 @@ cudaError_t launch_tc_epi(cudaStream_t st, int epi, int M, int N, const CUtensor
                           const CUtensorMap &mB, const CUtensorMap &mB64, const CUtensorMap &mB128,
                           int KpA, int KpB, const TcEpilogue &ep, int *err,
                           const int *dcnt, int mul_n, const GTile *tiles, int n_mtiles) {
-  // persistent: one CTA per SM at most, each walking its share of the tiles
   const int64_t n_tiles = epi == kBetaPartSplit
                               ? (int64_t)n_mtiles * ((M + TC_BM - 1) / TC_BM)
                               : (int64_t)n_mtiles * ((N + BN - 1) / BN) * ep.ksplit;
-  const int grid = (int)std::min<int64_t>(n_tiles, sm_count());
   switch (epi) {
     case kStoreF32:
-      return launch_tc<kStoreF32, BN, TF>(st, grid, mA, mB, mB64, mB128, M, N, KpA, KpB, ep, err,
+      return launch_tc<kStoreF32, BN, TF>(st, n_tiles, mA, mB, mB64, mB128, M, N, KpA, KpB, ep, err,
                                     dcnt, mul_n, tiles, n_mtiles);
     case kDscaleSplit:
-      return launch_tc<kDscaleSplit, BN, TF>(st, grid, mA, mB, mB64, mB128, M, N, KpA, KpB, ep, err,
+      return launch_tc<kDscaleSplit, BN, TF>(st, n_tiles, mA, mB, mB64, mB128, M, N, KpA, KpB, ep, err,
                                     dcnt, mul_n, tiles, n_mtiles);
     case kBetaPartSplit:
-      return launch_tc<kBetaPartSplit, BN, TF>(st, grid, mA, mB, mB64, mB128, M, N, KpA, KpB, ep,
+      return launch_tc<kBetaPartSplit, BN, TF>(st, n_tiles, mA, mB, mB64, mB128, M, N, KpA, KpB, ep,
                                                err, dcnt, mul_n, tiles, n_mtiles);
     case kGammaCatSplit:
-      return launch_tc<kGammaCatSplit, BN, TF>(st, grid, mA, mB, mB64, mB128, M, N, KpA, KpB, ep,
+      return launch_tc<kGammaCatSplit, BN, TF>(st, n_tiles, mA, mB, mB64, mB128, M, N, KpA, KpB, ep,
                                                err, dcnt, mul_n, tiles, n_mtiles);
     case kPartialF32:
-      return launch_tc<kPartialF32, BN, TF>(st, grid, mA, mB, mB64, mB128, M, N, KpA, KpB, ep, err,
+      return launch_tc<kPartialF32, BN, TF>(st, n_tiles, mA, mB, mB64, mB128, M, N, KpA, KpB, ep, err,
                                     dcnt, mul_n, tiles, n_mtiles);
     case kPartialOneF32:
-      return launch_tc<kPartialOneF32, BN, TF>(st, grid, mA, mB, mB64, mB128, M, N, KpA, KpB, ep,
+      return launch_tc<kPartialOneF32, BN, TF>(st, n_tiles, mA, mB, mB64, mB128, M, N, KpA, KpB, ep,
                                                err, dcnt, mul_n, tiles, n_mtiles);
     default:
       return cudaErrorInvalidValue;
@@ -921,6 +981,7 @@ cudaError_t launch_gemm_tc(cudaStream_t st, const TcOperand &A, const TcOperand 
   e.ksplit = 1;
   if (epi == kStoreF32 && ep.split_ok) {
     tc_split_plan(A.Kp, M, N, bn, &e.ksplit, &e.ncl);
+    e.n_fast = e.ncl > 1;
     if (e.ksplit > 1 && !ep.cleared) {
       cudaError_t r = cudaMemsetAsync(ep.outF, 0, (size_t)N * ep.ldo * sizeof(float), st);
       if (r != cudaSuccess) return r;

@@ -174,6 +174,7 @@ struct TcEpilogue {
   int cleared = 0;                 // kStoreF32: the caller has cleared outF for that
   int ksplit = 1;                  // set by the launcher
   int ncl = 1;                     // set by the launcher: > 1, clusters of ncl CTAs, one per N tile
+  int n_fast = 0;                  // set by the launcher: the N tile runs fastest
   const int *aoff = nullptr;       // kGammaCatSplit
   const int *orb_atom = nullptr;   // kGammaCatSplit
   const int *xoff5 = nullptr;      // kGammaCatSplit
