@@ -62,12 +62,20 @@ constexpr uint32_t OZ_A_BYTES = OZ_BM * OZ_BK * 2;   // 16 KB
 // its A tile from shared memory whatever its N, and the operand reads bound
 // it, so a wide tile does more per read and a narrow one pads less.
 // 9 stages of 24 KB, or 8 of 26 or 28 KB.
-template <int BN> struct OzShape {
+template <int S, int BN> struct OzShape {
   static constexpr int EPI_COLS = BN / 2;                      // columns per epilogue thread
   static constexpr uint32_t B_BYTES = BN * OZ_BK * 2;
-  static constexpr uint32_t STAGE_BYTES = OZ_A_BYTES + B_BYTES;
-  static constexpr int STAGES = BN == 64 ? 9 : 8;
-  static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + 256;
+  static constexpr int BS = 2 * S;                             // B slices: two K blocks
+  static constexpr int AS_FIT = (int)((227 * 1024 - 1024 - 1024 - BS * B_BYTES) / OZ_A_BYTES);
+  static constexpr int AS = AS_FIT < 9 ? AS_FIT : 9;           // A slices
+  static constexpr uint32_t A_OFF = BS * B_BYTES;
+  static constexpr size_t SMEM = A_OFF + (size_t)AS * OZ_A_BYTES + 1024 + 512;
+  // groups that one MMA takes, and the phases of a K block (see the issuer)
+  static constexpr int W = 256 / BN < S ? 256 / BN : S, NP = (S + W - 1) / W;
+  __host__ __device__ static constexpr int gh(int p) { return S - 1 - (NP - 1 - p) * W; }   // last group of phase p
+  __host__ __device__ static constexpr int gl(int p) { return p == 0 ? 0 : gh(p - 1) + 1; }
+  // A slices held while a phase before the last runs; the last one frees them
+  static_assert(NP < 2 || AS > S - 1 - W, "A ring too short");
 };
 __host__ __device__ constexpr int oz_wide_bn(int S) {
   return S * 96 <= 512 ? 96 : (S * 80 <= 512 ? 80 : 64);
@@ -128,7 +136,7 @@ __device__ __forceinline__ void add_group(long long (&acc)[EC], const float *v, 
 // 40 columns of an 80-wide group's half are five 8-column loads.
 template <int S, int BN>
 __device__ __forceinline__ void read_groups(uint32_t tcol, int h,
-                                            long long (&acc)[OzShape<BN>::EPI_COLS], int ns,
+                                            long long (&acc)[OzShape<S, BN>::EPI_COLS], int ns,
                                             int drop, uint64_t *tempty) {
 #pragma unroll 1
   for (int grp = 0; grp < ns; ++grp) {
@@ -151,7 +159,7 @@ __device__ __forceinline__ void read_groups(uint32_t tcol, int h,
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(&tempty[grp]);
     if constexpr (BN == 64 || BN == 80) {
-      add_group<OzShape<BN>::EPI_COLS>(acc, v, 0, sh);
+      add_group<OzShape<S, BN>::EPI_COLS>(acc, v, 0, sh);
     } else if (h == 0) {
       add_group<32>(acc, v, 0, sh);
       add_group<16>(acc, u, 32, sh);
@@ -191,9 +199,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                       const __grid_constant__ CUtensorMap mapB, OzArgs a) {
   int N = a.N;
   if (a.dcnt) N = (int)min((int64_t)N, (int64_t)a.mul_n * (*a.dcnt));
-  constexpr int OZ_STAGES = OzShape<BN>::STAGES;
-  constexpr uint32_t OZ_STAGE_BYTES = OzShape<BN>::STAGE_BYTES;
-  constexpr int OZ_EPI_COLS = OzShape<BN>::EPI_COLS;
+  using Shape = OzShape<S, BN>;
+  constexpr int AS = Shape::AS, BS = Shape::BS;
+  constexpr int OZ_EPI_COLS = Shape::EPI_COLS;
   // Persistent: CTA b walks tiles t = b, b + gridDim.x, ...  Tile t -> (mt,
   // nt) in an L2-aware order: the M tiles (rows of A, or entries of the tile
   // table) in groups of a.mgroup (A panels that fit in L2 together), every N
@@ -241,9 +249,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   };
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t *full = (uint64_t *)(smem + OZ_STAGES * OZ_STAGE_BYTES);
-  uint64_t *empty = full + OZ_STAGES;
-  uint64_t *tfull = empty + OZ_STAGES;
+  uint64_t *full_a = (uint64_t *)(smem + Shape::A_OFF + AS * OZ_A_BYTES);
+  uint64_t *empty_a = full_a + AS;
+  uint64_t *full_b = empty_a + AS;
+  uint64_t *empty_b = full_b + BS;
+  uint64_t *tfull = empty_b + BS;
   uint64_t *tempty = tfull + 1;   // [kOzMaxSlices] one per TMEM group
   uint64_t *drain = tempty + kOzMaxSlices;   // completion of every MMA this CTA issued
   uint32_t *tslot = (uint32_t *)(drain + 1);
@@ -256,9 +266,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   constexpr uint32_t tcols = S * BN <= 256 ? 256u : 512u;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < OZ_STAGES; ++i) {
-      mbar_init(&full[i], 1);
-      mbar_init(&empty[i], 1);
+    for (int i = 0; i < AS; ++i) {
+      mbar_init(&full_a[i], 1);
+      mbar_init(&empty_a[i], 1);
+    }
+    for (int i = 0; i < BS; ++i) {
+      mbar_init(&full_b[i], 1);
+      mbar_init(&empty_b[i], 1);
     }
     mbar_init(tfull, 1);
     for (int q = 0; q < kOzMaxSlices; ++q)
@@ -280,121 +294,126 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 
   if (warp == 0) {
     if (lane == 0) {
-      // producer: stage g = (kb * s + i) counted over this CTA's tiles holds
-      // slice i of K block kb
-      int g = 0;
+      // producer: the A slices go round a ring of AS tiles, the B slices
+      // round two K blocks.  Of a K block: what the first phase needs, A and
+      // B in turn, then the other B slices, then the other A slices (the last
+      // phase frees A slices from its first step on, which needs every B).
+      int ga = 0, gb = 0;   // slices issued
       bool ok = true;
+      auto load = [&](uint64_t *full, uint64_t *empty, int &g, int n, uint32_t bytes, uint8_t *base,
+                      const CUtensorMap *map, int x, int y) {
+        const int slot = g % n;
+        const uint32_t ph = (uint32_t)(g / n) & 1u;
+        if (!mbar_wait(&empty[slot], ph ^ 1u, lim)) {
+          atomicExch(a.err, 21);
+          abort_flag = 1;
+          return false;
+        }
+        if (*(volatile int *)&abort_flag) return false;
+        mbar_expect_tx(&full[slot], bytes);
+        tma_load_2d(base + slot * bytes, map, &full[slot], x, y);
+        ++g;
+        return true;
+      };
       for (int t = tile0; t < n_tiles && ok; t += tstep) {
         Tile T;
         if (!tile_of(t, T)) continue;
         for (int kb = 0; kb < T.nkb && ok; ++kb) {
-          for (int i = 0; i < s; ++i, ++g) {
-            const int slot = g % OZ_STAGES;
-            const uint32_t ph = (uint32_t)(g / OZ_STAGES) & 1u;
-            if (!mbar_wait(&empty[slot], ph ^ 1u, lim)) {
-              atomicExch(a.err, 21);
-              abort_flag = 1;
-              ok = false;
-              break;
-            }
-            if (*(volatile int *)&abort_flag) {
-              ok = false;
-              break;
-            }
-            uint8_t *sa = smem + slot * OZ_STAGE_BYTES;
-            mbar_expect_tx(&full[slot], OZ_STAGE_BYTES);
-            const int kx = (T.kb0 + kb) * OZ_BK;
-            tma_load_2d(sa, &mapA, &full[slot], i * a.KpA + kx, T.m0);
-            tma_load_2d(sa + OZ_A_BYTES, &mapB, &full[slot], i * a.KpB + T.xoff + kx, T.n0);
+          const int kx = (T.kb0 + kb) * OZ_BK;
+          auto load_a = [&](int i) {
+            ok = ok && load(full_a, empty_a, ga, AS, OZ_A_BYTES, smem + Shape::A_OFF, &mapA,
+                            i * a.KpA + kx, T.m0);
+          };
+          auto load_b = [&](int i) {
+            ok = ok && load(full_b, empty_b, gb, BS, Shape::B_BYTES, smem, &mapB,
+                            i * a.KpB + T.xoff + kx, T.n0);
+          };
+          for (int i = 0; i <= Shape::gh(0); ++i) {
+            load_a(i);
+            load_b(i);
           }
+          for (int i = Shape::gh(0) + 1; i < S; ++i) load_b(i);
+          for (int i = Shape::gh(0) + 1; i < S; ++i) load_a(i);
         }
       }
-      // copies in flight: the last OZ_STAGES stages issued (each the latest
-      // use of its slot) must have landed before the CTA may exit
-      for (int h = max(0, g - OZ_STAGES); h < g; ++h)
-        mbar_wait(&full[h % OZ_STAGES], (uint32_t)(h / OZ_STAGES) & 1u);
+      // copies in flight: the latest use of every slot must have landed
+      // before the CTA may exit
+      for (int h = max(0, ga - AS); h < ga; ++h) mbar_wait(&full_a[h % AS], (uint32_t)(h / AS) & 1u);
+      for (int h = max(0, gb - BS); h < gb; ++h) mbar_wait(&full_b[h % BS], (uint32_t)(h / BS) & 1u);
     }
     __syncwarp();
   } else if (warp == 1) {
-    // the whole warp runs the schedule; the elected lane issues
-    constexpr uint32_t idesc = idesc_bf16(OZ_BM, BN);
+    // The whole warp runs the schedule; the elected lane issues.  Slice A_i
+    // against neighbouring B slices is one MMA: the B tiles of a K block lie
+    // one after the other (rows of one operand), and the groups i + j of
+    // neighbouring j are neighbouring TMEM columns.  Up to W groups (256
+    // columns) at a time, in phases of groups gl .. gh: A_i x B_j, j from
+    // gl - i (or 0) to gh - i, for i = 0 .. gh; i = 0 touches every group of the phase
+    // first.  Exact integer sums: any order gives the same bits.
     const uint32_t leader = elect_one();
     const uint32_t lo0 = desc_lo(smem_u32(smem));
-    int slot0 = 0;        // ring slot and phase of the K block's slice 0
-    uint32_t phase0 = 0;
-    int gc = 0;   // chunks issued by this CTA (over its tiles)
+    int a0 = 0;            // A ring slot and phase of the K block's slice 0
+    uint32_t pa0 = 0;
+    int bc = 0;            // K blocks issued (the B half is bc & 1)
+    int gc = 0;            // chunks issued by this CTA (over its tiles)
     bool ok = true;
+    auto wait_for = [&](uint64_t *bar, uint32_t ph, int code) {
+      if (ok && !warp_wait(bar, ph, lim)) {
+        if (lane == 0) atomicExch(a.err, code);
+        abort_flag = 1;
+        ok = false;
+      }
+    };
     for (int t = tile0; t < n_tiles && ok; t += tstep) {
       Tile T;
       if (!tile_of(t, T)) continue;
       const int nchunks = (T.nkb + cb - 1) / cb;
       for (int c = 0; c < nchunks && ok; ++c, ++gc) {
         const int kb1 = min(T.nkb, (c + 1) * cb);
-        for (int kb = c * cb; kb < kb1 && ok; ++kb) {
+        for (int kb = c * cb; kb < kb1 && ok; ++kb, ++bc) {
           const bool first_kb = kb == c * cb;
-          // slot of slice i, and the descriptor words of its A and B tiles
-          auto slot_of = [&](int i) {
-            return slot0 + i >= OZ_STAGES ? slot0 + i - OZ_STAGES : slot0 + i;
-          };
-          auto lo_of = [&](int i) { return lo0 + (uint32_t)slot_of(i) * (OZ_STAGE_BYTES >> 4); };
-          constexpr uint32_t kB = OZ_A_BYTES >> 4;
-          // slice pairs (i, j), i >= j, i + j <= S - 1, in the order i, then
-          // j; the unrolled schedule is fixed by S.  (i, j) is the first
-          // pair of its group (i + j) in that order exactly when i - j <= 1.
+          const int b0 = (bc & 1) * S;
+          const uint32_t pb = (uint32_t)(bc >> 1) & 1u;
+          const uint32_t lob = lo0 + (uint32_t)b0 * (Shape::B_BYTES >> 4);
+          auto slot_of = [&](int i) { return (a0 + i) % AS; };
 #pragma unroll
-          for (int i = 0; i < S; ++i) {
-            const uint32_t ph = slot0 + i >= OZ_STAGES ? phase0 ^ 1u : phase0;
-            if (!warp_wait(&full[slot_of(i)], ph, lim)) {
-              if (lane == 0) atomicExch(a.err, 23);
-              abort_flag = 1;
-              ok = false;
-              break;
-            }
-            // each group of the previous chunk (of this tile or the one
-            // before) drained by the epilogue, which drains them in order,
-            // before its first MMA of this chunk: the groups first used at
-            // step i are 2i - 1 and 2i, so the MMAs of the first groups
-            // overlap the drain of the later ones
+          for (int p = 0; p < Shape::NP; ++p) {
+            const int gl = Shape::gl(p), gh = Shape::gh(p);
+#pragma unroll
+            for (int j = gl; j <= gh; ++j) wait_for(&full_b[b0 + j], pb, 23);
+            // the phase's groups of the previous chunk (of this tile or the
+            // one before) drained by the epilogue, which drains them in
+            // order: the first phase overlaps the drain of the later groups
             if (first_kb && gc > 0) {
 #pragma unroll
-              for (int grp = (i == 0 ? 0 : 2 * i - 1); grp <= 2 * i && grp < S; ++grp)
-                if (ok && !warp_wait(&tempty[grp], (uint32_t)(gc - 1) & 1u, lim)) {
-                  if (lane == 0) atomicExch(a.err, 22);
-                  abort_flag = 1;
-                  ok = false;
-                }
-              if (!ok) break;
+              for (int g = gl; g <= gh; ++g) wait_for(&tempty[g], (uint32_t)(gc - 1) & 1u, 22);
             }
-            fence_after();
-            const uint32_t si = lo_of(i);
+            if (!ok) break;
 #pragma unroll
-            for (int j = 0; j <= (i < S - 1 - i ? i : S - 1 - i); ++j) {
-              const uint32_t sj = lo_of(j);
-              const uint32_t d = tmem + (uint32_t)((i + j) * BN);
-              const bool overwrite = first_kb && (i - j <= 1);
-              // A slice i x B slice j (32 bytes per K step)
+            for (int i = 0; i <= gh; ++i) {
+              if (i >= gl) wait_for(&full_a[slot_of(i)], pa0 ^ ((uint32_t)((a0 + i) / AS) & 1u), 23);
+              if (!ok) break;
+              fence_after();
+              const int jl = gl > i ? gl - i : 0, n = gh - i - jl + 1;
+              const uint32_t la =
+                  lo0 + ((Shape::A_OFF + (uint32_t)slot_of(i) * OZ_A_BYTES) >> 4);
+              const uint32_t lb = lob + (uint32_t)jl * (Shape::B_BYTES >> 4);
+              const uint32_t d = tmem + (uint32_t)((i + jl) * BN);
 #pragma unroll
-              for (int k = 0; k < OZ_BK / 16; ++k)
-                mma_bf16_if(leader, d, desc_of(si + 2 * k), desc_of(sj + kB + 2 * k), idesc,
-                            (overwrite && k == 0) ? 0u : 1u);
-              if (j < i) {
-                // A slice j x B slice i
-#pragma unroll
-                for (int k = 0; k < OZ_BK / 16; ++k)
-                  mma_bf16_if(leader, d, desc_of(sj + 2 * k), desc_of(si + kB + 2 * k), idesc, 1u);
+              for (int k = 0; k < OZ_BK / 16; ++k)   // 32 bytes per K step
+                mma_bf16_if(leader, d, desc_of(la + 2 * k), desc_of(lb + 2 * k),
+                            idesc_bf16(OZ_BM, n * BN), (first_kb && i == 0 && k == 0) ? 0u : 1u);
+              if (p == Shape::NP - 1) {
+                // A_i and B_(S-1-i) have no later use (free once these MMAs complete)
+                mma_commit_if(leader, &empty_a[slot_of(i)]);
+                mma_commit_if(leader, &empty_b[b0 + S - 1 - i]);
               }
             }
-            // slice q is last used at step max(q, S-1-q): release what step i
-            // finished (the stage frees once these MMAs complete)
-            if (i >= S - 1 - i) mma_commit_if(leader, &empty[slot_of(i)]);
-            if (S - 1 - i < i) mma_commit_if(leader, &empty[slot_of(S - 1 - i)]);
+            if (!ok) break;
           }
           if (!ok) break;
-          slot0 += S;
-          if (slot0 >= OZ_STAGES) {
-            slot0 -= OZ_STAGES;
-            phase0 ^= 1u;
-          }
+          pa0 ^= (uint32_t)((a0 + S) / AS) & 1u;
+          a0 = (a0 + S) % AS;
         }
         if (ok) mma_commit_if(leader, tfull);
       }
@@ -817,13 +836,13 @@ template <int S, int BN>
 cudaError_t launch_oz_kernel(cudaStream_t st, int ctas, const CUtensorMap &mA,
                              const CUtensorMap &mB, const OzArgs &a) {
   if (a.ksplit <= 1) {
-    ozaki_gemm_kernel<S, BN, false><<<ctas, OZ_THREADS, OzShape<BN>::SMEM, st>>>(mA, mB, a);
+    ozaki_gemm_kernel<S, BN, false><<<ctas, OZ_THREADS, OzShape<S, BN>::SMEM, st>>>(mA, mB, a);
     return cudaGetLastError();
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas);
   cfg.blockDim = dim3(OZ_THREADS);
-  cfg.dynamicSmemBytes = OzShape<BN>::SMEM;
+  cfg.dynamicSmemBytes = OzShape<S, BN>::SMEM;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -837,7 +856,7 @@ cudaError_t launch_oz_kernel(cudaStream_t st, int ctas, const CUtensorMap &mA,
 
 template <int S, int BN>
 cudaError_t set_smem_attr() {
-  constexpr int bytes = (int)OzShape<BN>::SMEM;
+  constexpr int bytes = (int)OzShape<S, BN>::SMEM;
   const cudaError_t e = cudaFuncSetAttribute(ozaki_gemm_kernel<S, BN, false>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
@@ -853,7 +872,7 @@ int active_clusters(int c) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c * 256);
     cfg.blockDim = dim3(OZ_THREADS);
-    cfg.dynamicSmemBytes = OzShape<64>::SMEM;
+    cfg.dynamicSmemBytes = OzShape<6, 64>::SMEM;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = c;
@@ -880,6 +899,19 @@ int active_clusters(int c) {
 struct TilePlan {
   int bn, ks;
 };
+double block_clocks(int S, int bn) {
+  const int W = std::min(S, 256 / bn), np = (S + W - 1) / W;
+  double sum = 0;
+  for (int p = 0, gl = 0; p < np; ++p) {
+    const int gh = S - 1 - (np - 1 - p) * W;
+    for (int i = 0; i <= gh; ++i) {
+      const int n = (gh - std::max(i, gl) + 1) * bn;
+      sum += std::max(0.5 * n, 40 + 0.25 * n);
+    }
+    gl = gh + 1;
+  }
+  return 4 * sum;
+}
 TilePlan tile_plan(int S, int Mt, int N, int nch) {
   TilePlan best{64, 1};
   double least = 1e300;
@@ -889,7 +921,7 @@ TilePlan tile_plan(int S, int Mt, int N, int nch) {
       const int fit = active_clusters(ks);
       if (fit < 1) continue;
       const double cost = std::ceil(tiles / fit) * ((nch + ks - 1) / ks + (ks > 1 ? 0.83 : 0.33)) *
-                          (bn == 64 ? 55.0 : (bn == 80 ? 65.0 : 66.0));
+                          block_clocks(S, bn);
       if (cost < least) {
         least = cost;
         best = TilePlan{bn, ks};
