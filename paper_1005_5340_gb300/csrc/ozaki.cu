@@ -18,19 +18,24 @@
 // with an error of about (1 + (s+1)/4) 2^(-7s) 2^(eA+eB) K at most (2^-42
 // relative for s = 6).
 //
-// One CTA computes a 128 x 64 output tile:
+// One CTA computes a 128 x BN output tile (BN 64, 80 or 96):
 //   warp 0     TMA producer: per 64-deep K block, the s slices of the A tile
-//              (16 KB each) and of the B tile (8 KB each), one stage per
-//              slice index, into a 9-stage ring (128-byte swizzle)
-//   warp 1     tcgen05.mma issuer (M=128, N=64, K=16): once slice i of a K
-//              block has landed, every pair (i, j) and (j, i) with j <= i and
-//              i + j <= s+1 goes to the TMEM accumulator of group i+j (s
-//              groups x 64 columns); a slice's stage is released after the
-//              last pair that reads it, and a group of the next chunk starts
-//              as soon as the epilogue has drained it
-//   warps 2-9  epilogue (two warps per TMEM lane quadrant, 32 columns each):
-//              per chunk, TMEM -> registers -> int64 accumulators; at the end
+//              (16 KB each, a ring of 6 to 9) and of the B tile (8 to 12 KB
+//              each, side by side, two K blocks); 128-byte swizzle
+//   warp 1     tcgen05.mma issuer (M = 128, K = 16).  The pairs of slice A_i
+//              with neighbouring B slices are one MMA of up to 256 columns:
+//              the B slices are rows of one operand, their groups i + j
+//              neighbouring columns of tensor memory (s groups x BN columns).
+//              Pair by pair (N = BN) every MMA read its A tile for 64 to 96
+//              columns and took 55 to 66 clocks against 32 to 48 at the
+//              tensor core's rate; 64-atom operator, products 1447 -> 1150 us.
+//   warps 2-9  epilogue (two warps per TMEM lane quadrant, half of the columns
+//              each): per chunk, TMEM -> registers -> int64 accumulators, a
+//              phase's groups while the issuer is at the next one's; at the end
 //              the float64 tile is stored (C or C^T)
+// The issuer's waits and commits cost as much as its MMAs: one barrier per phase
+// of B slices and one release per K block (12 + 12 a block -> 8 + 7: 1.98 ->
+// 1.78 us per block of 6 slices, N = 64).
 // Every mbarrier wait is bounded; on expiry the CTA records an error code,
 // stops issuing work, waits (bounded) for its TMA copies in flight and still
 // frees its TMEM.
@@ -58,17 +63,15 @@ constexpr int OZ_EPI_WARPS = 8;                        // 2 per TMEM lane quadra
 constexpr int OZ_THREADS = 64 + 32 * OZ_EPI_WARPS;      // producer, MMA, epilogue
 constexpr uint32_t OZ_A_BYTES = OZ_BM * OZ_BK * 2;   // 16 KB
 // The N tile is 64 columns or the widest of 96 and 80 whose s groups fit in
-// tensor memory (s x BN <= 512), chosen per launch (tile_plan): an MMA reads
-// its A tile from shared memory whatever its N, and the operand reads bound
-// it, so a wide tile does more per read and a narrow one pads less.
-// 9 stages of 24 KB, or 8 of 26 or 28 KB.
+// tensor memory (s x BN <= 512), chosen per launch (tile_plan): a wide tile
+// reads fewer operand bytes per column, a narrow one pads less.  Shared memory
+// holds the B slices of two K blocks and as many A slices as fit.
 template <int S, int BN> struct OzShape {
   static constexpr int EPI_COLS = BN / 2;                      // columns per epilogue thread
   static constexpr uint32_t B_BYTES = BN * OZ_BK * 2;
-  static constexpr int BS = 2 * S;                             // B slices: two K blocks
-  static constexpr int AS_FIT = (int)((227 * 1024 - 1024 - 1024 - BS * B_BYTES) / OZ_A_BYTES);
+  static constexpr uint32_t A_OFF = 2 * S * B_BYTES;           // after two K blocks of B
+  static constexpr int AS_FIT = (int)((227 * 1024 - 1024 - 1024 - A_OFF) / OZ_A_BYTES);
   static constexpr int AS = AS_FIT < 9 ? AS_FIT : 9;           // A slices
-  static constexpr uint32_t A_OFF = BS * B_BYTES;
   static constexpr size_t SMEM = A_OFF + (size_t)AS * OZ_A_BYTES + 1024 + 512;
   // groups that one MMA takes, and the phases of a K block (see the issuer)
   static constexpr int W = 256 / BN < S ? 256 / BN : S, NP = (S + W - 1) / W;
@@ -120,7 +123,14 @@ constexpr int kOzMaxChunks = 1024;
 // Columns j0 .. j0 + n - 1 of acc from v (n = 16 or 32).
 template <int N, int EC>
 __device__ __forceinline__ void add_group(long long (&acc)[EC], const float *v, int j0, int sh) {
-  if (sh >= 0) {
+  // (one 32 x 32 + 64-bit multiply-add each; a weight above 2^30 occurs with 8
+  // slices only)
+  if (sh >= 0 && sh <= 30) {
+    const int w = 1 << sh;
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+      acc[j0 + j] += (long long)__float2int_rn(v[j]) * (long long)w;
+  } else if (sh >= 0) {
 #pragma unroll
     for (int j = 0; j < N; ++j) acc[j0 + j] += (long long)__float2int_rn(v[j]) << sh;
   } else {
@@ -135,11 +145,23 @@ __device__ __forceinline__ void add_group(long long (&acc)[EC], const float *v, 
 // 32, so that every 32-column load starts on a multiple of 32 columns; the
 // 40 columns of an 80-wide group's half are five 8-column loads.
 template <int S, int BN>
-__device__ __forceinline__ void read_groups(uint32_t tcol, int h,
+__device__ __forceinline__ bool read_groups(uint32_t tcol, int h,
                                             long long (&acc)[OzShape<S, BN>::EPI_COLS], int ns,
-                                            int drop, uint64_t *tempty) {
+                                            int drop, uint64_t *tempty, uint64_t *tfull,
+                                            uint32_t ph, uint64_t lim, int *abort_flag) {
+  using Shape = OzShape<S, BN>;
 #pragma unroll 1
   for (int grp = 0; grp < ns; ++grp) {
+    const int past = grp - Shape::gl(Shape::NP > 1 ? 1 : 0);   // groups past the first phase
+    if (grp == 0 || (past >= 0 && past % Shape::W == 0)) {
+      // the next phase's groups complete; tcgen05.ld is warp-collective: one
+      // decision per warp
+      const int p = grp == 0 ? 0 : 1 + past / Shape::W;
+      bool have = mbar_wait(&tfull[p], ph, lim);
+      have = __all_sync(0xffffffffu, have && !*(volatile int *)abort_flag);
+      if (!have) return false;
+      fence_after();
+    }
     const int sh = 7 * (S - 1 - grp) - drop;
     const uint32_t g0 = tcol + (uint32_t)(grp * BN);
     float v[BN == 80 ? 40 : 32], u[16];
@@ -168,6 +190,7 @@ __device__ __forceinline__ void read_groups(uint32_t tcol, int h,
       add_group<32>(acc, v, 16, sh);
     }
   }
+  return true;
 }
 
 // 2^e for a normal-range exponent (clamped to [-1022, 1023])
@@ -200,7 +223,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   int N = a.N;
   if (a.dcnt) N = (int)min((int64_t)N, (int64_t)a.mul_n * (*a.dcnt));
   using Shape = OzShape<S, BN>;
-  constexpr int AS = Shape::AS, BS = Shape::BS;
+  constexpr int AS = Shape::AS, NP = Shape::NP;
   constexpr int OZ_EPI_COLS = Shape::EPI_COLS;
   // Persistent: CTA b walks tiles t = b, b + gridDim.x, ...  Tile t -> (mt,
   // nt) in an L2-aware order: the M tiles (rows of A, or entries of the tile
@@ -252,9 +275,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   uint64_t *full_a = (uint64_t *)(smem + Shape::A_OFF + AS * OZ_A_BYTES);
   uint64_t *empty_a = full_a + AS;
   uint64_t *full_b = empty_a + AS;
-  uint64_t *empty_b = full_b + BS;
-  uint64_t *tfull = empty_b + BS;
-  uint64_t *tempty = tfull + 1;   // [kOzMaxSlices] one per TMEM group
+  uint64_t *empty_b = full_b + 2 * NP;    // full_b: [2][NP], a K block's B slices phase by phase
+  uint64_t *tfull = empty_b + 2;          // [NP] a chunk's groups, phase by phase
+  uint64_t *tempty = tfull + Shape::NP;   // [kOzMaxSlices] one per TMEM group
   uint64_t *drain = tempty + kOzMaxSlices;   // completion of every MMA this CTA issued
   uint32_t *tslot = (uint32_t *)(drain + 1);
   __shared__ int abort_flag;
@@ -270,11 +293,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       mbar_init(&full_a[i], 1);
       mbar_init(&empty_a[i], 1);
     }
-    for (int i = 0; i < BS; ++i) {
-      mbar_init(&full_b[i], 1);
-      mbar_init(&empty_b[i], 1);
-    }
-    mbar_init(tfull, 1);
+    for (int i = 0; i < 2 * NP; ++i) mbar_init(&full_b[i], 1);
+    for (int i = 0; i < 2; ++i) mbar_init(&empty_b[i], 1);
+    for (int p = 0; p < NP; ++p) mbar_init(&tfull[p], 1);
     for (int q = 0; q < kOzMaxSlices; ++q)
       mbar_init(&tempty[q], OZ_EPI_WARPS);   // one arrival per epilogue warp
     mbar_init(drain, 1);
@@ -295,25 +316,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   if (warp == 0) {
     if (lane == 0) {
       // producer: the A slices go round a ring of AS tiles, the B slices
-      // round two K blocks.  Of a K block: what the first phase needs, A and
-      // B in turn, then the other B slices, then the other A slices (the last
-      // phase frees A slices from its first step on, which needs every B).
-      int ga = 0, gb = 0;   // slices issued
+      // round two K blocks.  Of a K block: the first phase's B and A slices,
+      // the other phases' B slices, then the other A slices (the last phase
+      // frees A slices from its first step on, which needs every B).
+      int ga = 0, gb = 0;   // A slices and phases of B slices issued
       bool ok = true;
-      auto load = [&](uint64_t *full, uint64_t *empty, int &g, int n, uint32_t bytes, uint8_t *base,
-                      const CUtensorMap *map, int x, int y) {
-        const int slot = g % n;
-        const uint32_t ph = (uint32_t)(g / n) & 1u;
-        if (!mbar_wait(&empty[slot], ph ^ 1u, lim)) {
+      auto freed = [&](uint64_t *empty, uint32_t ph) {
+        if (!mbar_wait(empty, ph ^ 1u, lim)) {
           atomicExch(a.err, 21);
           abort_flag = 1;
           return false;
         }
-        if (*(volatile int *)&abort_flag) return false;
-        mbar_expect_tx(&full[slot], bytes);
-        tma_load_2d(base + slot * bytes, map, &full[slot], x, y);
-        ++g;
-        return true;
+        return !*(volatile int *)&abort_flag;
       };
       for (int t = tile0; t < n_tiles && ok; t += tstep) {
         Tile T;
@@ -321,25 +335,36 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         for (int kb = 0; kb < T.nkb && ok; ++kb) {
           const int kx = (T.kb0 + kb) * OZ_BK;
           auto load_a = [&](int i) {
-            ok = ok && load(full_a, empty_a, ga, AS, OZ_A_BYTES, smem + Shape::A_OFF, &mapA,
-                            i * a.KpA + kx, T.m0);
+            const int slot = ga % AS;
+            ok = ok && freed(&empty_a[slot], (uint32_t)(ga / AS) & 1u);
+            if (!ok) return;
+            mbar_expect_tx(&full_a[slot], OZ_A_BYTES);
+            tma_load_2d(smem + Shape::A_OFF + slot * OZ_A_BYTES, &mapA, &full_a[slot],
+                        i * a.KpA + kx, T.m0);
+            ++ga;
           };
-          auto load_b = [&](int i) {
-            ok = ok && load(full_b, empty_b, gb, BS, Shape::B_BYTES, smem, &mapB,
-                            i * a.KpB + T.xoff + kx, T.n0);
+          auto load_b = [&](int p) {
+            const int half = gb / NP & 1, lo = Shape::gl(p), hi = Shape::gh(p);
+            if (p == 0) ok = ok && freed(&empty_b[half], (uint32_t)(gb / NP >> 1) & 1u);
+            if (!ok) return;
+            uint64_t *bar = &full_b[gb % (2 * NP)];
+            mbar_expect_tx(bar, (hi - lo + 1) * Shape::B_BYTES);
+            for (int j = lo; j <= hi; ++j)
+              tma_load_2d(smem + (half * S + j) * Shape::B_BYTES, &mapB, bar,
+                          j * a.KpB + T.xoff + kx, T.n0);
+            ++gb;
           };
-          for (int i = 0; i <= Shape::gh(0); ++i) {
-            load_a(i);
-            load_b(i);
-          }
-          for (int i = Shape::gh(0) + 1; i < S; ++i) load_b(i);
+          load_b(0);
+          for (int i = 0; i <= Shape::gh(0); ++i) load_a(i);
+          for (int p = 1; p < NP; ++p) load_b(p);
           for (int i = Shape::gh(0) + 1; i < S; ++i) load_a(i);
         }
       }
-      // copies in flight: the latest use of every slot must have landed
+      // copies in flight: the latest use of every barrier must have completed
       // before the CTA may exit
       for (int h = max(0, ga - AS); h < ga; ++h) mbar_wait(&full_a[h % AS], (uint32_t)(h / AS) & 1u);
-      for (int h = max(0, gb - BS); h < gb; ++h) mbar_wait(&full_b[h % BS], (uint32_t)(h / BS) & 1u);
+      for (int h = max(0, gb - 2 * NP); h < gb; ++h)
+        mbar_wait(&full_b[h % (2 * NP)], (uint32_t)(h / (2 * NP)) & 1u);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -372,15 +397,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const int kb1 = min(T.nkb, (c + 1) * cb);
         for (int kb = c * cb; kb < kb1 && ok; ++kb, ++bc) {
           const bool first_kb = kb == c * cb;
-          const int b0 = (bc & 1) * S;
           const uint32_t pb = (uint32_t)(bc >> 1) & 1u;
-          const uint32_t lob = lo0 + (uint32_t)b0 * (Shape::B_BYTES >> 4);
+          const uint32_t lob = lo0 + (uint32_t)((bc & 1) * S) * (Shape::B_BYTES >> 4);
           auto slot_of = [&](int i) { return (a0 + i) % AS; };
 #pragma unroll
-          for (int p = 0; p < Shape::NP; ++p) {
+          for (int p = 0; p < NP; ++p) {
             const int gl = Shape::gl(p), gh = Shape::gh(p);
-#pragma unroll
-            for (int j = gl; j <= gh; ++j) wait_for(&full_b[b0 + j], pb, 23);
+            wait_for(&full_b[(bc & 1) * NP + p], pb, 23);
             // the phase's groups of the previous chunk (of this tile or the
             // one before) drained by the epilogue, which drains them in
             // order: the first phase overlaps the drain of the later groups
@@ -403,19 +426,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
               for (int k = 0; k < OZ_BK / 16; ++k)   // 32 bytes per K step
                 mma_bf16_if(leader, d, desc_of(la + 2 * k), desc_of(lb + 2 * k),
                             idesc_bf16(OZ_BM, n * BN), (first_kb && i == 0 && k == 0) ? 0u : 1u);
-              if (p == Shape::NP - 1) {
-                // A_i and B_(S-1-i) have no later use (free once these MMAs complete)
-                mma_commit_if(leader, &empty_a[slot_of(i)]);
-                mma_commit_if(leader, &empty_b[b0 + S - 1 - i]);
-              }
+              // A_i has no later use (free once these MMAs complete)
+              if (p == NP - 1) mma_commit_if(leader, &empty_a[slot_of(i)]);
             }
             if (!ok) break;
+            // (the epilogue reads them while the later phases still run)
+            if (kb == kb1 - 1) mma_commit_if(leader, &tfull[p]);
           }
           if (!ok) break;
+          mma_commit_if(leader, &empty_b[bc & 1]);
           pa0 ^= (uint32_t)((a0 + S) / AS) & 1u;
           a0 = (a0 + S) % AS;
         }
-        if (ok) mma_commit_if(leader, tfull);
       }
     }
     // every MMA issued here (also after an abort) completes before the
@@ -441,17 +463,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       for (int j = 0; j < OZ_EPI_COLS; ++j) acc[j] = 0;
       bool ok = true;
       for (int c = 0; c < nchunks; ++c, ++gc) {
-        bool have = mbar_wait(tfull, (uint32_t)gc & 1u, lim);
-        // tcgen05.ld is warp-collective: one decision per warp
-        have = __all_sync(0xffffffffu, have && !*(volatile int *)&abort_flag);
-        if (!have) {
+        if (!read_groups<S, BN>(tcol, h, acc, a.ns, a.drop, tempty, tfull, (uint32_t)gc & 1u, lim,
+                                &abort_flag)) {
           if (lane == 0) atomicExch(a.err, 24);
           abort_flag = 1;
           ok = false;
           break;
         }
-        fence_after();
-        read_groups<S, BN>(tcol, h, acc, a.ns, a.drop, tempty);
       }
       if (!ok) break;
       if constexpr (SPLIT) {
@@ -890,28 +908,33 @@ int active_clusters(int c) {
   return fit[c];
 }
 
-// N tile and K split of a product of Mt row tiles, N columns and nch K chunks:
-// the least of waves x chunks per CTA x clocks per MMA (measured: 55 at N =
-// 64, 65 at 80, 66 at 96, the reads of the A tile among them), with half a
-// chunk for the sum over a cluster and a third for a tile's start.  Exact
-// integer sums: every plan gives the same bits.
-// (1000 x 129 x 9080, 6 slices: 24 CTAs 455 us -> 16 clusters of 6, 101 us.)
-struct TilePlan {
-  int bn, ks;
-};
+// Clocks per K block of a tile: an MMA of N columns takes N / 2 at the tensor
+// core's rate and at least 40 + N / 4 (operand reads and issue), the slices
+// come from L2 at 54 bytes a clock at most.  Measured per block, 15% of it at
+// the chunks' ends: 5 slices 2670 clocks at N = 64 and 3530 at 96, 6 slices
+// 3400 at 64 and 4010 at 80 (pair by pair: 4600 at 64, 5460 at 80).
 double block_clocks(int S, int bn) {
   const int W = std::min(S, 256 / bn), np = (S + W - 1) / W;
-  double sum = 0;
+  double mma = 0;
   for (int p = 0, gl = 0; p < np; ++p) {
     const int gh = S - 1 - (np - 1 - p) * W;
     for (int i = 0; i <= gh; ++i) {
       const int n = (gh - std::max(i, gl) + 1) * bn;
-      sum += std::max(0.5 * n, 40 + 0.25 * n);
+      mma += std::max(0.5 * n, 40 + 0.25 * n);
     }
     gl = gh + 1;
   }
-  return 4 * sum;
+  return std::max(OZ_BK / 16 * mma, S * (OZ_BM + bn) * OZ_BK * 2 / 54.0);
 }
+
+// N tile and K split of a product of Mt row tiles, N columns and nch K chunks:
+// the least of waves x chunks per CTA x clocks per block, with half a chunk
+// for the sum over a cluster and a third for a tile's start.  Exact integer
+// sums: every plan gives the same bits.
+// (1000 x 129 x 9080, 6 slices: 24 CTAs 455 us -> 13 clusters of 6, 65 us.)
+struct TilePlan {
+  int bn, ks;
+};
 TilePlan tile_plan(int S, int Mt, int N, int nch) {
   TilePlan best{64, 1};
   double least = 1e300;
