@@ -282,21 +282,51 @@ __device__ __forceinline__ double2 d_factor(double w, double delta, double eps, 
   return make_double2(xm * im2 - xp * ip2, eps * (ip2 - im2));
 }
 
-// a[F][(2s, 2s+1)][E] *= D_EF(omega_s): one thread per (F, s, E), about
-// 25 FP64 operations each, which bound it (64 right-hand sides on 64 atoms: 254 us)
-__global__ void __launch_bounds__(256) dscale_kernel(
+// D of consecutive columns: computed anew where the frequency changes (the
+// three field directions of a frequency follow one another).
+struct DOfColumn {
+  double w;
+  double2 d;
+  __device__ __forceinline__ void at(bool first, double w_new, double delta, double eps, double e2,
+                                     double occ) {
+    if (!first && w_new == w) return;
+    w = w_new;
+    d = d_factor(w, delta, eps, e2, occ);
+  }
+};
+
+// a[F][(2s, 2s+1)][E] *= D_EF(omega_s): one thread per (F, G columns s, E).
+// Bound by its FP64 operations, about 21 for a D and 4 for a product with it
+// (64 right-hand sides on 64 atoms: a D per column 247 us, per frequency 123).
+template <int G>
+__global__ void __launch_bounds__(128) dscale_kernel(
     int n_virt, int S, int n_occ, double occ_value, const double *__restrict__ energy,
     const double *__restrict__ omega, double eps, double e2, double *__restrict__ a,
     const int *__restrict__ dcnt) {
-  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  const int64_t row = i / n_occ;   // F * S + s
-  const int F = (int)(row / S), s = (int)(row - (int64_t)F * S), E = (int)(i - row * n_occ);
-  if (F >= n_virt || (dcnt && s >= *dcnt)) return;
-  const double2 d = d_factor(omega[s], energy[n_occ + F] - energy[E], eps, e2, occ_value);
-  double *at = a + ((int64_t)F * 2 * S + 2 * s) * n_occ + E;
-  const double re = at[0], im = at[n_occ];
-  at[0] = d.x * re - d.y * im;
-  at[n_occ] = d.x * im + d.y * re;
+  const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  const int64_t row = i / n_occ;   // F * chunks + chunk
+  const int chunks = (S + G - 1) / G;
+  const int F = (int)(row / chunks), s0 = (int)(row - (int64_t)F * chunks) * G,
+            E = (int)(i - row * n_occ);
+  const int live = dcnt ? min(S, *dcnt) : S;
+  if (F >= n_virt || s0 >= live) return;
+  const double delta = energy[n_occ + F] - energy[E];
+  double *at = a + ((int64_t)F * 2 * S + 2 * s0) * n_occ + E;
+  double re[G], im[G];
+#pragma unroll
+  for (int q = 0; q < G; ++q)
+    if (s0 + q < live) {
+      re[q] = at[(int64_t)(2 * q) * n_occ];
+      im[q] = at[(int64_t)(2 * q + 1) * n_occ];
+    }
+  DOfColumn D;
+#pragma unroll
+  for (int q = 0; q < G; ++q)
+    if (s0 + q < live) {
+      D.at(q == 0, omega[s0 + q], delta, eps, e2, occ_value);
+      at[(int64_t)(2 * q) * n_occ] = D.d.x * re[q] - D.d.y * im[q];
+      at[(int64_t)(2 * q + 1) * n_occ] = D.d.x * im[q] + D.d.y * re[q];
+    }
 }
 
 __global__ void i2p_kernel(int n_rhs, int n, const double *__restrict__ in, double *__restrict__ out) {
@@ -320,23 +350,27 @@ __global__ void p2i_kernel(int n_rhs, int n, const double *__restrict__ in, doub
 }
 
 // a[F][(2s, 2s+1)][E] = D_EF(omega_{(g0+s)/3}) * a3[F][(2k, 2k+1)][E], k = (g0+s) % 3:
-// one thread per (F, s, E)
-__global__ void __launch_bounds__(256) rhs_expand_kernel(
+// one thread per (F, frequency, E), its three columns or those of them in 0 .. S - 1
+__global__ void __launch_bounds__(128) rhs_expand_kernel(
     int n_virt, int S, int n_occ, int g0, double occ_value, const double *__restrict__ energy,
     const double *__restrict__ omega_all, double eps, double e2, const double *__restrict__ a3,
     double *__restrict__ a) {
-  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  const int64_t row = i / n_occ;   // F * S + s
-  const int F = (int)(row / S), s = (int)(row - (int64_t)F * S), E = (int)(i - row * n_occ);
+  const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  const int64_t row = i / n_occ;   // F * frequencies + frequency
+  const int f0 = g0 / 3, nf = (g0 + S - 1) / 3 - f0 + 1;
+  const int F = (int)(row / nf), f = f0 + (int)(row - (int64_t)F * nf), E = (int)(i - row * n_occ);
   if (F >= n_virt) return;
-  const int g = g0 + s, k = g % 3;
-  const double2 d =
-      d_factor(omega_all[g / 3], energy[n_occ + F] - energy[E], eps, e2, occ_value);
-  const double *src = a3 + ((int64_t)F * 6 + 2 * k) * n_occ + E;
-  double *dst = a + ((int64_t)F * 2 * S + 2 * s) * n_occ + E;
-  const double re = src[0], im = src[n_occ];
-  dst[0] = d.x * re - d.y * im;
-  dst[n_occ] = d.x * im + d.y * re;
+  const double2 d = d_factor(omega_all[f], energy[n_occ + F] - energy[E], eps, e2, occ_value);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int s = 3 * f + k - g0;
+    if (s < 0 || s >= S) continue;
+    const double *src = a3 + ((int64_t)F * 6 + 2 * k) * n_occ + E;
+    double *dst = a + ((int64_t)F * 2 * S + 2 * s) * n_occ + E;
+    const double re = src[0], im = src[n_occ];
+    dst[0] = d.x * re - d.y * im;
+    dst[n_occ] = d.x * im + d.y * re;
+  }
 }
 
 // Z3 rows (d_0, 0, d_1, 0, d_2, 0)
@@ -432,18 +466,24 @@ cudaError_t launch_beta(cudaStream_t st, const DevSystem &sys, int ncols, const 
 
 cudaError_t launch_dscale(cudaStream_t st, const DevSystem &sys, int S, const double *omega,
                           double eps, double *a, const int *dcnt) {
-  const int64_t n = ((int64_t)sys.n_virt * S * sys.n_occ + 255) / 256;
+  // six columns per thread (two D where the frequencies come in threes, three
+  // where a group starts elsewhere), or three where that would leave SMs idle
+  const int64_t per = (int64_t)sys.n_virt * sys.n_occ;
+  const bool six = per * ((S + 5) / 6) >= 152 * 1024;
+  const int64_t n = (per * (six ? (S + 5) / 6 : (S + 2) / 3) + 127) / 128;
   if (n > INT32_MAX) return cudaErrorInvalidConfiguration;
-  dscale_kernel<<<(unsigned)n, 256, 0, st>>>(sys.n_virt, S, sys.n_occ, sys.occ_value, sys.energy,
-                                             omega, eps, eps * eps, a, dcnt);
+  auto *kernel = six ? dscale_kernel<6> : dscale_kernel<3>;
+  kernel<<<(unsigned)n, 128, 0, st>>>(sys.n_virt, S, sys.n_occ, sys.occ_value, sys.energy, omega,
+                                      eps, eps * eps, a, dcnt);
   return cudaGetLastError();
 }
 
 cudaError_t launch_rhs_expand(cudaStream_t st, const DevSystem &sys, int S, int g0,
                               const double *omega_all, double eps, const double *a3, double *a) {
-  const int64_t n = ((int64_t)sys.n_virt * S * sys.n_occ + 255) / 256;
+  const int nf = (g0 + S - 1) / 3 - g0 / 3 + 1;
+  const int64_t n = ((int64_t)sys.n_virt * nf * sys.n_occ + 127) / 128;
   if (n > INT32_MAX) return cudaErrorInvalidConfiguration;
-  rhs_expand_kernel<<<(unsigned)n, 256, 0, st>>>(sys.n_virt, S, sys.n_occ, g0,
+  rhs_expand_kernel<<<(unsigned)n, 128, 0, st>>>(sys.n_virt, S, sys.n_occ, g0,
                                                  sys.occ_value, sys.energy, omega_all, eps,
                                                  eps * eps, a3, a);
   return cudaGetLastError();
