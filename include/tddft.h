@@ -292,8 +292,9 @@ tddft_status tddft_kernel_apply(tddft_ctx *ctx, int32_t n_rhs, const double *z, 
  *  centres [n_centres][3] (bohr) and prod_centre [n_prod] (centre index of
  *  each product, 0 <= c < n_centres): HOST pointers.  z, out: DEVICE
  *  pointers, n_rhs x n_prod complex interleaved.  stream: cudaStream_t
- *  (NULL = legacy default), synchronised before returning.  Allocates and
- *  frees its scratch (about 32 n_rhs n_centres bytes).
+ *  (NULL = legacy default), synchronised before returning.  Its scratch
+ *  (about 32 n_rhs n_centres bytes) comes from the library's stream-ordered
+ *  pool, which keeps at most 256 MB and gives them back at tddft_destroy.
  * Errors: INVALID_ARG (NULL, sizes < 1, softening < 0 or NaN), SHAPE (a
  * centre index out of range), NOMEM, CUDA.
  */
