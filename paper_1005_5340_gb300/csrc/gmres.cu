@@ -913,7 +913,9 @@ __global__ void __launch_bounds__(NT, 3) gmres_step_kernel(Gs G, const int *__re
   __syncthreads();
   const double hn = s_hn;
   if (scalar && warp == 0) {
-    // the rotated entry is carried in registers from one rotation to the next
+    // the rotated entry is carried in registers from one rotation to the next;
+    // lane 0 leaves the column in hp, since the other lanes may still be
+    // reading hs (and gq, hq) where it is ahead of them
     double2 a = hs[0];
 #pragma unroll 4
     for (int i = 0; i < j; ++i) {
@@ -922,9 +924,11 @@ __global__ void __launch_bounds__(NT, 3) gmres_step_kernel(Gs G, const int *__re
       const double2 t = make_double2(csi * a.x + (sni.x * bb.x - sni.y * bb.y),
                                      csi * a.y + (sni.x * bb.y + sni.y * bb.x));
       const double2 cb = cmul(cconj(sni), a);
-      if (lane == 0) hs[i] = t;
+      if (lane == 0) hp[i] = t;
       a = make_double2(-cb.x + csi * bb.x, -cb.y + csi * bb.y);
     }
+    __syncwarp();
+    for (int i = lane; i < j; i += 32) hs[i] = hp[i];
     // new rotation mapping (a, hn) to (rho, 0); its three quotients, then the
     // last two, are one division each on three lanes
     const double aa = cabs2(a);
