@@ -398,9 +398,9 @@ tddft_status tddft_spectrum_adaptive(tddft_ctx *ctx, double w_lo, double w_hi, d
  * tddft_polarizability with warm starts and the solutions returned.
  *  x0 (may be NULL): n_omega x 3 x n_prod complex interleaved, row w*3+k the
  *      initial guess of (omega[w], direction k).  Each guess first costs one
- *      float64 product A x0; if ||b - A x0|| > ||b||, zero is used instead
- *      (stats flags bit 0), so plain zero-guess GMRES is both the fallback
- *      and the arbiter of a guess.
+ *      float64 product A x0; unless ||b - A x0|| <= ||b||, zero is used instead
+ *      (stats flags bit 0; so also for a guess with a NaN or an infinity), so
+ *      plain zero-guess GMRES is both the fallback and the arbiter of a guess.
  *  X (may be NULL): receives the solutions X_k(omega) in the same layout.
  *  x0 and X are device pointers: flags must include TDDFT_DEVICE_PTRS when
  *  either is given.  Everything else as tddft_polarizability.

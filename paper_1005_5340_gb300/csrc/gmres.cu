@@ -503,9 +503,9 @@ __global__ void __launch_bounds__(NT, 3) gmres_step_kernel(Gs G, const int *__re
     }
     double rho = sqrt(s2[0]);
     bool rejected = false;
-    if (cyc == 0 && rho > G.bnorm[r]) {
+    if (cyc == 0 && !(rho <= G.bnorm[r])) {
       // the residual of a supplied initial guess: zero is the fallback and the
-      // arbiter, so a guess worse than zero is dropped
+      // arbiter, so a guess worse than zero, or one with a NaN, is dropped
       for (int e = lo + tid; e < hi; e += NT) {
         Vr[e] = (T)b[e];
         Vr[N + e] = (T)b[N + e];
