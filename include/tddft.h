@@ -213,8 +213,9 @@ typedef struct {
   int64_t wait_timeout_ns;
 } tddft_options;
 
-/* Change the wait limit of a context's tensor-core kernels (see
- * tddft_options.wait_timeout_ns; 0 = 2 s) for its later calls.
+/* Change the wait limit of a context's tensor-core kernels, its guess
+ * network's (tddft_guess_load) among them (see
+ * tddft_options.wait_timeout_ns; 0 = 2 s), for its later calls.
  * Synchronises the context's stream. */
 tddft_status tddft_set_wait_timeout(tddft_ctx *ctx, int64_t wait_timeout_ns);
 
@@ -524,10 +525,23 @@ tddft_status tddft_gemm_f64_emulated(int32_t M, int32_t N, int32_t K, const doub
  */
 typedef struct tddft_mlp tddft_mlp;
 
-/* Allocate a network and scratch for up to max_rows rows on `stream`. */
+/* Allocate a network and scratch for up to max_rows rows on `stream`.
+ * Networks of up to 12 inputs, 256 units and 4 outputs run on tensor-core
+ * kernels, whose waits are bounded (tddft_options.wait_timeout_ns).  The
+ * calls that do not synchronise (tddft_mlp_forward, tddft_mlp_train_step,
+ * tddft_mlp_backward without grad_host) return before such a wait could give
+ * up.  Where one does, the rows that it cost are NaN, training steps leave
+ * the parameters and the Adam state as they are, and the next call on the
+ * network that synchronises (tddft_mlp_params, tddft_mlp_save,
+ * tddft_mlp_load, tddft_mlp_backward with grad_host) returns
+ * TDDFT_ERR_TIMEOUT, once; after that the network works as before. */
 tddft_status tddft_mlp_create(int32_t n_in, int32_t width, int32_t n_out, int64_t max_rows,
                               uint64_t seed, void *stream, tddft_mlp **out);
 void tddft_mlp_destroy(tddft_mlp *mlp);
+/* The wait limit of the network's tensor-core kernels for its later calls (as
+ * tddft_set_wait_timeout, which also sets it for a context's own network;
+ * 0 = 2 s).  Synchronises the network's stream. */
+tddft_status tddft_mlp_set_wait_timeout(tddft_mlp *mlp, int64_t wait_timeout_ns);
 const char *tddft_mlp_last_error(const tddft_mlp *mlp);
 int64_t tddft_mlp_num_params(const tddft_mlp *mlp);
 /* Copy the packed parameters to (set = 0) or from (set = 1) a host buffer of
@@ -544,7 +558,8 @@ tddft_status tddft_mlp_load(tddft_mlp *mlp, const char *path);
 tddft_status tddft_mlp_forward(tddft_mlp *mlp, int64_t rows, const float *F, float *Y,
                                int32_t bf16);
 /* Gradient of sum_rows dY . Y with respect to the parameters (float32
- * forward then backward); copied to grad_host (n floats) when not NULL. */
+ * forward then backward); copied to grad_host (n floats) when not NULL.
+ * TIMEOUT: a wait gave up and grad_host is not the gradient. */
 tddft_status tddft_mlp_backward(tddft_mlp *mlp, int64_t rows, const float *F, const float *dY,
                                 float *grad_host);
 /* One Adam step (beta 0.9 / 0.999, eps 1e-8, learning rate lr) on the mean
@@ -582,7 +597,8 @@ tddft_status tddft_guess_combine(int64_t n_target, int32_t n_prod, const float *
  * network's correction y for TDDFT_GUESS_LEARNED (features: the spacing
  * term is the pass's mean (omega+ - omega-) over eps).  Each guess is
  * arbitrated as in tddft_polarizability_guess, so every frequency meets the
- * same float64 tolerance whatever the mode.  Allocates its device buffers
+ * same float64 tolerance whatever the mode.  Returns TIMEOUT if a wait of the
+ * learned guess's network gave up.  Allocates its device buffers
  * per call (the solutions of all frequencies and one chunk's guesses).
  */
 /* pass[i] (0, 1, 2) and the neighbours left[i], right[i] (-1 in pass 0) of

@@ -121,7 +121,13 @@ __global__ void colsum_kernel(int64_t M, int N, const float *__restrict__ X, flo
 
 __global__ void adam_kernel(int64_t n, float *__restrict__ p, const float *__restrict__ g,
                             float *__restrict__ m, float *__restrict__ v, float lr, float b1,
-                            float b2, float eps, float c1, float c2) {
+                            float b2, float eps, float c1, float c2, int *__restrict__ err) {
+  // a wait of the network kernels gave up: g is not the gradient (err[1]
+  // counts the steps left out; err NULL: kernels without waits)
+  if (err && err[0] != 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(err + 1, 1);
+    return;
+  }
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const float gi = g[i];
@@ -298,16 +304,19 @@ __global__ void combine_kernel(int64_t n, const float *__restrict__ Y, const dou
 
 tddft_status mfail(tddft_mlp *p, tddft_status s, const std::string &msg);
 
-// After a synchronisation: a wait of the tensor-core kernels that gave up.
+// Whether a wait of the tensor-core kernels gave up in the calls up to now
+// (synchronises the network's stream); reported once.
 tddft_status check_waits(tddft_mlp *p) {
   if (!p->use_tc) return TDDFT_OK;
-  int code = 0;
-  cudaError_t e = cudaMemcpy(&code, p->tc.err, sizeof(int), cudaMemcpyDeviceToHost);
+  int h[2] = {0, 0};   // code, training steps left out since
+  cudaError_t e = cudaMemcpyAsync(h, p->tc.err, sizeof(h), cudaMemcpyDeviceToHost, p->st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);
+  if (e == cudaSuccess && h[0] != 0) e = cudaMemsetAsync(p->tc.err, 0, sizeof(h), p->st);
   if (e != cudaSuccess) return mfail(p, TDDFT_ERR_CUDA, cudaGetErrorString(e));
-  if (code == 0) return TDDFT_OK;
-  cudaMemset(p->tc.err, 0, sizeof(int));
+  if (h[0] == 0) return TDDFT_OK;
+  p->step -= h[1];
   return mfail(p, TDDFT_ERR_TIMEOUT, "a network kernel's wait gave up (code " +
-                                         std::to_string(code) + ")");
+                                         std::to_string(h[0]) + ")");
 }
 
 tddft_status mfail(tddft_mlp *p, tddft_status s, const std::string &msg) {
@@ -384,12 +393,15 @@ cudaError_t backward(tddft_mlp *p, int64_t rows, const float *F, const float *dY
 
 }  // namespace
 
+tddft_status mlp_check_waits(tddft_mlp *p) { return check_waits(p); }
+
 // accessor defined with the context
 const DevSystem *ctx_system(const tddft_ctx *c);
 cudaStream_t ctx_stream(const tddft_ctx *c);
 void ctx_set_error(tddft_ctx *c, const char *msg);
 const float *ctx_product_features(const tddft_ctx *c);
 int ctx_slots(const tddft_ctx *c);
+int64_t ctx_wait_timeout(const tddft_ctx *c);
 void ctx_set_guess_net(tddft_ctx *c, tddft_mlp *net);
 
 }  // namespace tddft
@@ -483,6 +495,16 @@ const char *tddft_mlp_last_error(const tddft_mlp *p) {
   return p ? p->err.c_str() : g_mlp_error.c_str();
 }
 
+tddft_status tddft_mlp_set_wait_timeout(tddft_mlp *p, int64_t ns) {
+  if (!p || ns < 0) return mfail(p, TDDFT_ERR_INVALID_ARG, "bad network or wait_timeout_ns < 0");
+  if (!p->use_tc) return TDDFT_OK;   // kernels without waits
+  const unsigned long long v = (unsigned long long)ns;
+  cudaError_t e = cudaMemcpyAsync(p->tc.err + 2, &v, sizeof(v), cudaMemcpyHostToDevice, p->st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);
+  if (e != cudaSuccess) return mfail(p, TDDFT_ERR_CUDA, cudaGetErrorString(e));
+  return TDDFT_OK;
+}
+
 int64_t tddft_mlp_num_params(const tddft_mlp *p) { return p ? p->n_params : 0; }
 
 tddft_status tddft_mlp_params(tddft_mlp *p, float *host, int64_t n, int32_t set) {
@@ -493,8 +515,9 @@ tddft_status tddft_mlp_params(tddft_mlp *p, float *host, int64_t n, int32_t set)
   if (e == cudaSuccess && set) e = cudaMemsetAsync(p->v, 0, n * sizeof(float), p->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);
   if (e != cudaSuccess) return mfail(p, TDDFT_ERR_CUDA, cudaGetErrorString(e));
+  const tddft_status waits = check_waits(p);
   if (set) p->step = 0;
-  return check_waits(p);
+  return waits;
 }
 
 tddft_status tddft_mlp_save(tddft_mlp *p, const char *path) {
@@ -591,7 +614,8 @@ tddft_status tddft_mlp_train_step(tddft_mlp *p, int32_t n_target, int32_t n_prod
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - std::pow(b1, (float)p->step), c2 = 1.f - std::pow(b2, (float)p->step);
     adam_kernel<<<grid1(p->n_params), 256, 0, p->st>>>(p->n_params, p->params, p->grad, p->m, p->v,
-                                                       lr, b1, b2, 1e-8f, c1, c2);
+                                                       lr, b1, b2, 1e-8f, c1, c2,
+                                                       p->use_tc ? p->tc.err : nullptr);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) return mfail(p, TDDFT_ERR_CUDA, cudaGetErrorString(e));
@@ -644,6 +668,7 @@ tddft_status tddft_guess_load(tddft_ctx *ctx, const char *path) {
   tddft_mlp *net = nullptr;
   tddft_status st = tddft_mlp_create(hd.n_in, hd.width, hd.n_out, rows, 0, ctx_stream(ctx), &net);
   if (st == TDDFT_OK) st = tddft_mlp_load(net, path);
+  if (st == TDDFT_OK) st = tddft_mlp_set_wait_timeout(net, ctx_wait_timeout(ctx));
   if (st != TDDFT_OK) {
     ctx_set_error(ctx, net ? net->err.c_str() : g_mlp_error.c_str());
     if (net) tddft_mlp_destroy(net);

@@ -30,7 +30,7 @@
 //
 // Every mbarrier wait is bounded; on expiry the kernel records an error code,
 // stops issuing work, lets its copies and MMAs in flight finish and frees its
-// tensor memory.
+// tensor memory; a forward CTA then sets every output of its rows to NaN.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -110,6 +110,7 @@ __global__ void mlp_prepare_kernel(MlpTc tc, const float *__restrict__ prm) {
 
 constexpr int kRingMax = 4;
 struct Ctl {
+  uint64_t lim;   // limit of the roles' waits (ns)
   uint64_t full[kRingMax], empty[kRingMax], afull[2], aempty[2], d2full, d2empty, yfull[2], drain;
   uint32_t tslot;
   int abort_flag;
@@ -118,7 +119,7 @@ struct Ctl {
 // Shared by the roles: a bounded wait of a whole warp that records its code.
 __device__ __forceinline__ bool role_wait(uint64_t *bar, uint32_t parity, Ctl *ct, int *err,
                                           int code) {
-  const bool ok = warp_wait(bar, parity, kWaitLimitNs) && !*(volatile int *)&ct->abort_flag;
+  const bool ok = warp_wait(bar, parity, ct->lim) && !*(volatile int *)&ct->abort_flag;
   if (__all_sync(0xffffffffu, ok)) return true;
   if ((threadIdx.x & 31) == 0) atomicExch(err, code);
   *(volatile int *)&ct->abort_flag = 1;
@@ -129,7 +130,8 @@ __device__ __forceinline__ void warp_arrive(uint64_t *bar) {
   if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
 }
 
-__device__ __forceinline__ void ctl_init(Ctl *ct, int full_arrivals) {
+__device__ __forceinline__ void ctl_init(Ctl *ct, int full_arrivals, const int *err) {
+  ct->lim = wait_limit(err);
   for (int i = 0; i < kRingMax; ++i) {
     mbar_init(&ct->full[i], full_arrivals);
     mbar_init(&ct->empty[i], 1);
@@ -176,7 +178,7 @@ __device__ __forceinline__ void ring_producer(Ctl *ct, uint8_t *ring, const CUte
     for (int c = 0; c < nc && ok; ++c)
       for (int p = 0; p < planes; ++p, ++g) {
         const int s = g % kRing;
-        if (!mbar_wait(&ct->empty[s], ((uint32_t)(g / kRing) & 1u) ^ 1u) ||
+        if (!mbar_wait(&ct->empty[s], ((uint32_t)(g / kRing) & 1u) ^ 1u, ct->lim) ||
             *(volatile int *)&ct->abort_flag) {
           atomicExch(err, 41);
           *(volatile int *)&ct->abort_flag = 1;
@@ -303,7 +305,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int W = tc.width, nc = (W + 63) / 64;
   const int n_tiles = (int)((rows + MT - 1) / MT);
-  if (threadIdx.x == 0) ctl_init(ct, 1);
+  if (threadIdx.x == 0) ctl_init(ct, 1, err);
   for (int i = threadIdx.x; i < MW; i += kThreads) {
     sb1[i] = tc.vec[i];
     sb2[i] = tc.vec[MW + i];
@@ -433,6 +435,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (ok && lt > 0) output(lt - 1, (int64_t)blockIdx.x + (int64_t)(lt - 1) * gridDim.x);
   }
   tmem_close(tmem, warp);
+  if (*(volatile int *)&ct->abort_flag) {
+    // (all roles have ended) nothing of this CTA passes for an output
+    for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+      const int64_t y0 = t * MT * tc.n_out, y1 = min(rows, (t + 1) * MT) * tc.n_out;
+      for (int64_t i = y0 + threadIdx.x; i < y1; i += kThreads) Y[i] = __int_as_float(0x7FC00000);
+    }
+  }
 }
 
 constexpr size_t kDh1Smem =
@@ -452,7 +461,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int W = tc.width, nc = (W + 63) / 64, no = tc.n_out;
   const int n_tiles = (int)((rows + MT - 1) / MT);
-  if (threadIdx.x == 0) ctl_init(ct, 1);
+  if (threadIdx.x == 0) ctl_init(ct, 1, err);
   for (int i = threadIdx.x; i < kMlpMaxOut * MW; i += kThreads) sw3[i] = tc.vec[2 * MW + i];
   const uint32_t tmem = tmem_open(ct, warp);
   if (warp == 0) {
@@ -572,7 +581,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int64_t n_blk = (rows + kDwRows - 1) / kDwRows, step = gridDim.x >> 1,
                 b0 = blockIdx.x >> 1;
   const int n_mine = (int)((n_blk - b0 + step - 1) / step);   // >= 1
-  if (threadIdx.x == 0) ctl_init(ct, kEpiWarps);
+  if (threadIdx.x == 0) ctl_init(ct, kEpiWarps, err);
   const uint32_t tmem = tmem_open(ct, warp);
   float *pw = part + b0 * tc.part_stride;
   if (warp == 1) {

@@ -19,7 +19,8 @@ struct MlpTc {
   __nv_bfloat16 *w2t = nullptr;    // [3][256][256] planes of W2^T
   float *w1 = nullptr;             // [2][256][12] W1 (float32; rounded to bf16)
   float *vec = nullptr;            // b1, b2, W3 (float32), W3 (rounded to bf16), b3: rows of 256
-  int *err = nullptr;              // error code of the kernels' waits (0: none)
+  int *err = nullptr;              // code of a wait that gave up (0: none), training steps
+                                   // skipped since, 64-bit wait limit in ns (0: 2 s)
   float *part2 = nullptr, *part1 = nullptr;   // per-CTA partial gradients
   int64_t part_stride = 0;
 };

@@ -29,6 +29,7 @@ void ctx_set_error(tddft_ctx *c, const char *msg);
 int ctx_slots(const tddft_ctx *c);
 int ctx_guess_mode(const tddft_ctx *c);
 tddft_mlp *ctx_guess_net(const tddft_ctx *c);
+tddft_status mlp_check_waits(tddft_mlp *p);
 tddft_status ctx_polarizability_groups(tddft_ctx *c, int32_t n_omega, const double *omega,
                                        double eps, const double *x0, double *X, double *P,
                                        tddft_solve_stats *stats, int32_t flags);
@@ -466,7 +467,14 @@ tddft_status sweep_polarizability(tddft_ctx *c, int32_t n_omega, const double *o
       if (e != cudaSuccess) return cuda_fail(e);
       const tddft_status s2 = ctx_polarizability_groups(c, m, d_om, eps, guess, Xp, Pp, cst.data(),
                                                         TDDFT_DEVICE_PTRS);
+      // (the solve has synchronised: whether the guesses' network gave up a wait)
+      const tddft_status waits =
+          guess && mode == TDDFT_GUESS_LEARNED ? mlp_check_waits(net) : TDDFT_OK;
       if (s2 != TDDFT_OK && s2 != TDDFT_ERR_NOT_CONVERGED) return s2;
+      if (waits != TDDFT_OK) {
+        ctx_set_error(c, (std::string("learned guess: ") + tddft_mlp_last_error(net)).c_str());
+        return waits;
+      }
       if (s2 == TDDFT_ERR_NOT_CONVERGED) all_conv = false;
       // scatter the chunk's solutions, P and statistics to their frequencies
       for (int w = 0; w < m && e == cudaSuccess; ++w) {

@@ -556,6 +556,8 @@ tddft_status tddft_set_wait_timeout(tddft_ctx *c, int64_t ns) {
   c->err.clear();
   if (ns < 0) return fail(c, TDDFT_ERR_INVALID_ARG, "wait_timeout_ns must be >= 0");
   CUDA_TRY(c, set_wait_limit(c, ns));
+  if (c->guess_net && tddft_mlp_set_wait_timeout(c->guess_net, ns) != TDDFT_OK)
+    return fail(c, TDDFT_ERR_CUDA, tddft_mlp_last_error(c->guess_net));
   c->opts.wait_timeout_ns = ns;
   return TDDFT_OK;
 }
@@ -1097,6 +1099,7 @@ int ctx_slots(const tddft_ctx *c) { return c->wk.slots; }
 const tddft_options *ctx_options(const tddft_ctx *c) { return &c->opts; }
 int ctx_guess_mode(const tddft_ctx *c) { return c->opts.guess; }
 tddft_mlp *ctx_guess_net(const tddft_ctx *c) { return c->guess_net; }
+int64_t ctx_wait_timeout(const tddft_ctx *c) { return c->opts.wait_timeout_ns; }
 void ctx_set_guess_net(tddft_ctx *c, tddft_mlp *net) {
   if (c->guess_net) tddft_mlp_destroy(c->guess_net);
   c->guess_net = net;

@@ -108,6 +108,7 @@ SIGNATURES = {
                                         ctypes.c_int64, ctypes.c_uint64, _P,
                                         ctypes.POINTER(ctypes.c_void_p)]),
     "tddft_mlp_destroy": (None, [_P]),
+    "tddft_mlp_set_wait_timeout": (ctypes.c_int, [_P, ctypes.c_int64]),
     "tddft_mlp_last_error": (ctypes.c_char_p, [_P]),
     "tddft_mlp_num_params": (ctypes.c_int64, [_P]),
     "tddft_mlp_params": (ctypes.c_int, [_P, _P, ctypes.c_int64, ctypes.c_int32]),
@@ -390,7 +391,8 @@ class Context:
         self._check(self._lib.tddft_guess_load(self.h, os.fsencode(path)))
 
     def set_wait_timeout(self, ns: int):
-        """tddft_set_wait_timeout: the limit of the tensor-core kernels' waits (0 = 2 s)."""
+        """tddft_set_wait_timeout: the limit of the tensor-core kernels' waits (0 = 2 s), the
+        loaded guess network's among them."""
         self._check(self._lib.tddft_set_wait_timeout(self.h, int(ns)))
 
     def kproduct_plan(self, n_rhs: int):
@@ -532,6 +534,10 @@ class Mlp:
     def _check(self, st):
         if st != OK:
             raise TddftError(st, self._lib.tddft_mlp_last_error(self.h).decode())
+
+    def set_wait_timeout(self, ns: int):
+        """tddft_mlp_set_wait_timeout: the limit of the network kernels' waits (0 = 2 s)."""
+        self._check(self._lib.tddft_mlp_set_wait_timeout(self.h, int(ns)))
 
     def get_params(self) -> np.ndarray:
         p = np.empty(self.n_params, dtype=np.float32)
