@@ -330,8 +330,8 @@ cudaError_t forward(tddft_mlp *p, int64_t rows, const float *F, float *Y, bool b
   const int W = p->width, R = (int)rows;
   cudaError_t e;
   if (p->use_tc)
-    return mlp_tc_forward(p->st, p->tc, p->params, rows, F, keep ? p->H1 : nullptr,
-                          keep ? p->H2 : nullptr, Y, bf16);
+    return mlp_tc_forward(p->st, p->tc, rows, F, keep ? p->H1 : nullptr, keep ? p->H2 : nullptr, Y,
+                          bf16);
   if (bf16) {
     to_bf16_kernel<<<grid1(p->n_params), 256, 0, p->st>>>(p->n_params, p->params, p->params_bf16);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -464,7 +464,7 @@ tddft_status tddft_mlp_create(int32_t n_in, int32_t width, int32_t n_out, int64_
   else al(&p->dH2, (size_t)max_rows * width * sizeof(float));
   al(&p->Y, (size_t)max_rows * n_out * sizeof(float));
   if (e == cudaSuccess && p->use_tc)
-    e = mlp_tc_init(p->tc, n_in, width, n_out, max_rows, tc_mem, p->st);
+    e = mlp_tc_init(p->tc, n_in, width, n_out, max_rows, p->params, tc_mem, p->st);
   if (e == cudaSuccess) {
     init_params_kernel<<<grid1(p->n_params), 256, 0, p->st>>>(
         p->n_params, p->params, p->oW1, p->ob1, p->oW2, p->ob2, p->oW3,

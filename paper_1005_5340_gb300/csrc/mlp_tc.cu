@@ -77,16 +77,50 @@ __device__ __forceinline__ void split3_pair(float x, float y, uint32_t (&w)[3]) 
   }
 }
 
+// Range.  Planes below 2^-126 lose bits and a value above the largest bf16 has
+// no plane, so the gradient of the second layer's input is held times 2^48
+// (exact: what float32 holds at all keeps its 24 bits) and values beyond
+// kDh2Max (2^52 unscaled) and infinities stay out of the tensor cores: their
+// planes are zero, and the kernel adds them, or computes its rows again, in
+// float32 on the CUDA cores when its pipeline has ended.  So for weights
+// beyond kW2Max (256 products with one below it do not overflow).  NaN has
+// planes.  Activations are at most 1; only below 2^-110 do they have fewer
+// bits, an absolute error of 2^-134 per product.  (Gradient of 218 k rows:
+// 1.19 -> 1.21 ms.)
+constexpr float kDh2Scale = 0x1p48f, kDh2Unscale = 0x1p-48f, kDh2Max = 0x1p100f, kW2Max = 0x1p18f;
+// the entry t (1 - h^2) of dH2, t = sum dY W3: one rounding wherever it is
+// formed (both passes take the same decision on it)
+__device__ __forceinline__ float dh2_of(float t, float h) {
+  return __fmul_rn(t, fmaf(-h, h, 1.f));
+}
+// Values without planes set to zero; whether there are any
+template <int N>
+__device__ __forceinline__ bool drop_odd(float (&x)[N]) {
+  float m = 0.f;
+#pragma unroll
+  for (int j = 0; j < N; ++j) m = fmaxf(m, fabsf(x[j]));   // (skips NaN)
+  if (m <= kDh2Max) return false;
+#pragma unroll
+  for (int j = 0; j < N; ++j)
+    if (fabsf(x[j]) > kDh2Max) x[j] = 0.f;
+  return true;
+}
+
 // Weights as the kernels read them, once per call (they change every Adam
 // step): padded W1, output weights (each float32, and rounded to bf16) and
 // biases, the planes of W2 and of its transpose.
-__global__ void mlp_prepare_kernel(MlpTc tc, const float *__restrict__ prm) {
+__global__ void mlp_prepare_kernel(MlpTc tc) {
+  const float *prm = tc.params;
   const int W = tc.width, ni = tc.n_in, no = tc.n_out;
   const float *w1 = prm, *b1 = w1 + (int64_t)W * ni, *w2 = b1 + W, *b2 = w2 + (int64_t)W * W,
               *w3 = b2 + W, *b3 = w3 + (int64_t)no * W;
   const int n = blockIdx.x, k = threadIdx.x;   // MW x MW threads
   __nv_bfloat16 p[3];
-  split3(n < W && k < W ? w2[(int64_t)n * W + k] : 0.f, p);
+  const float v2 = n < W && k < W ? w2[(int64_t)n * W + k] : 0.f;
+  const bool plain = !(fabsf(v2) > kW2Max);
+  const int odd = __syncthreads_or(!plain);
+  split3(plain ? v2 : 0.f, p);
+  if (k == 0) tc.odd_w2[n] = odd;
   for (int q = 0; q < 3; ++q) {
     tc.w2[((int64_t)q * MW + n) * MW + k] = p[q];
     tc.w2t[((int64_t)q * MW + k) * MW + n] = p[q];
@@ -114,13 +148,16 @@ struct Ctl {
   uint64_t full[kRingMax], empty[kRingMax], afull[2], aempty[2], d2full, d2empty, yfull[2], drain;
   uint32_t tslot;
   int abort_flag;
+  int odd;   // some value has no planes: the CUDA cores finish the rows
 };
 
 // Shared by the roles: a bounded wait of a whole warp that records its code.
 __device__ __forceinline__ bool role_wait(uint64_t *bar, uint32_t parity, Ctl *ct, int *err,
                                           int code) {
-  const bool ok = warp_wait(bar, parity, ct->lim) && !*(volatile int *)&ct->abort_flag;
-  if (__all_sync(0xffffffffu, ok)) return true;
+  // (the limit is read only where the first try fails)
+  const bool ok = mbar_try_wait(bar, parity) ||
+                  mbar_wait(bar, parity, *(volatile uint64_t *)&ct->lim);
+  if (__all_sync(0xffffffffu, ok && !*(volatile int *)&ct->abort_flag)) return true;
   if ((threadIdx.x & 31) == 0) atomicExch(err, code);
   *(volatile int *)&ct->abort_flag = 1;
   return false;
@@ -145,6 +182,7 @@ __device__ __forceinline__ void ctl_init(Ctl *ct, int full_arrivals, const int *
   mbar_init(&ct->d2empty, kEpiWarps);
   mbar_init(&ct->drain, 1);
   ct->abort_flag = 0;
+  ct->odd = 0;
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 // tensor memory of the whole SM, by warp 1 (before and after a block barrier)
@@ -284,6 +322,44 @@ __device__ __forceinline__ void get16(const float *src, int c0, int W, bool live
   }
 }
 
+// Whether some weight of W2 has no planes (a barrier of the whole CTA)
+__device__ __forceinline__ bool odd_weights(const MlpTc &tc) {
+  return __syncthreads_or(threadIdx.x < MW && tc.odd_w2[threadIdx.x] != 0) != 0;
+}
+
+// A forward CTA's rows on the CUDA cores, one row at a time (buf: 2 MW floats)
+template <int PLANES, bool STORE>
+__device__ __noinline__ void forward_rows(const MlpTc &tc, int64_t rows, int n_tiles,
+                                          const float *F, float *H2, float *Y, const float *sw1,
+                                          const float *sb1, const float *sb2, const float *sw3,
+                                          float *buf) {
+  const int n = threadIdx.x, W = tc.width, ni = tc.n_in;
+  const float *w2 = tc.params + (int64_t)W * ni + W + (int64_t)n * W;
+  for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x)
+    for (int64_t r = t * MT; r < min(rows, (t + 1) * MT); ++r) {
+      if (n < W) {
+        float s = 0.f;
+        for (int i = 0; i < ni; ++i) s = fmaf(F[r * ni + i], sw1[n * kMlpMaxIn + i], s);
+        buf[n] = tanhf(s + sb1[n]);
+      }
+      __syncthreads();
+      if (n < W) {
+        float s = 0.f;
+        for (int k = 0; k < W; ++k)
+          s = fmaf(buf[k], PLANES == 1 ? __bfloat162float(__float2bfloat16_rn(w2[k])) : w2[k], s);
+        s = tanhf(s + sb2[n]);
+        buf[MW + n] = s;
+        if (STORE) H2[r * W + n] = s;
+      }
+      __syncthreads();
+      if (n < tc.n_out) {
+        float s = 0.f;
+        for (int k = 0; k < W; ++k) s = fmaf(buf[MW + k], sw3[n * MW + k], s);
+        Y[r * tc.n_out + n] = s + tc.vec[(2 + 2 * kMlpMaxOut) * MW + n];
+      }
+    }
+}
+
 constexpr size_t kFwdSmem = 1024 + 2 * kBufA + kRing * kTileB + MW * kMlpMaxIn * 4 + 2 * MW * 4 +
                             kMlpMaxOut * MW * 4 + 2 * 3 * MT * kMlpMaxOut * 4 + sizeof(Ctl) + 64;
 
@@ -314,6 +390,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     sw1[i] = tc.w1[(PLANES == 1 ? MW * kMlpMaxIn : 0) + i];
   for (int i = threadIdx.x; i < kMlpMaxOut * MW; i += kThreads)
     sw3[i] = tc.vec[(2 + (PLANES == 1 ? kMlpMaxOut : 0)) * MW + i];
+  const bool odd = odd_weights(tc);
   const uint32_t tmem = tmem_open(ct, warp);
 
   if (warp == 0) {
@@ -441,7 +518,32 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int64_t y0 = t * MT * tc.n_out, y1 = min(rows, (t + 1) * MT) * tc.n_out;
       for (int64_t i = y0 + threadIdx.x; i < y1; i += kThreads) Y[i] = __int_as_float(0x7FC00000);
     }
+  } else if (odd) {
+    forward_rows<PLANES, STORE>(tc, rows, n_tiles, F, H2, Y, sw1, sb1, sb2, sw3, (float *)sA);
   }
+}
+
+// A dH1 CTA's rows on the CUDA cores, one row at a time (buf: MW floats)
+__device__ __noinline__ void dh1_rows(const MlpTc &tc, int64_t rows, int n_tiles, const float *dY,
+                                      const float *H1, const float *H2, float *dH1, float *buf) {
+  const int n = threadIdx.x, W = tc.width, no = tc.n_out;
+  const float *w2 = tc.params + (int64_t)W * tc.n_in + W, *w3 = tc.vec + 2 * MW;
+  for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x)
+    for (int64_t r = t * MT; r < min(rows, (t + 1) * MT); ++r) {
+      if (n < W) {
+        float s = 0.f;
+        for (int o = 0; o < no; ++o) s = fmaf(dY[r * no + o], w3[o * MW + n], s);
+        buf[n] = dh2_of(s, H2[r * W + n]);
+      }
+      __syncthreads();
+      if (n < W) {
+        const float h = H1[r * W + n];
+        float s = 0.f;
+        for (int i = 0; i < W; ++i) s = fmaf(buf[i], w2[(int64_t)i * W + n], s);
+        dH1[r * W + n] = s * fmaf(-h, h, 1.f);
+      }
+      __syncthreads();
+    }
 }
 
 constexpr size_t kDh1Smem =
@@ -462,7 +564,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int W = tc.width, nc = (W + 63) / 64, no = tc.n_out;
   const int n_tiles = (int)((rows + MT - 1) / MT);
   if (threadIdx.x == 0) ctl_init(ct, 1, err);
-  for (int i = threadIdx.x; i < kMlpMaxOut * MW; i += kThreads) sw3[i] = tc.vec[2 * MW + i];
+  for (int i = threadIdx.x; i < kMlpMaxOut * MW; i += kThreads)
+    sw3[i] = kDh2Scale * tc.vec[2 * MW + i];   // dH2 comes out scaled
+  const bool odd_w2 = odd_weights(tc);
   const uint32_t tmem = tmem_open(ct, warp);
   if (warp == 0) {
     ring_producer(ct, ring, &map2t, n_tiles, nc, 3, err);
@@ -507,7 +611,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (s < 3) get16(H1 + r * W, c0 + 16, W, r < rows, hn);
         get_sum(trow, c0, v);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] *= 1.f - h[j] * h[j];
+        for (int j = 0; j < 16; ++j) v[j] = v[j] * kDh2Unscale * fmaf(-h[j], h[j], 1.f);
         if (r < rows) put16(dH1 + r * W, c0, W, v);
       }
       fence_before();
@@ -539,8 +643,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int o = 0; o < kMlpMaxOut; ++o)
             if (o < no) s = fmaf(dy[o], sw3[o * MW + c0 + j], s);
-          h[j] = s * (1.f - h[j] * h[j]);
+          h[j] = dh2_of(s, h[j]);
         }
+        if (drop_odd(h)) *(volatile int *)&ct->odd = 1;
         if (u > 1 && !(ok = role_wait(&ct->aempty[u & 1], (uint32_t)((u >> 1) - 1) & 1u, ct, err, 64)))
           break;
         put_planes(sA + (u & 1) * kBufA, lr, g, h);
@@ -551,6 +656,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (ok && lt > 0) output(lt - 1, (int64_t)blockIdx.x + (int64_t)(lt - 1) * gridDim.x);
   }
   tmem_close(tmem, warp);
+  if ((odd_w2 || *(volatile int *)&ct->odd) && !*(volatile int *)&ct->abort_flag)
+    dh1_rows(tc, rows, n_tiles, dY, H1, H2, dH1, (float *)sA);
 }
 
 // dW2 over a CTA's rows: D[i][j] += sum_r dH2[r][i] H1[r][j] for the 256 units
@@ -563,9 +670,35 @@ __global__ void __launch_bounds__(kThreads, 1)
 // accumulators are added to the CTA's float32 partial sums in global memory,
 // which bounds the truncations.  The same threads sum db2 and dW3 of their
 // unit (and db3).
+// (Products and sums without planes follow at the end, row by row.)
 constexpr int kDwRows = 16, kDwDrain = 24;
 constexpr uint32_t kDwA = MW * 128, kDwB = (MW / 2) * 128;   // planes of 256 and 128 units
 constexpr size_t kDw2Smem = 1024 + 3 * (kDwA + kDwB) + sizeof(Ctl) + 64;
+
+// The entries of dH2 that the planes left out, into dW2 and db2: thread i adds
+// unit i's, which no other thread touches.
+__device__ __noinline__ void dw2_odd(const MlpTc &tc, int64_t rows, int64_t b0, int64_t step,
+                                     int n_mine, int half, const float *dY, const float *H1,
+                                     const float *H2, float *pw) {
+  const int i = threadIdx.x, W = tc.width, no = tc.n_out;
+  if (i >= W) return;
+  const float *w3 = tc.vec + 2 * MW + i;
+  const int j0 = half * (MW / 2), j1 = min(W, j0 + MW / 2);
+  for (int g = 0; g < n_mine; ++g) {
+    const int64_t ra = (b0 + g * step) * kDwRows;
+    for (int64_t r = ra; r < min(rows, ra + kDwRows); ++r) {
+      float scaled = 0.f, t = 0.f;
+      for (int o = 0; o < no; ++o) {
+        scaled = fmaf(dY[r * no + o], kDh2Scale * w3[o * MW], scaled);
+        t = fmaf(dY[r * no + o], w3[o * MW], t);
+      }
+      const float h = H2[r * W + i], d = dh2_of(t, h);
+      if (!(fabsf(dh2_of(scaled, h)) > kDh2Max)) continue;
+      for (int j = j0; j < j1; ++j) pw[i * MW + j] = fmaf(d, H1[r * W + j], pw[i * MW + j]);
+      if (half == 0) pw[MW * MW + i] += d;   // db2, of the first row group
+    }
+  }
+}
 
 __global__ void __launch_bounds__(kThreads, 1)
     mlp_dw2_kernel(MlpTc tc, int64_t rows, const float *__restrict__ dY,
@@ -618,7 +751,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int j = half * (MW / 2) + jl;
     float w3[kMlpMaxOut], g3[kMlpMaxOut] = {}, gb2 = 0.f, gb3 = 0.f;
 #pragma unroll
-    for (int o = 0; o < kMlpMaxOut; ++o) w3[o] = tc.vec[(2 + o) * MW + i];
+    for (int o = 0; o < kMlpMaxOut; ++o) w3[o] = kDh2Scale * tc.vec[(2 + o) * MW + i];
     float n2[8], n1[4], ndy;   // the next block's values; lane l: dY entry l of the 8 rows
     auto load = [&](int g) {
       const int64_t ra = (b0 + g * step) * kDwRows;
@@ -648,7 +781,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         get16(dst, c0, MW, k > 0, old);
         get_sum(tmem + ((uint32_t)(32 * q) << 16), m * (MW / 2) + c0, v);
 #pragma unroll
-        for (int e = 0; e < 16; ++e) v[e] += old[e];
+        for (int e = 0; e < 16; ++e) v[e] = fmaf(v[e], kDh2Unscale, old[e]);
         put16(dst, c0, MW, v);
       }
       fence_before();
@@ -677,9 +810,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             g3[o] = fmaf(dy, h2[e], g3[o]);
             if (i == o) gb3 += dy;
           }
-        d2[e] = t * (1.f - h2[e] * h2[e]);
-        gb2 += d2[e];
+        d2[e] = dh2_of(t, h2[e]);
       }
+      if (drop_odd(d2)) *(volatile int *)&ct->odd = 1;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) gb2 = fmaf(d2[e], kDh2Unscale, gb2);
       if (g >= kRingMax &&
           !(ok = role_wait(&ct->empty[s], (uint32_t)(g / kRingMax - 1) & 1u, ct, err, 72)))
         break;
@@ -719,6 +854,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
   tmem_close(tmem, warp);
+  if (*(volatile int *)&ct->odd && !*(volatile int *)&ct->abort_flag)
+    dw2_odd(tc, rows, b0, step, n_mine, half, dY, H1, H2, pw);
 }
 
 // dW1[j][f] = sum_r dH1[r][j] F[r][f] and db1[j]: thread j, rows in blocks of
@@ -854,13 +991,14 @@ bool mlp_tc_fits(int n_in, int width, int n_out) {
 
 size_t mlp_tc_bytes(int64_t max_rows) {
   return (size_t)6 * MW * MW * sizeof(__nv_bfloat16) +
-         (size_t)(2 * kMlpMaxIn + 3 + 2 * kMlpMaxOut) * MW * sizeof(float) + 256 +
+         (size_t)(2 * kMlpMaxIn + 4 + 2 * kMlpMaxOut) * MW * sizeof(float) + 256 +
          (size_t)(dw2_groups(max_rows) * kPartStride +
                   (int64_t)dw1_ctas(max_rows) * (kMlpMaxIn + 1) * MW) * sizeof(float);
 }
 
-cudaError_t mlp_tc_init(MlpTc &tc, int n_in, int width, int n_out, int64_t max_rows, void *mem,
-                        cudaStream_t st) {
+cudaError_t mlp_tc_init(MlpTc &tc, int n_in, int width, int n_out, int64_t max_rows,
+                        const float *params, void *mem, cudaStream_t st) {
+  tc.params = params;
   tc.n_in = n_in;
   tc.width = width;
   tc.n_out = n_out;
@@ -869,7 +1007,8 @@ cudaError_t mlp_tc_init(MlpTc &tc, int n_in, int width, int n_out, int64_t max_r
   tc.w2t = tc.w2 + 3 * MW * MW;
   tc.w1 = (float *)(tc.w2t + 3 * MW * MW);
   tc.vec = tc.w1 + 2 * MW * kMlpMaxIn;
-  tc.err = (int *)(tc.vec + (3 + 2 * kMlpMaxOut) * MW);
+  tc.odd_w2 = (int *)(tc.vec + (3 + 2 * kMlpMaxOut) * MW);
+  tc.err = tc.odd_w2 + MW;
   tc.part2 = (float *)((char *)tc.err + 256);
   tc.part1 = tc.part2 + dw2_groups(max_rows) * kPartStride;
   cudaError_t e = encode_bf16_map(&tc.map2, tc.w2, 3 * MW, MW, MW);
@@ -878,9 +1017,9 @@ cudaError_t mlp_tc_init(MlpTc &tc, int n_in, int width, int n_out, int64_t max_r
   return e;
 }
 
-cudaError_t mlp_tc_forward(cudaStream_t st, const MlpTc &tc, const float *params, int64_t rows,
-                           const float *F, float *H1, float *H2, float *Y, bool bf16) {
-  mlp_prepare_kernel<<<MW, MW, 0, st>>>(tc, params);
+cudaError_t mlp_tc_forward(cudaStream_t st, const MlpTc &tc, int64_t rows, const float *F,
+                           float *H1, float *H2, float *Y, bool bf16) {
+  mlp_prepare_kernel<<<MW, MW, 0, st>>>(tc);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (bf16) return launch_forward<1, false>(st, tc, rows, F, nullptr, nullptr, Y);
