@@ -167,8 +167,7 @@ __device__ __forceinline__ void warp_arrive(uint64_t *bar) {
   if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
 }
 
-__device__ __forceinline__ void ctl_init(Ctl *ct, int full_arrivals, const int *err) {
-  ct->lim = wait_limit(err);
+__device__ __forceinline__ void ctl_init(Ctl *ct, int full_arrivals) {
   for (int i = 0; i < kRingMax; ++i) {
     mbar_init(&ct->full[i], full_arrivals);
     mbar_init(&ct->empty[i], 1);
@@ -185,8 +184,10 @@ __device__ __forceinline__ void ctl_init(Ctl *ct, int full_arrivals, const int *
   ct->odd = 0;
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
-// tensor memory of the whole SM, by warp 1 (before and after a block barrier)
-__device__ __forceinline__ uint32_t tmem_open(Ctl *ct, int warp) {
+// tensor memory of the whole SM, by warp 1 (before and after a block barrier),
+// and the roles' wait limit
+__device__ __forceinline__ uint32_t tmem_open(Ctl *ct, int warp, uint64_t lim) {
+  if (threadIdx.x == 0) ct->lim = lim;
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
         smem_u32(&ct->tslot)));
@@ -322,9 +323,9 @@ __device__ __forceinline__ void get16(const float *src, int c0, int W, bool live
   }
 }
 
-// Whether some weight of W2 has no planes (a barrier of the whole CTA)
-__device__ __forceinline__ bool odd_weights(const MlpTc &tc) {
-  return __syncthreads_or(threadIdx.x < MW && tc.odd_w2[threadIdx.x] != 0) != 0;
+// This thread's share of whether some weight of W2 has no planes
+__device__ __forceinline__ int odd_weight(const MlpTc &tc) {
+  return threadIdx.x < MW ? tc.odd_w2[threadIdx.x] : 0;
 }
 
 // A forward CTA's rows on the CUDA cores, one row at a time (buf: 2 MW floats)
@@ -373,6 +374,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                        const float *__restrict__ F, float *__restrict__ H1,
                        float *__restrict__ H2, float *__restrict__ Y, int *err) {
   extern __shared__ uint8_t smem_raw[];
+  const uint64_t lim = wait_limit(err);   // (loaded ahead of their use)
+  const int odd_w = odd_weight(tc);
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *sA = smem, *ring = sA + 2 * kBufA;
   float *sw1 = (float *)(ring + kRing * kTileB), *sb1 = sw1 + MW * kMlpMaxIn, *sb2 = sb1 + MW,
@@ -381,7 +384,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int W = tc.width, nc = (W + 63) / 64;
   const int n_tiles = (int)((rows + MT - 1) / MT);
-  if (threadIdx.x == 0) ctl_init(ct, 1, err);
+  if (threadIdx.x == 0) ctl_init(ct, 1);
   for (int i = threadIdx.x; i < MW; i += kThreads) {
     sb1[i] = tc.vec[i];
     sb2[i] = tc.vec[MW + i];
@@ -390,8 +393,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     sw1[i] = tc.w1[(PLANES == 1 ? MW * kMlpMaxIn : 0) + i];
   for (int i = threadIdx.x; i < kMlpMaxOut * MW; i += kThreads)
     sw3[i] = tc.vec[(2 + (PLANES == 1 ? kMlpMaxOut : 0)) * MW + i];
-  const bool odd = odd_weights(tc);
-  const uint32_t tmem = tmem_open(ct, warp);
+  const bool odd = __syncthreads_or(odd_w) != 0;
+  const uint32_t tmem = tmem_open(ct, warp, lim);
 
   if (warp == 0) {
     ring_producer(ct, ring, &map2, n_tiles, nc, PLANES, err);
@@ -556,6 +559,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                    const float *__restrict__ dY, const float *__restrict__ H1,
                    const float *__restrict__ H2, float *__restrict__ dH1, int *err) {
   extern __shared__ uint8_t smem_raw[];
+  const uint64_t lim = wait_limit(err);
+  const int odd_w = odd_weight(tc);
   uint8_t *sA = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *ring = sA + 2 * kBufA;
   float *sw3 = (float *)(ring + kRing * kTileB);
@@ -563,11 +568,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int W = tc.width, nc = (W + 63) / 64, no = tc.n_out;
   const int n_tiles = (int)((rows + MT - 1) / MT);
-  if (threadIdx.x == 0) ctl_init(ct, 1, err);
+  if (threadIdx.x == 0) ctl_init(ct, 1);
   for (int i = threadIdx.x; i < kMlpMaxOut * MW; i += kThreads)
     sw3[i] = kDh2Scale * tc.vec[2 * MW + i];   // dH2 comes out scaled
-  const bool odd_w2 = odd_weights(tc);
-  const uint32_t tmem = tmem_open(ct, warp);
+  const bool odd_w2 = __syncthreads_or(odd_w) != 0;
+  const uint32_t tmem = tmem_open(ct, warp, lim);
   if (warp == 0) {
     ring_producer(ct, ring, &map2t, n_tiles, nc, 3, err);
     __syncwarp();
@@ -705,6 +710,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                    const float *__restrict__ H1, const float *__restrict__ H2,
                    float *__restrict__ part, int *err) {
   extern __shared__ uint8_t smem_raw[];
+  const uint64_t lim = wait_limit(err);
   uint8_t *sa = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *sb = sa + 3 * kDwA;
   Ctl *ct = (Ctl *)(sb + 3 * kDwB);
@@ -714,8 +720,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int64_t n_blk = (rows + kDwRows - 1) / kDwRows, step = gridDim.x >> 1,
                 b0 = blockIdx.x >> 1;
   const int n_mine = (int)((n_blk - b0 + step - 1) / step);   // >= 1
-  if (threadIdx.x == 0) ctl_init(ct, kEpiWarps, err);
-  const uint32_t tmem = tmem_open(ct, warp);
+  if (threadIdx.x == 0) ctl_init(ct, kEpiWarps);
+  const uint32_t tmem = tmem_open(ct, warp, lim);
   float *pw = part + b0 * tc.part_stride;
   if (warp == 1) {
     constexpr uint32_t idesc = idesc_bf16(MT, MW / 2);
