@@ -329,7 +329,13 @@ tddft_status mfail(tddft_mlp *p, tddft_status s, const std::string &msg) {
 cudaError_t forward(tddft_mlp *p, int64_t rows, const float *F, float *Y, bool bf16, bool keep) {
   const int W = p->width, R = (int)rows;
   cudaError_t e;
-  if (p->use_tc)
+  // The tensor-core kernels have a floor of two dependent launches with their
+  // set-up, so narrow networks of few rows keep the three small CUDA-core
+  // launches for float32 inference: 8 units, 280 rows 16.8 against 18.9 us, 16
+  // units, 3000 rows 16.9 against 18.9 (30000 rows: 23 each, 218000: 80 against
+  // 65; 32 units: 19 to 21 each).  bf16 weights take one launch more there.
+  const bool narrow = !keep && !bf16 && p->width <= 16 && rows <= 16384;
+  if (p->use_tc && !narrow)
     return mlp_tc_forward(p->st, p->tc, rows, F, keep ? p->H1 : nullptr, keep ? p->H2 : nullptr, Y,
                           bf16);
   if (bf16) {
