@@ -134,12 +134,12 @@ cudaError_t launch_block_dot(cudaStream_t st, int ncols, const DevSystem &sys,
                                                gamma, Zin, subtract, Out, dcnt);
     return cudaGetLastError();
   };
-  // as many columns per CTA as leave about four CTAs per SM (152)
+  // as many columns per CTA as leave about four CTAs per SM
   auto ctas = [&](int bc) { return (int64_t)sys.n_blocks * ((ncols + bc - 1) / bc); };
-  constexpr int64_t kWant = 4 * 152;
-  if (ctas(8) >= kWant) return go(std::integral_constant<int, 8>{});
-  if (ctas(4) >= kWant) return go(std::integral_constant<int, 4>{});
-  if (ctas(2) >= kWant) return go(std::integral_constant<int, 2>{});
+  const int64_t want = 4 * (int64_t)sm_count();
+  if (ctas(8) >= want) return go(std::integral_constant<int, 8>{});
+  if (ctas(4) >= want) return go(std::integral_constant<int, 4>{});
+  if (ctas(2) >= want) return go(std::integral_constant<int, 2>{});
   return go(std::integral_constant<int, 1>{});
 }
 

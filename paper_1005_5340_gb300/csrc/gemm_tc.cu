@@ -836,26 +836,16 @@ void set_attr_all() {
 }  // namespace
 
 void tc_init_attributes() {
-  static bool done = false;
-  if (done) return;
-  set_attr_all<128>();
-  set_attr_all<64>();
-  set_attr_all<256>();
-  done = true;
+  static PerDevice done;
+  done.get([] {
+    set_attr_all<128>();
+    set_attr_all<64>();
+    set_attr_all<256>();
+    return 1;
+  });
 }
 
 namespace {
-int sm_count() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-      n = 1;
-  }
-  return n;
-}
-
 template <int EPI, int BN, bool TF>
 cudaError_t launch_tc(cudaStream_t st, int64_t work, const CUtensorMap &mA, const CUtensorMap &mB,
                       const CUtensorMap &mB64, const CUtensorMap &mB128, int M, int N, int KpA,
@@ -882,24 +872,26 @@ cudaError_t launch_tc(cudaStream_t st, int64_t work, const CUtensorMap &mA, cons
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  static int fit[5] = {0, 0, 0, 0, 0};   // co-resident clusters per cluster size
+  static PerDevice fits[5];   // co-resident clusters per cluster size
   if (ep.ncl > 4) return cudaErrorInvalidValue;
-  if (fit[ep.ncl] == 0) {
-    cfg.gridDim = dim3(ep.ncl * sm_count());
+  const int fit = fits[ep.ncl].get([&] {
+    cfg.gridDim = dim3(ep.ncl * sms);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_kernel<EPI, BN, TF>, &cfg) != cudaSuccess ||
-        n < 1)
-      return cudaErrorInvalidConfiguration;
-    fit[ep.ncl] = n;
+    return cudaOccupancyMaxActiveClusters(&n, gemm_tc_kernel<EPI, BN, TF>, &cfg) == cudaSuccess
+               ? n : 0;
+  });
+  if (fit < 1) {
+    cudaGetLastError();
+    return plain();
   }
   // Clusters of 3 or 4 leave SMs without one (46 and 36 clusters fit on 152
   // SMs): where that costs a fifth more waves or above, single CTAs in the
   // same tile order instead.  64 atoms, 384 columns: 142 clusters, 4 waves
   // against 3, 160 us against 127; 128 atoms: 7 against 6, 702 us against 710
   // (without the cluster an A tile is fetched by both dies).
-  const int64_t wc = (work / ep.ncl + fit[ep.ncl] - 1) / fit[ep.ncl], wp = (work + sms - 1) / sms;
+  const int64_t wc = (work / ep.ncl + fit - 1) / fit, wp = (work + sms - 1) / sms;
   if (5 * wp <= 4 * wc) return plain();
-  cfg.gridDim = dim3(std::min(grid / ep.ncl, fit[ep.ncl]) * ep.ncl);
+  cfg.gridDim = dim3(std::min(grid / ep.ncl, fit) * ep.ncl);
   return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<EPI, BN, TF>, mA, mB, mB64, mB128, M, N, KpA, KpB,
                             ep, err, dcnt, mul_n, tiles, n_mtiles);
 }

@@ -2,6 +2,7 @@
 // Nothing here crosses the C boundary (include/tddft.h).
 #pragma once
 
+#include <atomic>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -223,6 +224,25 @@ void tc_split_plan(int Kp, int M, int N, int bn, int *ksplit, int *ncl);
 // gives back what the pools keep.
 cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st);
 void scratch_trim();
+
+// A positive number per device, found on first use.  Safe from several threads
+// (two that ask at once both find the same number); a failure (find gives 0
+// or less) is returned but not kept.
+struct PerDevice {
+  static constexpr int kMax = 128;
+  std::atomic<int> known[kMax] = {};
+  template <class F>
+  int get(F &&find) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMax) return find();
+    int v = known[dev].load(std::memory_order_acquire);
+    if (v > 0) return v;
+    v = find();
+    if (v > 0) known[dev].store(v, std::memory_order_release);
+    return v;
+  }
+};
+int sm_count();   // SMs of the current device (1 if it cannot be asked)
 
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 

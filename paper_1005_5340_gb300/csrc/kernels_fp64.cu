@@ -30,16 +30,6 @@ namespace tddft {
 // ---------------------------------------------------------------------------
 namespace {
 
-int sm_count() {
-  static const int n = [] {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0
-               ? v : 1;
-  }();
-  return n;
-}
-
 // ---------------------------------------------------------------------------
 // C[M x N] = A[M x K] . B[K x N], all row-major float64 (DFMA).
 // A BM x BN tile per CTA; the four warps take one K quarter each
@@ -482,7 +472,7 @@ cudaError_t launch_dscale(cudaStream_t st, const DevSystem &sys, int S, const do
   // six columns per thread (two D where the frequencies come in threes, three
   // where a group starts elsewhere), or three where that would leave SMs idle
   const int64_t per = (int64_t)sys.n_virt * sys.n_occ;
-  const bool six = per * ((S + 5) / 6) >= 152 * 1024;
+  const bool six = per * ((S + 5) / 6) >= (int64_t)sm_count() * 1024;
   const int64_t n = (per * (six ? (S + 5) / 6 : (S + 2) / 3) + 127) / 128;
   if (n > INT32_MAX) return cudaErrorInvalidConfiguration;
   auto *kernel = six ? dscale_kernel<6> : dscale_kernel<3>;

@@ -405,7 +405,7 @@ cudaError_t launch_apply_operator_lp(cudaStream_t st, const DevSystem &sys, LpWo
     // two M blocks per tile halve the reads of Gcat; where that leaves SMs
     // without a tile, one M block and 64 columns (an output's K order is the
     // same: same bits)
-    if ((int64_t)ar.n_tiles5lp * ((ncols + 127) / 128) >= 152)
+    if ((int64_t)ar.n_tiles5lp * ((ncols + 127) / 128) >= sm_count())
       err = launch_gemm_tc_grouped(st, ar.a5, ar.gcat, ar.tiles5lp, ar.n_tiles5lp, ncols,
                                    kPartialF32, e5, lp.err, lp.dcnt, 2);
     else

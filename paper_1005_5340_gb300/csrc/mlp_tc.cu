@@ -955,16 +955,6 @@ __global__ void __launch_bounds__(256) mlp_reduce_kernel(MlpTc tc, int n2,
   }
 }
 
-int sm_count() {
-  static const int n = [] {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0
-               ? v : 1;
-  }();
-  return n;
-}
-
 template <class K>
 cudaError_t allow_smem(K k, size_t bytes) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);

@@ -884,9 +884,10 @@ cudaError_t set_smem_attr() {
 
 // Clusters of c CTAs (one CTA per SM) that run at once.  GPCs hold 16 to 20
 // SMs, so 152 SMs take 76 clusters of 2, 36 of 4, 23 of 6, but 15 of 7 or 8.
+// (0 for a size that cannot be asked; single CTAs always run.)
 int active_clusters(int c) {
-  static int fit[9] = {};
-  if (fit[c] == 0) {
+  static PerDevice fits[9];
+  const int fit = fits[c].get([c] {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c * 256);
     cfg.blockDim = dim3(OZ_THREADS);
@@ -903,9 +904,9 @@ int active_clusters(int c) {
       cudaGetLastError();
       n = 0;
     }
-    fit[c] = n > 0 ? n : -1;
-  }
-  return fit[c];
+    return n;
+  });
+  return c == 1 && fit < 1 ? sm_count() : fit;
 }
 
 // Clocks per K block of a tile: an MMA of N columns takes N / 2 at the tensor
@@ -958,16 +959,17 @@ TilePlan tile_plan(int S, int Mt, int N, int nch) {
 // Dynamic shared memory limits of every slice count (once; outside any
 // stream capture).
 cudaError_t oz_init_attributes() {
-  static cudaError_t done = cudaErrorNotReady;
-  if (done == cudaSuccess) return done;
+  static PerDevice done;
   cudaError_t e = cudaSuccess;
-  for (int n = kOzMinSlices; n <= kOzMaxSlices && e == cudaSuccess; ++n)
-    e = with_slices(n, [](auto sc) {
-      constexpr int S = decltype(sc)::value, W = oz_wide_bn(S);
-      const cudaError_t r = set_smem_attr<S, 64>();
-      return W == 64 || r != cudaSuccess ? r : set_smem_attr<S, W>();
-    });
-  done = e;
+  done.get([&e] {
+    for (int n = kOzMinSlices; n <= kOzMaxSlices && e == cudaSuccess; ++n)
+      e = with_slices(n, [](auto sc) {
+        constexpr int S = decltype(sc)::value, W = oz_wide_bn(S);
+        const cudaError_t r = set_smem_attr<S, 64>();
+        return W == 64 || r != cudaSuccess ? r : set_smem_attr<S, W>();
+      });
+    return e == cudaSuccess ? 1 : 0;
+  });
   return e;
 }
 

@@ -49,6 +49,17 @@ cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st) {
   return e != cudaSuccess ? e : cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
+int sm_count() {
+  static PerDevice n;
+  const int v = n.get([] {
+    int dev = 0, sms = 0;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+                   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess
+               ? sms : 0;
+  });
+  return v > 0 ? v : 1;
+}
+
 void scratch_trim() {
   std::lock_guard<std::mutex> lock(g_mutex);
   for (cudaMemPool_t p : g_pool)
