@@ -66,16 +66,6 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, u
       "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(c0), "r"(c1)
       : "memory");
 }
-// K-major operand tile, 128-byte swizzle: rows of 64 bf16 (128 B), 8-row
-// groups 1024 B apart; start address advanced by 32 B per K=16 step.
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
-  uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1 << 16;                 // leading byte offset (unused for SW128 K-major)
-  d |= (uint64_t)(1024 >> 4) << 32;       // stride byte offset: 8 rows x 128 B
-  d |= (uint64_t)1 << 46;                 // descriptor version (tcgen05)
-  d |= (uint64_t)2 << 61;                 // 128-byte swizzle
-  return d;
-}
 // kind::f16 instruction descriptor: D f32, A and B bf16, both K-major.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
@@ -88,34 +78,12 @@ __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) |
          ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc,
-                                         uint32_t accum) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-      "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
-}
 // x rounded to tf32 (10 explicit mantissa bits, to nearest, ties away), as a
 // float whose 13 low mantissa bits are zero
 __device__ __forceinline__ float tf32_round(float x) {
   uint32_t y;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(y) : "f"(x));
   return __uint_as_float(y);
-}
-__device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc,
-                                         uint32_t accum) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-      "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
-}
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_u32(bar))
-      : "memory");
 }
 // One lane of a converged warp (the same one at every call).  A role that
 // issues MMAs runs as a whole warp, with warp-uniform loop state, and only the
@@ -132,11 +100,16 @@ __device__ __forceinline__ uint32_t elect_one() {
       : "=r"(is));
   return is;
 }
-// Low word of desc_sw128 of a shared address (the 14-bit address field never
-// carries: shared memory ends below 2^18), and the descriptor at a low word.
+// Descriptor of a K-major operand tile in shared memory, 128-byte swizzle: rows
+// of 64 bf16 (128 B), 8-row groups 1024 B apart; the start address advances by
+// 32 B per K = 16 step.  Its low word is the address in 16-byte units (14 bits,
+// which never carry: shared memory ends below 2^18) and the leading byte offset
+// (unused in this layout).
 __device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return (saddr >> 4) | (1u << 16); }
 __device__ __forceinline__ uint64_t desc_of(uint32_t lo) {
-  constexpr uint32_t kHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+  constexpr uint32_t kHi = (1024u >> 4)   // stride byte offset: 8 rows x 128 B
+                           | (1u << 14)   // descriptor version (tcgen05)
+                           | (2u << 29);  // 128-byte swizzle
   return ((uint64_t)kHi << 32) | lo;
 }
 __device__ __forceinline__ void mma_bf16_if(uint32_t leader, uint32_t dtmem, uint64_t ad,
