@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "exact.h"
 #include "internal.h"
 #include "tc_ptx.h"
 
@@ -159,16 +160,6 @@ __global__ void __launch_bounds__(256) gather_split_kernel(int ncols, int kcat,
         __floats2bfloat162_rn(x0 - __bfloat162float(h.x), x1 - __bfloat162float(h.y));
   }
 }
-
-// float32 -> float64 in the integer pipe (a conversion would take the FP64
-// pipe's time); subnormals, infinities and NaN convert.
-__device__ __forceinline__ double to_f64(float x) {
-  const unsigned int u = __float_as_uint(x), e = (u >> 23) & 0xFF;
-  if (e == 0xFF || (e == 0 && (u << 1) != 0)) return (double)x;
-  const unsigned int top = (u & 0x80000000u) | (e == 0 ? 0u : ((u & 0x7FFFFFFFu) >> 3) + 0x38000000u);
-  return __hiloint2double((int)top, (int)(u << 29));
-}
-__device__ __forceinline__ double to_f64(double x) { return x; }
 
 // Out = Zin - n or n, n_mu the sum of product mu's one or two partials (first
 // the smaller atom's): tiles of 32 products x 32 columns, the partials read

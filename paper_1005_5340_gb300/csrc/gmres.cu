@@ -25,6 +25,7 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
+#include "exact.h"
 #include "internal.h"
 #include "tc_ptx.h"
 
@@ -51,24 +52,6 @@ __device__ inline double2 cdiv(double2 a, double2 b) {
     double r = b.x / b.y, d = b.y + r * b.x;
     return make_double2((a.x * r + a.y) / d, (a.y * r - a.x) / d);
   }
-}
-
-// n / d, correctly rounded, from inv = 1 / d (itself correctly rounded):
-// remainders correct the product n inv twice, first to within one unit in the
-// last place, then to the rounded quotient (Markstein, IBM J. Res. Dev. 34,
-// 1990); five dependent operations instead of a whole division.  The theorem
-// needs its products clear of under- and overflow and a denominator whose
-// significand is not all ones; others divide.
-__device__ inline double quotient(double n, double d, double inv) {
-  const unsigned en = (unsigned)(__double2hiint(n) >> 20) & 0x7FFu,
-                 ed = (unsigned)(__double2hiint(d) >> 20) & 0x7FFu;
-  const bool plain = en - 400u < 1247u && ed - 400u < 1247u &&
-                     (__double_as_longlong(d) & 0xFFFFFFFFFFFFFll) != 0xFFFFFFFFFFFFFll;
-  const int gap = (int)en - (int)ed;
-  if (!plain || gap > 500 || gap < -500) return n / d;
-  double q = n * inv;
-  q = fma(fma(-q, d, n), inv, q);
-  return fma(fma(-q, d, n), inv, q);
 }
 
 // Sum of NV values over the CTA; every thread receives the totals.

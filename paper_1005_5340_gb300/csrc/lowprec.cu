@@ -17,6 +17,7 @@
 
 #include <algorithm>
 
+#include "exact.h"
 #include "internal.h"
 #include "tc_ptx.h"
 
@@ -63,36 +64,6 @@ __global__ void split_rows_kernel(const double *__restrict__ src, int64_t rs, in
     dst[r * 2 * Kp + k] = hi;
     dst[r * 2 * Kp + Kp + k] = lo;
   }
-}
-
-// The split of a float64 value as __double2bfloat16 gives it, hi = bf16(x) and
-// lo = bf16(x - hi), to nearest even, in integer arithmetic on the mantissa
-// (the conversions and the subtraction would run on the FP64 pipe, one
-// operation per 15 clocks and warp on an SM).  Exponents far from 1, zeros,
-// infinities and NaN take the conversions.
-__device__ __forceinline__ void split_f64(double x, __nv_bfloat16 &hi, __nv_bfloat16 &lo) {
-  const long long b = __double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7FF);
-  if (e < 1023 - 64 || e > 1023 + 64) {
-    hi = __double2bfloat16(x);
-    lo = __double2bfloat16(x - (double)__bfloat162float(hi));
-    return;
-  }
-  const unsigned int sign = (unsigned int)((unsigned long long)b >> 63) << 31;
-  const long long m = (b & 0xFFFFFFFFFFFFFll) | (1ll << 52);   // |x| = m 2^(e - 1075)
-  const long long h = (m + ((1ll << 44) - 1) + ((m >> 45) & 1)) >> 45;   // 128 .. 256
-  const long long r = m - (h << 45);                           // |r| <= 2^44
-  // float32(h) 2^(e - 1030): h has 8 significant bits
-  const unsigned int fh = __float_as_uint((float)(int)h) + ((unsigned int)(e - 1030) << 23);
-  hi = __ushort_as_bfloat16((unsigned short)((fh | sign) >> 16));
-  const unsigned long long q = (unsigned long long)(r < 0 ? -r : r);
-  const int sh = max(0, 63 - __clzll((long long)(q | 1)) - 7);   // bits below the 8 kept
-  const unsigned int l = sh == 0 ? (unsigned int)q
-                                 : (unsigned int)((q + ((1ull << (sh - 1)) - 1) + ((q >> sh) & 1)) >> sh);
-  // float32(l) 2^(sh + e - 1075), zero for r = 0
-  const unsigned int fl = __float_as_uint((float)(int)l) + ((unsigned int)(sh + e - 1075) << 23);
-  lo = __ushort_as_bfloat16(
-      (unsigned short)(l == 0 ? 0u : ((fl | (r < 0 ? sign ^ 0x80000000u : sign)) >> 16)));
 }
 
 // Four consecutive entries of an operand row: split bf16 (hi at p, lo at p +
