@@ -295,7 +295,8 @@ tddft_status tddft_kernel_apply(tddft_ctx *ctx, int32_t n_rhs, const double *z, 
  *  pointers, n_rhs x n_prod complex interleaved.  stream: cudaStream_t
  *  (NULL = legacy default), synchronised before returning.  Its scratch
  *  (about 32 n_rhs n_centres bytes) comes from the library's stream-ordered
- *  pool, which keeps at most 256 MB and gives them back at tddft_destroy.
+ *  pool, which keeps at most 256 MB between calls and gives them back when a
+ *  context is destroyed (at the process's end in a program that makes none).
  * Errors: INVALID_ARG (NULL, sizes < 1, softening < 0 or NaN), SHAPE (a
  * centre index out of range), NOMEM, CUDA.
  */
@@ -495,8 +496,10 @@ tddft_status tddft_selftest_gemm_tf32(int32_t M, int32_t N, int32_t K, uint64_t 
  *     |C - AB|_mn <= about (1 + (slices+1)/4) 2^(-7 slices) max_k|A_mk| max_k|B_kn| K
  * (2.3e-13 relative to that scale for 6 slices); an exact result whenever
  * the operands' entries are integers of at most 7*slices - 1 bits scaled
- * alike.  Allocates and frees its own slice buffers (about
- * (M+N) * slices * 2 bytes per K entry).  Errors: INVALID_ARG (NULL, sizes
+ * alike.  Its slice buffers (about (M+N) * slices * 2 bytes per K entry)
+ * come from the library's stream-ordered pool of the device, which keeps at
+ * most 256 MB between calls and gives them back when a context is destroyed
+ * (at the process's end in a program that makes none).  Errors: INVALID_ARG (NULL, sizes
  * < 1, slices outside 3..8), SHAPE (lda < K, ldb < N or ldc < N), NOMEM,
  * CUDA, TIMEOUT (a bounded wait inside the kernel gave up).
  */

@@ -25,8 +25,8 @@
 //   mlp_reduce_kernel    the partial sums of all CTAs, in order
 // The forward pass is bound by the 512 tanhf per row (ALU); the backward
 // kernels by the traffic of H1, H2 and dH1.
-// 1.74 M rows, bf16 weights: 15.7 -> 1.5 ms; a gradient of 218 k rows in
-// float32: 6.1 -> 1.2 ms (against the CUDA-core kernels).
+// 1.74 M rows, bf16 weights: 15.8 -> 1.34 ms; a gradient of 218 k rows in
+// float32: 6.17 -> 1.21 ms (against the CUDA-core kernels).
 //
 // Every mbarrier wait is bounded; on expiry the kernel records an error code,
 // stops issuing work, lets its copies and MMAs in flight finish and frees its

@@ -115,12 +115,9 @@ int drop_bits(int S, int chunks) {
 }
 constexpr int kOzMaxChunks = 1024;
 
-// acc += G_t of every group (t = grp + 2) read from tensor memory (this
-// thread's 32 columns at tcol), at weight 2^(7 (S - 1 - grp) - u); a negative
-// weight is a rounded right shift of the (exact, < 2^25) group sum.  One
-// group's values are live at a time (the loop is not unrolled).
-// (ns == S, passed at run time so that the loop stays rolled)
-// Columns j0 .. j0 + n - 1 of acc from v (n = 16 or 32).
+// Columns j0 .. j0 + N - 1 of acc (N = 16, 32 or 40) from a group's values v, at
+// weight 2^sh; a negative sh is a rounded right shift of the (exact, < 2^25)
+// group sum.
 template <int N, int EC>
 __device__ __forceinline__ void add_group(long long (&acc)[EC], const float *v, int j0, int sh) {
   // (one 32 x 32 + 64-bit multiply-add each; a weight above 2^30 occurs with 8
@@ -140,6 +137,9 @@ __device__ __forceinline__ void add_group(long long (&acc)[EC], const float *v, 
   }
 }
 
+// acc += G_t of every group (t = grp + 2) read from tensor memory, at weight
+// 2^(7 (S - 1 - grp) - drop).  One group's values are live at a time (the loop is
+// not unrolled: ns == S, passed at run time).
 // tcol: this thread's lane and its first column (h EPI_COLS) in group 0.
 // With 96-wide groups, half h = 0 reads 32 + 16 columns, h = 1 reads 16 +
 // 32, so that every 32-column load starts on a multiple of 32 columns; the
@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     __syncwarp();
   } else {
     // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (rows of the tile)
-    // and columns 32 h .. 32 h + 31 of every group, h = (w - 2) / 4
+    // and half h = (w - 2) / 4 of every group's columns (EPI_COLS of them)
     const int q = warp & 3, h = (warp - 2) >> 2;
     const int lr = q * 32 + lane;
     const uint32_t tcol = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * OZ_EPI_COLS);
@@ -932,7 +932,8 @@ double block_clocks(int S, int bn) {
 // the least of waves x chunks per CTA x clocks per block, with half a chunk
 // for the sum over a cluster and a third for a tile's start.  Exact integer
 // sums: every plan gives the same bits.
-// (1000 x 129 x 9080, 6 slices: 24 CTAs 455 us -> 13 clusters of 6, 65 us.)
+// (1000 x 129 x 9080, 6 slices: 24 CTAs of 64 columns 455 us -> 16
+// clusters of 6, 80 columns each, 65 us.)
 struct TilePlan {
   int bn, ks;
 };
@@ -1062,7 +1063,6 @@ cudaError_t launch_gemm_oz_ex(cudaStream_t st, const OzOperand &A, const OzOpera
   a.tiles = tiles;
   {
     // M tiles whose A panels (s slices of the whole K) fill about 40 MB of L2
-    // (grid.x = Mt, the tiles or 128-row blocks)
     const double panel = (double)OZ_BM * A.s * A.Kp * sizeof(__nv_bfloat16);
     const int Mt = tiles ? n_tiles : (M + OZ_BM - 1) / OZ_BM;
     a.mgroup = std::max(1, std::min(Mt, (int)(40.0e6 / panel)));

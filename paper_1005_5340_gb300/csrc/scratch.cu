@@ -4,7 +4,7 @@
 // stream, so calls from several threads and streams never share a buffer in
 // flight.  The pool keeps at most kKeepBytes between calls (a cudaMalloc and
 // cudaFree pair costs about 90 us, most of a small product) and gives them
-// back when a context is destroyed.
+// back when a context is destroyed, or at the process's end.
 #include <mutex>
 
 #include "internal.h"
