@@ -88,8 +88,12 @@ __device__ __forceinline__ void split3_pair(float x, float y, uint32_t (&w)[3]) 
 // bits, an absolute error of 2^-134 per product.  (Gradient of 218 k rows:
 // 1.19 -> 1.21 ms.)
 constexpr float kDh2Scale = 0x1p48f, kDh2Unscale = 0x1p-48f, kDh2Max = 0x1p100f, kW2Max = 0x1p18f;
-// the entry t (1 - h^2) of dH2, t = sum dY W3: one rounding wherever it is
-// formed (both passes take the same decision on it)
+// the entry t (1 - h^2) of dH2 times 2^48, t = sum dY W3 as float32 has it (the
+// scale comes in with 1 - h^2, so that no term of t overflows for it): one
+// rounding wherever it is formed (both passes take the same decision on it)
+__device__ __forceinline__ float dh2_scaled(float t, float h) {
+  return __fmul_rn(t, fmaf(-kDh2Scale * h, h, kDh2Scale));
+}
 __device__ __forceinline__ float dh2_of(float t, float h) {
   return __fmul_rn(t, fmaf(-h, h, 1.f));
 }
@@ -570,7 +574,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int n_tiles = (int)((rows + MT - 1) / MT);
   if (threadIdx.x == 0) ctl_init(ct, 1);
   for (int i = threadIdx.x; i < kMlpMaxOut * MW; i += kThreads)
-    sw3[i] = kDh2Scale * tc.vec[2 * MW + i];   // dH2 comes out scaled
+    sw3[i] = tc.vec[2 * MW + i];
   const bool odd_w2 = __syncthreads_or(odd_w) != 0;
   const uint32_t tmem = tmem_open(ct, warp, lim);
   if (warp == 0) {
@@ -648,7 +652,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int o = 0; o < kMlpMaxOut; ++o)
             if (o < no) s = fmaf(dy[o], sw3[o * MW + c0 + j], s);
-          h[j] = dh2_of(s, h[j]);
+          h[j] = dh2_scaled(s, h[j]);
         }
         if (drop_odd(h)) *(volatile int *)&ct->odd = 1;
         if (u > 1 && !(ok = role_wait(&ct->aempty[u & 1], (uint32_t)((u >> 1) - 1) & 1u, ct, err, 64)))
@@ -692,13 +696,10 @@ __device__ __noinline__ void dw2_odd(const MlpTc &tc, int64_t rows, int64_t b0, 
   for (int g = 0; g < n_mine; ++g) {
     const int64_t ra = (b0 + g * step) * kDwRows;
     for (int64_t r = ra; r < min(rows, ra + kDwRows); ++r) {
-      float scaled = 0.f, t = 0.f;
-      for (int o = 0; o < no; ++o) {
-        scaled = fmaf(dY[r * no + o], kDh2Scale * w3[o * MW], scaled);
-        t = fmaf(dY[r * no + o], w3[o * MW], t);
-      }
+      float t = 0.f;
+      for (int o = 0; o < no; ++o) t = fmaf(dY[r * no + o], w3[o * MW], t);
       const float h = H2[r * W + i], d = dh2_of(t, h);
-      if (!(fabsf(dh2_of(scaled, h)) > kDh2Max)) continue;
+      if (!(fabsf(dh2_scaled(t, h)) > kDh2Max)) continue;
       for (int j = j0; j < j1; ++j) pw[i * MW + j] = fmaf(d, H1[r * W + j], pw[i * MW + j]);
       if (half == 0) pw[MW * MW + i] += d;   // db2, of the first row group
     }
@@ -757,7 +758,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int j = half * (MW / 2) + jl;
     float w3[kMlpMaxOut], g3[kMlpMaxOut] = {}, gb2 = 0.f, gb3 = 0.f;
 #pragma unroll
-    for (int o = 0; o < kMlpMaxOut; ++o) w3[o] = kDh2Scale * tc.vec[(2 + o) * MW + i];
+    for (int o = 0; o < kMlpMaxOut; ++o) w3[o] = tc.vec[(2 + o) * MW + i];
     float n2[8], n1[4], ndy;   // the next block's values; lane l: dY entry l of the 8 rows
     auto load = [&](int g) {
       const int64_t ra = (b0 + g * step) * kDwRows;
@@ -816,7 +817,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             g3[o] = fmaf(dy, h2[e], g3[o]);
             if (i == o) gb3 += dy;
           }
-        d2[e] = dh2_of(t, h2[e]);
+        d2[e] = dh2_scaled(t, h2[e]);
       }
       if (drop_odd(d2)) *(volatile int *)&ct->odd = 1;
 #pragma unroll

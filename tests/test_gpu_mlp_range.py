@@ -106,3 +106,27 @@ def test_weights_without_planes(bf16, value):
         with np.errstate(invalid="ignore"):
             g = MO.backward(p, f.astype(np.float64), dy.astype(np.float64), DIMS)
         assert same(net.backward(cuda(f), cuda(dy)), g, 6e-6)
+
+
+@pytest.mark.parametrize("rows", [300, 20000])
+@pytest.mark.parametrize("value", [1e20, 1e25, 1e30])
+def test_large_output_weights(rows, value):
+    # no row overflows, and zero gradients stay zero (also those of the last
+    # tile's rows past the end)
+    rng = np.random.default_rng(rows)
+    ni, w, no = DIMS
+    p = params(rng)
+    p[-(no * w + no) + 7] = value          # W3[0][7]
+    f = rng.normal(size=(rows, ni)).astype(np.float32)
+    dy = rng.normal(size=(rows, no)).astype(np.float32)
+    dy[::5] = 0.0
+    ref = MO.backward(p, f.astype(np.float64), dy.astype(np.float64), DIMS)
+    g = network(rows, p).backward(cuda(f), cuda(dy)).astype(np.float64)
+    assert np.isfinite(g).all()
+    parts = np.cumsum([w * ni, w, w * w, w, no * w])
+    for a, b in zip(np.split(g, parts), np.split(ref, parts)):
+        assert np.linalg.norm(a - b) <= 6e-6 * np.linalg.norm(b)
+    # dW2 and db2 unit by unit: unit 7 would hide the others
+    unit = lambda x: np.linalg.norm(x.reshape(w, -1), axis=1)
+    for i, j in ((parts[1], parts[2]), (parts[2], parts[3])):
+        assert np.all(unit(g[i:j] - ref[i:j]) <= 6e-5 * unit(ref[i:j]))
