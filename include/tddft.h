@@ -423,9 +423,12 @@ tddft_status tddft_tuning(const tddft_ctx *ctx, int32_t *n_tiles);
 /*
  * Launch plan of the split-bf16 K product (tensor-core forms) for n_rhs
  * right-hand sides (2 n_rhs real columns) with the context's N tile: *ncl
- * receives the cluster size (1: no clusters; 2..4: one CTA per N tile of an
- * M row block, in one cluster), *ksplit the number of K slices (1 or 2, the
- * slices added into a zeroed output).  Host-side query, no device work.
+ * receives the CTAs that take an M row block together, one per N tile (1:
+ * none do; 2..4: the tiles of a row block follow one another, and its CTAs
+ * are launched as one cluster unless clusters of that size, which leave SMs
+ * without one, would need a fifth more waves or above than single CTAs in the
+ * same order), *ksplit the number of K slices (1 or 2, the slices added into
+ * a zeroed output).  Host-side query, no device work.
  */
 tddft_status tddft_kproduct_plan(const tddft_ctx *ctx, int32_t n_rhs, int32_t *ncl,
                                  int32_t *ksplit);

@@ -174,7 +174,8 @@ struct TcEpilogue {
   int split_ok = 0;                // kStoreF32: the launch may split K in two (adds into outF)
   int cleared = 0;                 // kStoreF32: the caller has cleared outF for that
   int ksplit = 1;                  // set by the launcher
-  int ncl = 1;                     // set by the launcher: > 1, clusters of ncl CTAs, one per N tile
+  int ncl = 1;                     // set by the launcher: > 1, ncl CTAs (one per N tile) share an M row
+                                   // block, in a cluster where that costs few waves (launch_tc)
   int n_fast = 0;                  // set by the launcher: the N tile runs fastest
   const int *aoff = nullptr;       // kGammaCatSplit
   const int *orb_atom = nullptr;   // kGammaCatSplit
@@ -215,7 +216,7 @@ cudaError_t launch_gemm_tc_grouped(cudaStream_t st, const TcOperand &A, const Tc
                                    const TcEpilogue &ep, int *err, const int *dcnt = nullptr,
                                    int mul_n = 0, int bn = 128);
 void tc_init_attributes();
-// Split K (ksplit 1 or 2) and cluster size (ncl 1..4) of a kStoreF32 product
+// Split K (ksplit 1 or 2) and CTAs per M row block (ncl 1..4) of a kStoreF32 product
 // with split_ok (the K product): A of M rows and padded K Kp, N columns, N tile bn.
 void tc_split_plan(int Kp, int M, int N, int bn, int *ksplit, int *ncl);
 

@@ -396,7 +396,8 @@ class Context:
         self._check(self._lib.tddft_set_wait_timeout(self.h, int(ns)))
 
     def kproduct_plan(self, n_rhs: int):
-        """(cluster size, K slices) of the split-bf16 K product for n_rhs vectors."""
+        """(CTAs per M row block, one per N tile, and K slices) of the split-bf16 K product
+        for n_rhs vectors."""
         ncl, ks = ctypes.c_int32(), ctypes.c_int32()
         self._check(self._lib.tddft_kproduct_plan(self.h, n_rhs, ctypes.byref(ncl),
                                                   ctypes.byref(ks)))
