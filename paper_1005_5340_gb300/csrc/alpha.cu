@@ -127,6 +127,16 @@ __global__ void alpha_part_kernel(int64_t rows, int K2max, int n_occ, int n_orb,
   }
 }
 
+// Groups of columns run over grid.y and, beyond its limit, grid.z (any number of
+// right-hand sides runs).
+dim3 column_grid(unsigned x, int ncols, int per) {
+  const unsigned n = (unsigned)((ncols + per - 1) / per), y = std::min(n, 32768u);
+  return dim3(x, y, (n + y - 1) / y);
+}
+__device__ __forceinline__ int column_group() {
+  return (int)(blockIdx.z * gridDim.y + blockIdx.y);
+}
+
 // Ycat[c][k] = Y[c][lcat[k]] (0 where lcat[k] < 0), split bf16 (or tf32): two
 // neighbouring k per thread (4-byte stores), their list entries read once for
 // kGatherCols columns.  Y: rows c of ld, or, interleaved, complex vectors of ld.
@@ -141,9 +151,9 @@ __global__ void __launch_bounds__(256) gather_split_kernel(int ncols, int kcat,
   const int k = 2 * (blockIdx.x * 256 + threadIdx.x);
   if (k >= kcat) return;
   const int2 mu = *(const int2 *)(lcat + k);
-  const int c1 = min(ncols, ((int)blockIdx.y + 1) * kGatherCols);
+  const int c0 = column_group() * kGatherCols, c1 = min(ncols, c0 + kGatherCols);
 #pragma unroll 4
-  for (int c = blockIdx.y * kGatherCols; c < c1; ++c) {
+  for (int c = c0; c < c1; ++c) {
     const T *y = inter ? Y + (int64_t)(c >> 1) * 2 * ld + (c & 1) : Y + c * ld;
     const int st = inter ? 2 : 1;
     const float x0 = mu.x >= 0 ? (float)y[(int64_t)mu.x * st] : 0.f;
@@ -175,7 +185,7 @@ __global__ void __launch_bounds__(256) combine_kernel(int ncols, int n_prod,
   __shared__ TP ta[32][33], tb[32][33];
   if (dcnt) ncols = min(ncols, 2 * *dcnt);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int mu0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
+  const int mu0 = blockIdx.x * 32, c0 = column_group() * 32;
   if (c0 >= ncols) return;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -433,8 +443,7 @@ cudaError_t alpha_setup(cudaStream_t st, const tddft_system *h, const DevSystem 
 
 cudaError_t launch_alpha_gather_lp(cudaStream_t st, const AlphaRoute &ar, int ncols, const void *Y,
                                    bool y_f64, bool inter, int64_t ld, const int *dcnt) {
-  const dim3 grid((ar.kcat2 / 2 + 255) / 256, (ncols + kGatherCols - 1) / kGatherCols);
-  if (grid.y > 65535) return cudaErrorInvalidConfiguration;
+  const dim3 grid = column_grid((ar.kcat2 / 2 + 255) / 256, ncols, kGatherCols);
   __nv_bfloat16 *dst = ar.ycat_q;
   if (y_f64)
     gather_split_kernel<double><<<grid, 256, 0, st>>>(ncols, ar.kcat2, ar.lcat, (const double *)Y,
@@ -448,8 +457,7 @@ cudaError_t launch_alpha_gather_lp(cudaStream_t st, const AlphaRoute &ar, int nc
 cudaError_t launch_alpha_combine(cudaStream_t st, const AlphaRoute &ar, int ncols, int n_prod,
                                  bool p_f64, const double *Zin, int subtract, double *Out,
                                  const int *dcnt, bool inter) {
-  const dim3 grid((n_prod + 31) / 32, (ncols + 31) / 32);
-  if (grid.y > 65535) return cudaErrorInvalidConfiguration;
+  const dim3 grid = column_grid((n_prod + 31) / 32, ncols, 32);
   if (p_f64)
     combine_kernel<double><<<grid, 256, 0, st>>>(ncols, n_prod, ar.pos5, ar.P2d, ar.ldp, Zin,
                                                  subtract, Out, inter, dcnt);
