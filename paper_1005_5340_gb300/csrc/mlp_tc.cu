@@ -124,7 +124,6 @@ __global__ void mlp_prepare_kernel(MlpTc tc) {
   const bool plain = !(fabsf(v2) > kW2Max);
   const int odd = __syncthreads_or(!plain);
   split3(plain ? v2 : 0.f, p);
-  if (k == 0) tc.odd_w2[n] = odd;
   for (int q = 0; q < 3; ++q) {
     tc.w2[((int64_t)q * MW + n) * MW + k] = p[q];
     tc.w2t[((int64_t)q * MW + k) * MW + n] = p[q];
@@ -137,11 +136,18 @@ __global__ void mlp_prepare_kernel(MlpTc tc) {
   if (k == 0) {
     tc.vec[n] = n < W ? b1[n] : 0.f;
     tc.vec[MW + n] = n < W ? b2[n] : 0.f;
+    bool inf3 = false;
     for (int o = 0; o < kMlpMaxOut; ++o) {
       const float v = n < W && o < no ? w3[(int64_t)o * W + n] : 0.f;
       tc.vec[(2 + o) * MW + n] = v;
       tc.vec[(2 + kMlpMaxOut + o) * MW + n] = __bfloat162float(__float2bfloat16_rn(v));
+      inf3 |= isinf(v) != 0;
     }
+    // dW2's copy: a unit with an infinite weight (0 x inf in rows past the end)
+    // is zero there and left to the CUDA cores
+    for (int o = 0; o < kMlpMaxOut; ++o)
+      tc.w3_dw2[o * MW + n] = inf3 ? 0.f : tc.vec[(2 + o) * MW + n];
+    tc.odd_w[n] = (odd ? 1 : 0) | (inf3 ? 2 : 0);
     if (n < kMlpMaxOut) tc.vec[(2 + 2 * kMlpMaxOut) * MW + n] = n < no ? b3[n] : 0.f;
   }
 }
@@ -327,9 +333,9 @@ __device__ __forceinline__ void get16(const float *src, int c0, int W, bool live
   }
 }
 
-// This thread's share of whether some weight of W2 has no planes
-__device__ __forceinline__ int odd_weight(const MlpTc &tc) {
-  return threadIdx.x < MW ? tc.odd_w2[threadIdx.x] : 0;
+// This thread's share of whether some unit has bit `what` of odd_w
+__device__ __forceinline__ int odd_weight(const MlpTc &tc, int what) {
+  return threadIdx.x < MW ? tc.odd_w[threadIdx.x] & what : 0;
 }
 
 // A forward CTA's rows on the CUDA cores, one row at a time (buf: 2 MW floats)
@@ -379,7 +385,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                        float *__restrict__ H2, float *__restrict__ Y, int *err) {
   extern __shared__ uint8_t smem_raw[];
   const uint64_t lim = wait_limit(err);   // (loaded ahead of their use)
-  const int odd_w = odd_weight(tc);
+  const int odd_w = odd_weight(tc, 1);
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *sA = smem, *ring = sA + 2 * kBufA;
   float *sw1 = (float *)(ring + kRing * kTileB), *sb1 = sw1 + MW * kMlpMaxIn, *sb2 = sb1 + MW,
@@ -564,7 +570,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                    const float *__restrict__ H2, float *__restrict__ dH1, int *err) {
   extern __shared__ uint8_t smem_raw[];
   const uint64_t lim = wait_limit(err);
-  const int odd_w = odd_weight(tc);
+  const int odd_w = odd_weight(tc, 1);
   uint8_t *sA = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *ring = sA + 2 * kBufA;
   float *sw3 = (float *)(ring + kRing * kTileB);
@@ -692,6 +698,7 @@ __device__ __noinline__ void dw2_odd(const MlpTc &tc, int64_t rows, int64_t b0, 
   const int i = threadIdx.x, W = tc.width, no = tc.n_out;
   if (i >= W) return;
   const float *w3 = tc.vec + 2 * MW + i;
+  const bool all = (tc.odd_w[i] & 2) != 0;
   const int j0 = half * (MW / 2), j1 = min(W, j0 + MW / 2);
   for (int g = 0; g < n_mine; ++g) {
     const int64_t ra = (b0 + g * step) * kDwRows;
@@ -699,7 +706,7 @@ __device__ __noinline__ void dw2_odd(const MlpTc &tc, int64_t rows, int64_t b0, 
       float t = 0.f;
       for (int o = 0; o < no; ++o) t = fmaf(dY[r * no + o], w3[o * MW], t);
       const float h = H2[r * W + i], d = dh2_of(t, h);
-      if (!(fabsf(dh2_scaled(t, h)) > kDh2Max)) continue;
+      if (!all && !(fabsf(dh2_scaled(t, h)) > kDh2Max)) continue;
       for (int j = j0; j < j1; ++j) pw[i * MW + j] = fmaf(d, H1[r * W + j], pw[i * MW + j]);
       if (half == 0) pw[MW * MW + i] += d;   // db2, of the first row group
     }
@@ -712,6 +719,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                    float *__restrict__ part, int *err) {
   extern __shared__ uint8_t smem_raw[];
   const uint64_t lim = wait_limit(err);
+  const int odd_w3 = odd_weight(tc, 2);
   uint8_t *sa = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *sb = sa + 3 * kDwA;
   Ctl *ct = (Ctl *)(sb + 3 * kDwB);
@@ -723,6 +731,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int n_mine = (int)((n_blk - b0 + step - 1) / step);   // >= 1
   if (threadIdx.x == 0) ctl_init(ct, kEpiWarps);
   const uint32_t tmem = tmem_open(ct, warp, lim);
+  if (odd_w3) *(volatile int *)&ct->odd = 1;
   float *pw = part + b0 * tc.part_stride;
   if (warp == 1) {
     constexpr uint32_t idesc = idesc_bf16(MT, MW / 2);
@@ -758,7 +767,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int j = half * (MW / 2) + jl;
     float w3[kMlpMaxOut], g3[kMlpMaxOut] = {}, gb2 = 0.f, gb3 = 0.f;
 #pragma unroll
-    for (int o = 0; o < kMlpMaxOut; ++o) w3[o] = tc.vec[(2 + o) * MW + i];
+    for (int o = 0; o < kMlpMaxOut; ++o) w3[o] = tc.w3_dw2[o * MW + i];
     float n2[8], n1[4], ndy;   // the next block's values; lane l: dY entry l of the 8 rows
     auto load = [&](int g) {
       const int64_t ra = (b0 + g * step) * kDwRows;
@@ -988,7 +997,7 @@ bool mlp_tc_fits(int n_in, int width, int n_out) {
 
 size_t mlp_tc_bytes(int64_t max_rows) {
   return (size_t)6 * MW * MW * sizeof(__nv_bfloat16) +
-         (size_t)(2 * kMlpMaxIn + 4 + 2 * kMlpMaxOut) * MW * sizeof(float) + 256 +
+         (size_t)(2 * kMlpMaxIn + 4 + 3 * kMlpMaxOut) * MW * sizeof(float) + 256 +
          (size_t)(dw2_groups(max_rows) * kPartStride +
                   (int64_t)dw1_ctas(max_rows) * (kMlpMaxIn + 1) * MW) * sizeof(float);
 }
@@ -1004,8 +1013,9 @@ cudaError_t mlp_tc_init(MlpTc &tc, int n_in, int width, int n_out, int64_t max_r
   tc.w2t = tc.w2 + 3 * MW * MW;
   tc.w1 = (float *)(tc.w2t + 3 * MW * MW);
   tc.vec = tc.w1 + 2 * MW * kMlpMaxIn;
-  tc.odd_w2 = (int *)(tc.vec + (3 + 2 * kMlpMaxOut) * MW);
-  tc.err = tc.odd_w2 + MW;
+  tc.w3_dw2 = tc.vec + (3 + 2 * kMlpMaxOut) * MW;
+  tc.odd_w = (int *)(tc.w3_dw2 + kMlpMaxOut * MW);
+  tc.err = tc.odd_w + MW;
   tc.part2 = (float *)((char *)tc.err + 256);
   tc.part1 = tc.part2 + dw2_groups(max_rows) * kPartStride;
   cudaError_t e = encode_bf16_map(&tc.map2, tc.w2, 3 * MW, MW, MW);

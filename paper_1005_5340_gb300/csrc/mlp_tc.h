@@ -20,7 +20,9 @@ struct MlpTc {
   __nv_bfloat16 *w2t = nullptr;    // [3][256][256] planes of W2^T
   float *w1 = nullptr;             // [2][256][12] W1 (float32; rounded to bf16)
   float *vec = nullptr;            // b1, b2, W3 (float32), W3 (rounded to bf16), b3: rows of 256
-  int *odd_w2 = nullptr;           // [256] whether a row of W2 has weights without planes
+  float *w3_dw2 = nullptr;         // [4][256] W3 as dW2 takes it (infinite: see odd_w)
+  int *odd_w = nullptr;            // [256] per unit: 1 its row of W2 has weights without planes,
+                                   // 2 it has an infinite output weight
   int *err = nullptr;              // code of a wait that gave up (0: none), training steps
                                    // skipped since, 64-bit wait limit in ns (0: 2 s)
   float *part2 = nullptr, *part1 = nullptr;   // per-CTA partial gradients

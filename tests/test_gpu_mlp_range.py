@@ -130,3 +130,18 @@ def test_large_output_weights(rows, value):
     unit = lambda x: np.linalg.norm(x.reshape(w, -1), axis=1)
     for i, j in ((parts[1], parts[2]), (parts[2], parts[3])):
         assert np.all(unit(g[i:j] - ref[i:j]) <= 6e-5 * unit(ref[i:j]))
+
+
+@pytest.mark.parametrize("rows", [300, 304, 20001])
+@pytest.mark.parametrize("value", [float("inf"), -float("inf")])
+def test_infinite_output_weight(rows, value):
+    # every infinity of a sum has the weight's sign; rows past the end have no share
+    rng = np.random.default_rng(rows)
+    ni, w, no = DIMS
+    p = params(rng, lo=0.01)
+    p[-(no * w + no) + 7] = value          # W3[0][7]
+    f = rng.uniform(0.1, 1.0, (rows, ni)).astype(np.float32)
+    dy = rng.uniform(0.1, 1.0, (rows, no)).astype(np.float32)
+    ref = MO.backward(p, f.astype(np.float64), dy.astype(np.float64), DIMS)
+    assert not np.isnan(ref).any() and np.isinf(ref).any()
+    assert same(network(rows, p).backward(cuda(f), cuda(dy)), ref, 6e-6)
